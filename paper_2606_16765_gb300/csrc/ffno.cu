@@ -1,6 +1,8 @@
 // ffno.cu -- the factorised Fourier Neural Operator of include/ffno.h:
 // forward, hand-written backward and Adam in FP32 (activations and
-// arithmetic), one thread per output element.
+// arithmetic).  Networks of up to 32 channels whose lines fit shared memory
+// run on the tiled kernels of ffno_fast.cu (forward_fast, backward_fast); the
+// others on the general kernels below, one thread per output element.
 //
 // Fields are [batch][channel][z][y][x].  A spectrum along axis d keeps the
 // field's layout with that axis's samples replaced by its first m_d wave
@@ -30,12 +32,15 @@
 #include <cuda_runtime.h>
 
 #include "../../include/ffno.h"
+#include "ffno_fast.h"
 #include "sm_count.h"
 
 namespace {
 
 constexpr int TPB = 256;
-enum { ACT_NONE = 0, ACT_GELU = 1, ACT_SIREN = 2 };
+using ffno::ACT_GELU;
+using ffno::ACT_NONE;
+using ffno::ACT_SIREN;
 
 int grid_for(int64_t n)
 {
@@ -283,16 +288,28 @@ __global__ void __launch_bounds__(TPB) k_mse_partial(const float *y, const float
     }
 }
 
-__global__ void k_mse_final(const double *part, int nb, int C, double *res)
+// one block: strided sums, then a tree (fixed order)
+__global__ void __launch_bounds__(TPB) k_mse_final(const double *part, int nb, int C, double *res)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double a = 0.0, w = 0.0;
-        for (int k = 0; k < nb; ++k) {
-            a += part[2 * k];
-            w += part[2 * k + 1];
+    __shared__ double s1[TPB], s2[TPB];
+    double a = 0.0, w = 0.0;
+    for (int k = threadIdx.x; k < nb; k += TPB) {
+        a += part[2 * k];
+        w += part[2 * k + 1];
+    }
+    s1[threadIdx.x] = a;
+    s2[threadIdx.x] = w;
+    __syncthreads();
+    for (int h = TPB / 2; h > 0; h >>= 1) {
+        if ((int)threadIdx.x < h) {
+            s1[threadIdx.x] += s1[threadIdx.x + h];
+            s2[threadIdx.x] += s2[threadIdx.x + h];
         }
-        res[0] = a / (C * w);        // loss
-        res[1] = w;                  // sum of the weights
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        res[0] = s1[0] / (C * s2[0]);        // loss
+        res[1] = s2[0];                      // sum of the weights
     }
 }
 
@@ -346,6 +363,19 @@ struct ffno_ctx {
     float *gy = nullptr, *gh = nullptr, *gv = nullptr, *gz = nullptr, *gu = nullptr, *ga = nullptr;
     double *part = nullptr, *res = nullptr;
     int nb_loss = 0;
+    // tiled path: axis plans, the weights packed per wave number (again after
+    // every change of the parameters), partial sums
+    bool fast = false;
+    ffno::Axis ax[3];
+    std::vector<float2 *> rf, ra;                            // [3 l + d]
+    std::vector<float *> vspec;                              // [3 l + d]
+    float *gspec = nullptr, *wpart = nullptr;
+    float2 *rpart = nullptr;
+    float *tables = nullptr;
+
+    ffno::Mlp lift() const { return {c.cin, c.lift_hidden, c.width, ACT_GELU, c.omega0, params + oP1w, params + oP1b, params + oP2w, params + oP2b}; }
+    ffno::Mlp ff(int l) const { return {c.width, c.ff_hidden, c.width, ACT_GELU, c.omega0, params + oF1w[l], params + oF1b[l], params + oF2w[l], params + oF2b[l]}; }
+    ffno::Mlp proj() const { return {c.width, c.hidden, c.cout, ACT_SIREN, c.omega0, params + oQ1w, params + oQ1b, params + oQ2w, params + oQ2b}; }
 };
 
 namespace {
@@ -396,6 +426,19 @@ bool is_host(const void *p)
         return true;
     }
     return at.type != cudaMemoryTypeDevice && at.type != cudaMemoryTypeManaged;
+}
+
+// spectral weights per wave number, for the forward and (conjugate
+// transposed) the backward: launched where the parameters change
+void pack_weights(ffno_ctx *f)
+{
+    if (!f->fast) return;
+    for (int l = 0; l < f->c.layers; ++l) {
+        ffno::PackR p{};
+        for (int d = 0; d < 3; ++d)
+            p.a[d] = {f->params + f->oR[3 * l + d], f->se[d].e[d], f->rf[3 * l + d], f->ra[3 * l + d]};
+        ffno::pack_r(p, f->c.width, f->s);
+    }
 }
 
 std::string validate(const ffno_config &c)
@@ -469,21 +512,50 @@ extern "C" lbm_status ffno_create(const ffno_config *cfg, void *stream, ffno_ctx
     auto A = [&](auto *&p, int64_t n) { if (st == LBM_OK) st = alloc(f, p, n); };
     A(f->params, f->np); A(f->grads, f->np); A(f->m1, f->np); A(f->m2, f->np);
     const int64_t BN = (int64_t)B * f->N;
-    A(f->xin, BN * c.cin); A(f->tin, BN * c.cout); A(f->min, BN);
-    A(f->apre, BN * LH); A(f->a, BN * LH); A(f->hkeep, BN * c.hidden); A(f->h, BN * c.hidden); A(f->y, BN * c.cout);
-    f->v.assign(L + 1, nullptr); f->u.assign(L, nullptr); f->z.assign(L, nullptr); f->hff.assign(L, nullptr);
-    f->spec.assign(3 * L, nullptr);
-    for (int l = 0; l <= L; ++l) A(f->v[l], BN * W);
-    int64_t smax = 0;
-    for (int d = 0; d < 3; ++d) smax = std::max(smax, f->se[d].n());
-    for (int l = 0; l < L; ++l) {
-        A(f->u[l], BN * W); A(f->z[l], BN * H); A(f->hff[l], BN * H);
-        for (int d = 0; d < 3; ++d) A(f->spec[3 * l + d], (int64_t)B * W * f->se[d].n());
+    // samples S apart (z, y) or contiguous (x)
+    f->fast = ffno::axis_plan(f->ax[0], c.nz, c.mz, 0, (int64_t)c.ny * c.nx, 1, W) &&
+              ffno::axis_plan(f->ax[1], c.ny, c.my, 0, c.nx, c.nz, W) &&
+              ffno::axis_plan(f->ax[2], c.nx, c.mx, 1, 1, (int64_t)c.nz * c.ny, W) &&
+              ffno::mlp_fits(c.cin, LH, W) && ffno::mlp_fits(W, H, W) && ffno::mlp_fits(W, c.hidden, c.cout) &&
+              ffno::set_attrs();
+    A(f->xin, BN * c.cin); A(f->tin, BN * c.cout); A(f->min, BN); A(f->y, BN * c.cout);
+    A(f->gy, BN * c.cout); A(f->gv, BN * W); A(f->gu, BN * W);
+    f->u.assign(L, nullptr);
+    for (int l = 0; l < L; ++l) A(f->u[l], BN * W);
+    if (f->fast) {
+        f->v.assign(1, nullptr);
+        A(f->v[0], BN * W);
+        f->rf.assign(3 * L, nullptr); f->ra.assign(3 * L, nullptr); f->vspec.assign(3 * L, nullptr);
+        const int Wp = (W + 3) & ~3;
+        int64_t smax = 1, rmax = 1;
+        for (int d = 0; d < 3; ++d) {
+            const int64_t sn = 2 * (int64_t)m[d] * W * B * f->ax[d].lines();
+            smax = std::max(smax, sn);
+            // fewer lines (a smaller batch) never take more parts
+            rmax = std::max(rmax, (int64_t)ffno::grad_r_parts(m[d], B * f->ax[d].lines()) * m[d] * W * W);
+            for (int l = 0; l < L; ++l) {
+                A(f->rf[3 * l + d], (int64_t)m[d] * W * Wp); A(f->ra[3 * l + d], (int64_t)m[d] * W * Wp);
+                A(f->vspec[3 * l + d], sn);
+            }
+        }
+        const int64_t nw = std::max<int64_t>({(int64_t)LH * (c.cin + W + 1) + W, (int64_t)H * (2 * W + 1) + W,
+                                              (int64_t)c.hidden * (W + c.cout + 1) + c.cout});
+        A(f->gspec, smax); A(f->rpart, rmax); A(f->wpart, nw * ffno::mlp_parts());
+    } else {
+        A(f->apre, BN * LH); A(f->a, BN * LH); A(f->hkeep, BN * c.hidden); A(f->h, BN * c.hidden);
+        f->v.assign(L + 1, nullptr); f->z.assign(L, nullptr); f->hff.assign(L, nullptr);
+        f->spec.assign(3 * L, nullptr);
+        for (int l = 0; l <= L; ++l) A(f->v[l], BN * W);
+        int64_t smax = 0;
+        for (int d = 0; d < 3; ++d) smax = std::max(smax, f->se[d].n());
+        for (int l = 0; l < L; ++l) {
+            A(f->z[l], BN * H); A(f->hff[l], BN * H);
+            for (int d = 0; d < 3; ++d) A(f->spec[3 * l + d], (int64_t)B * W * f->se[d].n());
+        }
+        A(f->mixw, (int64_t)B * W * smax); A(f->mixw2, (int64_t)B * W * smax);
+        const int64_t cmax = std::max<int64_t>({(int64_t)W, (int64_t)H, (int64_t)LH, (int64_t)c.hidden, (int64_t)c.cout});
+        A(f->gh, BN * c.hidden); A(f->gz, BN * cmax); A(f->ga, BN * LH);
     }
-    A(f->mixw, (int64_t)B * W * smax); A(f->mixw2, (int64_t)B * W * smax);
-    const int64_t cmax = std::max<int64_t>({(int64_t)W, (int64_t)H, (int64_t)LH, (int64_t)c.hidden, (int64_t)c.cout});
-    A(f->gy, BN * c.cout); A(f->gh, BN * c.hidden); A(f->gv, BN * W); A(f->gz, BN * cmax); A(f->gu, BN * W);
-    A(f->ga, BN * LH);
     f->nb_loss = grid_for(BN);
     A(f->part, 2 * (int64_t)f->nb_loss); A(f->res, 2);
     for (int d = 0; d < 3; ++d) { A(f->tw[d], (int64_t)m[d] * f->fe.e[d]); A(f->ck[d], m[d]); A(f->ones[d], m[d]); }
@@ -512,6 +584,27 @@ extern "C" lbm_status ffno_create(const ffno_config *cfg, void *stream, ffno_ctx
             return ffail(nullptr, LBM_ERR_CUDA, "table upload failed");
         }
     }
+    if (f->fast) {
+        std::vector<float> all, one;
+        size_t at[3][4], cnt[4];
+        for (int d = 0; d < 3; ++d) {
+            ffno::axis_tables(f->ax[d], one, cnt);
+            size_t o4 = all.size();
+            for (int k = 0; k < 4; ++k) { at[d][k] = o4; o4 += cnt[k]; }     // multiples of 4 floats
+            all.insert(all.end(), one.begin(), one.end());
+        }
+        if (alloc(f, f->tables, (int64_t)all.size()) != LBM_OK ||
+            cudaMemcpy(f->tables, all.data(), all.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) {
+            ffno_destroy(f);
+            return ffail(nullptr, LBM_ERR_CUDA, "table upload failed");
+        }
+        for (int d = 0; d < 3; ++d) {
+            f->ax[d].ctab = reinterpret_cast<const float4 *>(f->tables + at[d][0]);
+            f->ax[d].stab = reinterpret_cast<const float4 *>(f->tables + at[d][1]);
+            f->ax[d].cinv = reinterpret_cast<const float4 *>(f->tables + at[d][2]);
+            f->ax[d].sinv = reinterpret_cast<const float4 *>(f->tables + at[d][3]);
+        }
+    }
     // initial parameters: uniform within 1/sqrt(fan_in), spectral weights
     // within 1/width^2, SIREN within 1/fan_in (first layer) and
     // sqrt(6/fan_in)/omega0 (output layer)
@@ -535,6 +628,7 @@ extern "C" lbm_status ffno_create(const ffno_config *cfg, void *stream, ffno_ctx
         ffno_destroy(f);
         return ffail(nullptr, LBM_ERR_CUDA, "parameter upload failed");
     }
+    pack_weights(f);
     *out = f;
     return LBM_OK;
 }
@@ -545,6 +639,8 @@ extern "C" lbm_status ffno_set_params(ffno_ctx *f, const float *src)
     FCK(cudaMemcpyAsync(f->params, src, f->np * sizeof(float), cudaMemcpyDefault, f->s));
     FCK(cudaStreamSynchronize(f->s));
     f->adam_t = 0;
+    pack_weights(f);
+    FCK(cudaGetLastError());
     FCK(cudaMemsetAsync(f->m1, 0, f->np * sizeof(float), f->s));
     FCK(cudaMemsetAsync(f->m2, 0, f->np * sizeof(float), f->s));
     return LBM_OK;
@@ -569,6 +665,43 @@ extern "C" lbm_status ffno_sync(ffno_ctx *f)
 }
 
 namespace {
+
+// Tiled forward of B samples, x and y on the device.  With `keep` the spectra
+// and every layer's u stay for the backward; v is updated in place (each cell
+// reads and writes its own residual).
+void forward_fast(ffno_ctx *f, const float *x, float *y, int B, bool keep)
+{
+    const int W = f->c.width;
+    float *v = f->v[0];
+    ffno::mlp(f->lift(), x, nullptr, v, B, f->N, f->s);
+    for (int l = 0; l < f->c.layers; ++l) {
+        float *u = f->u[keep ? l : 0];
+        for (int d = 0; d < 3; ++d)
+            ffno::spectral(f->ax[d], v, u, B, W, f->N, f->rf[3 * l + d], nullptr, f->ck[d],
+                           keep ? f->vspec[3 * l + d] : nullptr, d > 0, f->s);
+        ffno::mlp(f->ff(l), u, v, v, B, f->N, f->s);
+    }
+    ffno::mlp(f->proj(), v, nullptr, y, B, f->N, f->s);
+}
+
+// Tiled backward of the loss whose output gradient is in f->gy.
+void backward_fast(ffno_ctx *f, const float *x, int B)
+{
+    const int W = f->c.width;
+    float *G = f->grads;
+    ffno::mlp_bwd(f->proj(), f->v[0], f->gy, f->gv, f->wpart, G + f->oQ1w, B, f->N, f->s);
+    for (int l = f->c.layers - 1; l >= 0; --l) {
+        // v_{l+1} = v_l + F2 GELU(F1 u + b1) + b2: the residual path keeps gv,
+        // each axis adds the adjoint of its branch
+        ffno::mlp_bwd(f->ff(l), f->u[l], f->gv, f->gu, f->wpart, G + f->oF1w[l], B, f->N, f->s);
+        for (int d = 0; d < 3; ++d) {
+            ffno::spectral(f->ax[d], f->gu, f->gv, B, W, f->N, f->ra[3 * l + d], f->ck[d], nullptr, f->gspec, true, f->s);
+            ffno::grad_r(f->gspec, f->vspec[3 * l + d], W, f->se[d].e[d], B * f->ax[d].lines(), f->rpart,
+                         G + f->oR[3 * l + d], f->s);
+        }
+    }
+    ffno::mlp_bwd(f->lift(), x, f->gv, nullptr, f->wpart, G + f->oP1w, B, f->N, f->s);
+}
 
 // the forward pass of `B` samples staged in f->xin; every activation kept
 void forward_impl(ffno_ctx *f, int B)
@@ -648,16 +781,22 @@ extern "C" lbm_status ffno_forward(ffno_ctx *f, const float *x, float *y, int32_
     if (!f || !x || !y) return ffail(f, LBM_ERR_ARG, "null argument");
     if (batch < 1) return ffail(f, LBM_ERR_ARG, "batch must be positive");
     const ffno_config &c = f->c;
+    const bool xh = is_host(x), yh = is_host(y);        // device memory is read and written where it is
     for (int32_t b0 = 0; b0 < batch; b0 += c.max_batch) {
         const int B = std::min(c.max_batch, batch - b0);
-        FCK(cudaMemcpyAsync(f->xin, x + (int64_t)b0 * c.cin * f->N, sizeof(float) * B * c.cin * f->N, cudaMemcpyDefault,
-                            f->s));
-        forward_impl(f, B);
+        const float *xb = x + (int64_t)b0 * c.cin * f->N;
+        float *yb = y + (int64_t)b0 * c.cout * f->N;
+        if (!f->fast || xh) {
+            FCK(cudaMemcpyAsync(f->xin, xb, sizeof(float) * B * c.cin * f->N, cudaMemcpyDefault, f->s));
+            xb = f->xin;
+        }
+        if (f->fast) forward_fast(f, xb, yh ? f->y : yb, B, false);
+        else forward_impl(f, B);
         FCK(cudaGetLastError());
-        FCK(cudaMemcpyAsync(y + (int64_t)b0 * c.cout * f->N, f->y, sizeof(float) * B * c.cout * f->N, cudaMemcpyDefault,
-                            f->s));
+        if (!f->fast || yh)
+            FCK(cudaMemcpyAsync(yb, f->y, sizeof(float) * B * c.cout * f->N, cudaMemcpyDefault, f->s));
     }
-    if (is_host(y)) FCK(cudaStreamSynchronize(f->s));
+    if (yh) FCK(cudaStreamSynchronize(f->s));
     return LBM_OK;
 }
 
@@ -669,14 +808,22 @@ extern "C" lbm_status ffno_loss_grad(ffno_ctx *f, const float *x, const float *t
     if (batch < 1 || batch > c.max_batch) return ffail(f, LBM_ERR_ARG, "batch must lie in [1, max_batch]");
     const int B = batch;
     const int64_t N = f->N;
-    FCK(cudaMemcpyAsync(f->xin, x, sizeof(float) * B * c.cin * N, cudaMemcpyDefault, f->s));
-    FCK(cudaMemcpyAsync(f->tin, t, sizeof(float) * B * c.cout * N, cudaMemcpyDefault, f->s));
-    FCK(cudaMemcpyAsync(f->min, m, sizeof(float) * B * N, cudaMemcpyDefault, f->s));
-    forward_impl(f, B);
-    k_mse_partial<<<f->nb_loss, TPB, 0, f->s>>>(f->y, f->tin, f->min, c.cout, B, N, f->part);
-    k_mse_final<<<1, 32, 0, f->s>>>(f->part, f->nb_loss, c.cout, f->res);
-    k_mse_grad<<<grid_for((int64_t)B * c.cout * N), TPB, 0, f->s>>>(f->y, f->tin, f->min, c.cout, B, N, f->res, f->gy);
-    backward_impl(f, B);
+    auto stage = [&](const float *&src, float *dst, int64_t n) {
+        if (f->fast && !is_host(src)) return cudaSuccess;
+        const cudaError_t e = cudaMemcpyAsync(dst, src, sizeof(float) * n, cudaMemcpyDefault, f->s);
+        src = dst;
+        return e;
+    };
+    FCK(stage(x, f->xin, B * c.cin * N));
+    FCK(stage(t, f->tin, B * c.cout * N));
+    FCK(stage(m, f->min, B * N));
+    if (f->fast) forward_fast(f, x, f->y, B, true);
+    else forward_impl(f, B);
+    k_mse_partial<<<f->nb_loss, TPB, 0, f->s>>>(f->y, t, m, c.cout, B, N, f->part);
+    k_mse_final<<<1, TPB, 0, f->s>>>(f->part, f->nb_loss, c.cout, f->res);
+    k_mse_grad<<<grid_for((int64_t)B * c.cout * N), TPB, 0, f->s>>>(f->y, t, m, c.cout, B, N, f->res, f->gy);
+    if (f->fast) backward_fast(f, x, B);
+    else backward_impl(f, B);
     FCK(cudaGetLastError());
     double r[2] = {0, 0};
     FCK(cudaMemcpyAsync(r, f->res, sizeof(r), cudaMemcpyDeviceToHost, f->s));
@@ -692,6 +839,7 @@ extern "C" lbm_status ffno_adam_step(ffno_ctx *f, float lr, float b1, float b2, 
     const float c1 = (float)(1.0 - std::pow((double)b1, (double)f->adam_t));
     const float c2 = (float)(1.0 - std::pow((double)b2, (double)f->adam_t));
     k_adam<<<grid_for(f->np), TPB, 0, f->s>>>(f->params, f->grads, f->m1, f->m2, f->np, lr, b1, b2, eps, c1, c2);
+    pack_weights(f);
     FCK(cudaGetLastError());
     return LBM_OK;
 }

@@ -1,0 +1,992 @@
+// ffno_fast.cu -- tiled kernels of the factorised surrogate (FP32 activations
+// and arithmetic).
+//   k_spectral   one axis of u [+]= IDFT(R . DFT(v)): a block takes T lines of
+//                all channels through the folded transform, the channel mixing
+//                and the inverse in shared memory
+//   k_grad_r     the spectral weights' gradient, a split reduction over lines
+//   k_mlp        the pointwise networks, two cells per thread in registers
+//   k_mlp_bwd    their backward: hidden values recomputed, weight gradients
+//                accumulated per block and summed in a fixed order
+#include <algorithm>
+#include <cmath>
+
+#include "ffno_fast.h"
+#include "sm_count.h"
+
+namespace ffno {
+namespace {
+
+constexpr int TPB = 256;
+constexpr size_t SMEM_TWO = 113 * 1024;      // two blocks per SM
+constexpr size_t SMEM_MAX = 226 * 1024;
+
+__device__ __forceinline__ float4 f4(float v) { return make_float4(v, v, v, v); }
+__device__ __forceinline__ float4 operator+(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__device__ __forceinline__ float4 operator-(float4 a, float4 b) { return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
+__device__ __forceinline__ void fma4(float4 &d, float s, const float4 &v)
+{
+    d.x = fmaf(s, v.x, d.x);
+    d.y = fmaf(s, v.y, d.y);
+    d.z = fmaf(s, v.z, d.z);
+    d.w = fmaf(s, v.w, d.w);
+}
+__device__ __forceinline__ float4 mul4(float s, const float4 &v) { return make_float4(s * v.x, s * v.y, s * v.z, s * v.w); }
+
+// ---------------------------------------------------------------------------
+// spectral convolution along one axis
+// ---------------------------------------------------------------------------
+// Four neighbouring lines of sample n of a channel: contiguous along the lines
+// (ROWS = 0), or one element of each of four rows (ROWS = 1).
+struct Tile {
+    int64_t base;        // element of sample 0, line 0 of channel 0
+    int64_t sn;          // between samples
+    int64_t sl;          // between lines
+    int valid;           // lines of this tile that exist
+};
+
+template <int ROWS>
+__device__ __forceinline__ float4 load4(const float *p, const Tile &t, int64_t off, int l, bool vec)
+{
+    if (!ROWS && vec) return l < t.valid ? *reinterpret_cast<const float4 *>(p + off) : f4(0.f);
+    float4 r = f4(0.f);
+    if (l < t.valid) r.x = p[off];
+    if (l + 1 < t.valid) r.y = p[off + t.sl];
+    if (l + 2 < t.valid) r.z = p[off + 2 * t.sl];
+    if (l + 3 < t.valid) r.w = p[off + 3 * t.sl];
+    return r;
+}
+
+template <int ROWS>
+__device__ __forceinline__ void store4(float *p, const Tile &t, int64_t off, int l, bool vec, const float4 &v)
+{
+    if (!ROWS && vec) {
+        if (l < t.valid) *reinterpret_cast<float4 *>(p + off) = v;
+        return;
+    }
+    if (l < t.valid) p[off] = v.x;
+    if (l + 1 < t.valid) p[off + t.sl] = v.y;
+    if (l + 2 < t.valid) p[off + 2 * t.sl] = v.z;
+    if (l + 3 < t.valid) p[off + 3 * t.sl] = v.w;
+}
+
+// A block: T lines x W channels x L samples.  Phases, a barrier between them:
+//   fold     global -> D [c][class][n][T]: even and odd parts of the lines,
+//            split by the parity of the wave number they serve
+//   forward  V [k][c][T]: thread = 4 wave numbers x 4 lines, real and
+//            imaginary part: 32 multiply-adds per four 16-byte operands
+//   mix      G [k][o][T] over D: thread = 4 lines x 4 outputs (complex), the
+//            weights read once per block from L2
+//   inverse  thread = 4 terms x 4 lines of all four symmetric sums, unfolded
+//            into 16 samples and stored
+template <int ROWS>
+__global__ void __launch_bounds__(TPB, 2) k_spectral(const Axis a, const float *__restrict__ v, float *u, int W,
+                                                     int64_t N, const float2 *__restrict__ R,
+                                                     const float *__restrict__ wk, const float *__restrict__ ak,
+                                                     float *__restrict__ spec, int64_t NL, int tiles, int accumulate)
+{
+    extern __shared__ float4 raw[];
+    float *D = reinterpret_cast<float *>(raw);
+    float *Gre = D, *Gim = D + a.m * a.KS;
+    float *Vre = D + max(W * a.DS, 2 * a.m * a.KS), *Vim = Vre + a.m * a.KS;
+    const int T = a.T, TQ = T >> 2, tid = threadIdx.x;
+    const int tqs = TQ == 1 ? 0 : (TQ == 2 ? 1 : 2);
+    // the block's lines
+    Tile t;
+    int64_t line0;
+    {
+        int64_t w = blockIdx.x;
+        const int64_t ti = w % tiles;
+        w /= tiles;
+        if (ROWS) {
+            const int64_t b = w;
+            t.base = b * W * N + ti * T * a.L;
+            t.sn = 1;
+            t.sl = a.L;
+            t.valid = (int)min((int64_t)T, a.outer - ti * T);
+            line0 = b * a.outer + ti * T;
+        } else {
+            const int64_t o = w % a.outer, b = w / a.outer;
+            t.base = b * W * N + o * a.L * a.S + ti * T;
+            t.sn = a.S;
+            t.sl = 1;
+            t.valid = (int)min((int64_t)T, a.S - ti * T);
+            line0 = (b * a.outer + o) * a.S + ti * T;
+        }
+    }
+    const bool vec = !ROWS && (a.S & 3) == 0;
+    const int L = a.L, nq = a.nq, cls = nq * T;
+
+    // fold
+    for (int idx = tid; idx < W * nq * TQ; idx += TPB) {
+        int j, l, c;
+        if (ROWS) {                                 // neighbouring threads: neighbouring samples
+            j = idx % nq;
+            const int r = idx / nq;
+            l = (r & (TQ - 1)) << 2;
+            c = r >> tqs;
+        } else {
+            l = (idx & (TQ - 1)) << 2;
+            const int r = idx >> tqs;
+            j = r % nq;
+            c = r / nq;
+        }
+        const int64_t p0 = t.base + (int64_t)c * N + (int64_t)l * t.sl;
+        auto ld = [&](int n) { return load4<ROWS>(v, t, p0 + (int64_t)n * t.sn, l, vec); };
+        float *d = D + c * a.DS + j * T + l;
+        if (a.q == 2) {
+            float4 e0, e1, o0, o1;
+            if (j == 0) {
+                const float4 x = ld(0), y = ld(L / 2);
+                e0 = x + y;
+                e1 = x - y;
+                o0 = o1 = f4(0.f);
+            } else if (4 * j == L) {
+                const float4 x = ld(j), y = ld(L - j);
+                e0 = x + y;
+                o1 = x - y;
+                e1 = o0 = f4(0.f);
+            } else {
+                const float4 x = ld(j), y = ld(L - j), z = ld(L / 2 - j), w = ld(L / 2 + j);
+                const float4 ea = x + y, eb = z + w, oa = x - y, ob = z - w;
+                e0 = ea + eb;
+                e1 = ea - eb;
+                o0 = oa - ob;
+                o1 = oa + ob;
+            }
+            *reinterpret_cast<float4 *>(d) = e0;
+            *reinterpret_cast<float4 *>(d + cls) = e1;
+            *reinterpret_cast<float4 *>(d + 2 * cls) = o0;
+            *reinterpret_cast<float4 *>(d + 3 * cls) = o1;
+        } else {
+            float4 e = ld(j), o = f4(0.f);
+            if (j > 0 && 2 * j != L) {
+                const float4 y = ld(L - j);
+                o = e - y;
+                e = e + y;
+            }
+            *reinterpret_cast<float4 *>(d) = e;
+            *reinterpret_cast<float4 *>(d + cls) = o;
+        }
+    }
+    __syncthreads();
+
+    // forward: V(k) = wk (sum_n E cos - i sum_n O sin)
+    for (int idx = tid; idx < W * TQ * a.q * a.KG; idx += TPB) {
+        const int kg = idx % a.KG;
+        int r = idx / a.KG;
+        const int par = a.q == 2 ? (r & 1) : 0;
+        r = a.q == 2 ? r >> 1 : r;
+        const int l = (r & (TQ - 1)) << 2, c = r >> tqs;
+        const float *e = D + c * a.DS + par * cls + l, *o = e + a.q * cls;
+        const float4 *ct = a.ctab + (int64_t)par * nq * a.KG + kg, *st = a.stab + (int64_t)par * nq * a.KG + kg;
+        float4 re[4], im[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) re[k] = im[k] = f4(0.f);
+#pragma unroll 4
+        for (int n = 0; n < nq; ++n) {
+            const float4 cw = __ldg(ct + n * a.KG), sw = __ldg(st + n * a.KG);
+            const float4 x = *reinterpret_cast<const float4 *>(e + n * T);
+            const float4 y = *reinterpret_cast<const float4 *>(o + n * T);
+            fma4(re[0], cw.x, x);
+            fma4(re[1], cw.y, x);
+            fma4(re[2], cw.z, x);
+            fma4(re[3], cw.w, x);
+            fma4(im[0], sw.x, y);
+            fma4(im[1], sw.y, y);
+            fma4(im[2], sw.z, y);
+            fma4(im[3], sw.w, y);
+        }
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            const int k = par + a.q * (4 * kg + kk);
+            if (k >= a.m) break;
+            const float w = wk ? wk[k] : 1.f;
+            const float4 vr = mul4(w, re[kk]), vi = mul4(-w, im[kk]);
+            *reinterpret_cast<float4 *>(Vre + k * a.KS + c * T + l) = vr;
+            *reinterpret_cast<float4 *>(Vim + k * a.KS + c * T + l) = vi;
+            if (spec) {
+                const int64_t at = ((int64_t)k * W + c) * NL + line0 + l;
+                float *sr = spec + at, *si = sr + (int64_t)a.m * W * NL;
+                if (l + 4 <= t.valid && (at & 3) == 0 && (NL & 3) == 0) {
+                    *reinterpret_cast<float4 *>(sr) = vr;
+                    *reinterpret_cast<float4 *>(si) = vi;
+                } else {
+                    const float *pr = &vr.x, *pi = &vi.x;
+                    for (int q = 0; q < 4 && l + q < t.valid; ++q) {
+                        sr[q] = pr[q];
+                        si[q] = pi[q];
+                    }
+                }
+            }
+        }
+    }
+    __syncthreads();
+
+    // mix: G(o) = ak sum_i V(i) R(i, o)
+    const int OG = (W + 3) >> 2;
+    for (int idx = tid; idx < a.m * TQ * OG; idx += TPB) {
+        const int og = idx % OG;
+        int r = idx / OG;
+        const int l = (r & (TQ - 1)) << 2, k = r >> tqs;
+        const float4 *rp = reinterpret_cast<const float4 *>(R + (int64_t)k * W * OG * 4 + og * 4);
+        const float *vr = Vre + k * a.KS + l, *vi = Vim + k * a.KS + l;
+        float4 gr[4], gi[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) gr[o] = gi[o] = f4(0.f);
+#pragma unroll 4
+        for (int i = 0; i < W; ++i) {
+            const float4 r01 = __ldg(rp + (int64_t)i * OG * 2), r23 = __ldg(rp + (int64_t)i * OG * 2 + 1);
+            const float4 x = *reinterpret_cast<const float4 *>(vr + i * T);
+            const float4 y = *reinterpret_cast<const float4 *>(vi + i * T);
+            fma4(gr[0], r01.x, x);
+            fma4(gr[0], -r01.y, y);
+            fma4(gi[0], r01.y, x);
+            fma4(gi[0], r01.x, y);
+            fma4(gr[1], r01.z, x);
+            fma4(gr[1], -r01.w, y);
+            fma4(gi[1], r01.w, x);
+            fma4(gi[1], r01.z, y);
+            fma4(gr[2], r23.x, x);
+            fma4(gr[2], -r23.y, y);
+            fma4(gi[2], r23.y, x);
+            fma4(gi[2], r23.x, y);
+            fma4(gr[3], r23.z, x);
+            fma4(gr[3], -r23.w, y);
+            fma4(gi[3], r23.w, x);
+            fma4(gi[3], r23.z, y);
+        }
+        const float w = ak ? ak[k] : 1.f;
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            if (4 * og + o >= W) break;
+            *reinterpret_cast<float4 *>(Gre + k * a.KS + (4 * og + o) * T + l) = mul4(w, gr[o]);
+            *reinterpret_cast<float4 *>(Gim + k * a.KS + (4 * og + o) * T + l) = mul4(w, gi[o]);
+        }
+    }
+    __syncthreads();
+
+    // inverse: u(n) = sum_k (Gre cos - Gim sin)
+    for (int idx = tid; idx < W * TQ * a.NG; idx += TPB) {
+        const int ng = idx % a.NG;
+        int r = idx / a.NG;
+        const int l = (r & (TQ - 1)) << 2, c = r >> tqs;
+        const float *gr = Gre + c * T + l, *gi = Gim + c * T + l;
+        const float4 *ct = a.cinv + ng, *st = a.sinv + ng;
+        const int64_t p0 = t.base + (int64_t)c * N + (int64_t)l * t.sl;
+        auto put = [&](int n, const float4 &x) {
+            const int64_t off = p0 + (int64_t)n * t.sn;
+            store4<ROWS>(u, t, off, l, vec, accumulate ? load4<ROWS>(u, t, off, l, vec) + x : x);
+        };
+        if (a.q == 2) {
+            float4 ce[4], co[4], se[4], so[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) ce[j] = co[j] = se[j] = so[j] = f4(0.f);
+            for (int kk = 0; kk < a.mk; ++kk) {
+                const int k0 = 2 * kk, k1 = min(2 * kk + 1, a.m - 1);       // past the end: zero tables
+                const float4 x0 = *reinterpret_cast<const float4 *>(gr + k0 * a.KS);
+                const float4 y0 = *reinterpret_cast<const float4 *>(gi + k0 * a.KS);
+                const float4 x1 = *reinterpret_cast<const float4 *>(gr + k1 * a.KS);
+                const float4 y1 = *reinterpret_cast<const float4 *>(gi + k1 * a.KS);
+                const float4 c0 = __ldg(ct + kk * a.NG), s0 = __ldg(st + kk * a.NG);
+                const float4 c1 = __ldg(ct + (a.mk + kk) * a.NG), s1 = __ldg(st + (a.mk + kk) * a.NG);
+                fma4(ce[0], c0.x, x0);
+                fma4(ce[1], c0.y, x0);
+                fma4(ce[2], c0.z, x0);
+                fma4(ce[3], c0.w, x0);
+                fma4(se[0], s0.x, y0);
+                fma4(se[1], s0.y, y0);
+                fma4(se[2], s0.z, y0);
+                fma4(se[3], s0.w, y0);
+                fma4(co[0], c1.x, x1);
+                fma4(co[1], c1.y, x1);
+                fma4(co[2], c1.z, x1);
+                fma4(co[3], c1.w, x1);
+                fma4(so[0], s1.x, y1);
+                fma4(so[1], s1.y, y1);
+                fma4(so[2], s1.z, y1);
+                fma4(so[3], s1.w, y1);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int n = ng + j * a.NG;
+                if (n >= nq) break;
+                const float4 p = ce[j] + co[j], m = ce[j] - co[j], s = se[j] + so[j], d = se[j] - so[j];
+                put(n, p - s);
+                if (n == 0) {
+                    put(L / 2, m);
+                } else {
+                    put(L - n, p + s);
+                    if (4 * n != L) {
+                        put(L / 2 - n, m + d);
+                        put(L / 2 + n, m - d);
+                    }
+                }
+            }
+        } else {
+            float4 ce[4], se[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) ce[j] = se[j] = f4(0.f);
+            for (int kk = 0; kk < a.mk; ++kk) {
+                const float4 x = *reinterpret_cast<const float4 *>(gr + kk * a.KS);
+                const float4 y = *reinterpret_cast<const float4 *>(gi + kk * a.KS);
+                const float4 c0 = __ldg(ct + kk * a.NG), s0 = __ldg(st + kk * a.NG);
+                fma4(ce[0], c0.x, x);
+                fma4(ce[1], c0.y, x);
+                fma4(ce[2], c0.z, x);
+                fma4(ce[3], c0.w, x);
+                fma4(se[0], s0.x, y);
+                fma4(se[1], s0.y, y);
+                fma4(se[2], s0.z, y);
+                fma4(se[3], s0.w, y);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int n = ng + j * a.NG;
+                if (n >= nq) break;
+                put(n, ce[j] - se[j]);
+                if (n > 0 && 2 * n != L) put(L - n, ce[j] + se[j]);
+            }
+        }
+    }
+}
+
+// R [i][o][m] -> rf [m][i][Wp] and the conjugate transpose ra [m][o][Wp]
+__global__ void k_pack_r(const PackR pr, int W, int Wp)
+{
+    const float *R = pr.a[blockIdx.y].R;
+    float2 *rf = pr.a[blockIdx.y].rf, *ra = pr.a[blockIdx.y].ra;
+    const int m = pr.a[blockIdx.y].m, n = m * W * Wp;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+        const int p = t % Wp, r = (t / Wp) % W, k = t / (Wp * W);
+        float2 f = make_float2(0.f, 0.f), g = f;
+        if (p < W) {
+            const int64_t j = (((int64_t)r * W + p) * m + k) * 2, h = (((int64_t)p * W + r) * m + k) * 2;
+            f = make_float2(R[j], R[j + 1]);
+            g = make_float2(R[h], -R[h + 1]);
+        }
+        rf[t] = f;
+        ra[t] = g;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// gradient of the spectral weights
+// ---------------------------------------------------------------------------
+constexpr int GL = 64, GLP = GL + 4;         // lines per shared-memory tile, row stride
+
+// Block (k, split): a W x W complex product over the split's lines, thread =
+// 4 x 4 entries of one of four line groups (rows n4 apart keep the 16-byte
+// operand reads free of bank conflicts); 256 multiply-adds per 16 operands.
+__global__ void __launch_bounds__(TPB, 2) k_grad_r(const float *__restrict__ G, const float *__restrict__ V, int W,
+                                                   int m, int64_t NL, int splits, float2 *__restrict__ part)
+{
+    __shared__ __align__(16) float sh[4][MAXW][GLP];      // G re, G im, V re, V im
+    const int k = blockIdx.x % m, sp = blockIdx.x / m, tid = threadIdx.x;
+    const int64_t quads = (NL + GL - 1) / GL;
+    const int64_t l0 = quads * sp / splits * GL, l1 = min(NL, quads * (sp + 1) / splits * GL);
+    const int64_t plane = (int64_t)m * W * NL;
+    const float *src[4] = {G + (int64_t)k * W * NL, G + plane + (int64_t)k * W * NL, V + (int64_t)k * W * NL,
+                           V + plane + (int64_t)k * W * NL};
+    const int n4 = (W + 3) >> 2, grp = tid >> 6, e = tid & 63;
+    const int ig = e % n4, og = e / n4;
+    const bool active = og < n4;
+    const bool vec = (NL & 3) == 0;
+    float re[4][4], im[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int o = 0; o < 4; ++o) re[i][o] = im[i][o] = 0.f;
+    for (int q = tid; q < 4 * MAXW * GLP; q += TPB) (&sh[0][0][0])[q] = 0.f;
+    __syncthreads();
+    for (int64_t l = l0; l < l1; l += GL) {
+        for (int q = tid; q < 4 * W * (GL / 4); q += TPB) {
+            const int x = (q % (GL / 4)) * 4, c = (q / (GL / 4)) % W, f = q / (GL / 4 * W);
+            const float *p = src[f] + (int64_t)c * NL + l + x;
+            float4 w = f4(0.f);
+            if (vec) {
+                if (l + x < l1) w = *reinterpret_cast<const float4 *>(p);
+            } else {
+                if (l + x < l1) w.x = p[0];
+                if (l + x + 1 < l1) w.y = p[1];
+                if (l + x + 2 < l1) w.z = p[2];
+                if (l + x + 3 < l1) w.w = p[3];
+            }
+            *reinterpret_cast<float4 *>(&sh[f][c][x]) = w;
+        }
+        __syncthreads();
+        if (active) {
+            for (int x = grp * 4; x < GL; x += 16) {
+                float4 gr[4], gi[4];
+#pragma unroll
+                for (int o = 0; o < 4; ++o) {
+                    const int row = min(og + n4 * o, MAXW - 1);
+                    gr[o] = *reinterpret_cast<const float4 *>(&sh[0][row][x]);
+                    gi[o] = *reinterpret_cast<const float4 *>(&sh[1][row][x]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int row = min(ig + n4 * i, MAXW - 1);
+                    const float4 vr = *reinterpret_cast<const float4 *>(&sh[2][row][x]);
+                    const float4 vi = *reinterpret_cast<const float4 *>(&sh[3][row][x]);
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) {           // g conj(v)
+                        float a = re[i][o], b = im[i][o];
+                        a = fmaf(gr[o].x, vr.x, a); a = fmaf(gi[o].x, vi.x, a);
+                        b = fmaf(gi[o].x, vr.x, b); b = fmaf(-gr[o].x, vi.x, b);
+                        a = fmaf(gr[o].y, vr.y, a); a = fmaf(gi[o].y, vi.y, a);
+                        b = fmaf(gi[o].y, vr.y, b); b = fmaf(-gr[o].y, vi.y, b);
+                        a = fmaf(gr[o].z, vr.z, a); a = fmaf(gi[o].z, vi.z, a);
+                        b = fmaf(gi[o].z, vr.z, b); b = fmaf(-gr[o].z, vi.z, b);
+                        a = fmaf(gr[o].w, vr.w, a); a = fmaf(gi[o].w, vi.w, a);
+                        b = fmaf(gi[o].w, vr.w, b); b = fmaf(-gr[o].w, vi.w, b);
+                        re[i][o] = a;
+                        im[i][o] = b;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+    // the four line groups' sums, in order
+    float2 *acc = reinterpret_cast<float2 *>(&sh[0][0][0]);      // [MAXW][MAXW]
+    for (int g = 0; g < 4; ++g) {
+        if (active && grp == g)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int o = 0; o < 4; ++o) {
+                    const int ri = ig + n4 * i, ro = og + n4 * o;
+                    if (ri >= W || ro >= W) continue;
+                    float2 *d = acc + ri * MAXW + ro;
+                    *d = g == 0 ? make_float2(re[i][o], im[i][o]) : make_float2(d->x + re[i][o], d->y + im[i][o]);
+                }
+        __syncthreads();
+    }
+    float2 *out = part + ((int64_t)sp * m + k) * W * W;
+    for (int q = tid; q < W * W; q += TPB) out[q] = acc[q / W * MAXW + q % W];
+}
+
+// part [splits][k][i][o] -> gR [i][o][k]
+__global__ void k_grad_r_sum(const float2 *__restrict__ part, int W, int m, int splits, float *__restrict__ gR)
+{
+    const int n = m * W * W, t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    float re = 0.f, im = 0.f;
+    for (int s = 0; s < splits; ++s) {
+        const float2 p = part[(int64_t)s * n + t];
+        re += p.x;
+        im += p.y;
+    }
+    const int k = t / (W * W), io = t % (W * W);
+    gR[((int64_t)io * m + k) * 2] = re;
+    gR[((int64_t)io * m + k) * 2 + 1] = im;
+}
+
+// ---------------------------------------------------------------------------
+// pointwise networks
+// ---------------------------------------------------------------------------
+template <int ACT>
+__device__ __forceinline__ float act_of(float z, float w0)
+{
+    if (ACT == ACT_GELU) return 0.5f * z * (1.f + erff(z * 0.70710678118654752f));
+    return sinf(w0 * z);
+}
+
+// value and derivative
+template <int ACT>
+__device__ __forceinline__ void act_both(float z, float w0, float &h, float &dh)
+{
+    if (ACT == ACT_GELU) {
+        const float c = 0.5f * (1.f + erff(z * 0.70710678118654752f));
+        h = z * c;
+        dh = c + z * expf(-0.5f * z * z) * 0.39894228040143268f;
+    } else {
+        float sn, cs;
+        sincosf(w0 * z, &sn, &cs);
+        h = sn;
+        dh = w0 * cs;
+    }
+}
+
+// weights into shared memory: W1 [ch][CI], W2 transposed [ch][CO], zeros in
+// the padding (chp rows)
+template <int CI, int CO>
+__device__ __forceinline__ void stage_weights(const Mlp &p, int chp, float *w1, float *w2, float *b1, float *b2)
+{
+    for (int q = threadIdx.x; q < chp * CI; q += blockDim.x) {
+        const int j = q / CI, c = q % CI;
+        w1[q] = j < p.ch && c < p.ci ? p.W1[j * p.ci + c] : 0.f;
+    }
+    for (int q = threadIdx.x; q < chp * CO; q += blockDim.x) {
+        const int j = q / CO, o = q % CO;
+        w2[q] = j < p.ch && o < p.co ? p.W2[o * p.ch + j] : 0.f;
+    }
+    for (int q = threadIdx.x; q < chp; q += blockDim.x) b1[q] = q < p.ch ? p.b1[q] : 0.f;
+    if (b2)
+        for (int q = threadIdx.x; q < CO; q += blockDim.x) b2[q] = q < p.co ? p.b2[q] : 0.f;
+}
+
+template <int V> struct Vec;
+template <> struct Vec<1> { using T = float; };
+template <> struct Vec<2> { using T = float2; };
+
+// A thread's V cells keep their CI inputs and CO outputs in registers; the
+// weights are broadcast from shared memory, so the kernel is bound by the
+// multiply-adds and the activation.
+template <int CI, int CO, int ACT, int V>
+__global__ void __launch_bounds__(TPB) k_mlp(const Mlp p, const float *__restrict__ x, const float *res, float *y,
+                                             int B, int64_t N)
+{
+    extern __shared__ float4 raw[];
+    const int chp = (p.ch + 1) & ~1;
+    float *w1 = reinterpret_cast<float *>(raw), *w2 = w1 + chp * CI, *b1 = w2 + chp * CO, *b2 = b1 + ((chp + 3) & ~3);
+    stage_weights<CI, CO>(p, chp, w1, w2, b1, b2);
+    __syncthreads();
+    using T = typename Vec<V>::T;
+    const int64_t items = B * N / V;
+    for (int64_t it = (int64_t)blockIdx.x * TPB + threadIdx.x; it < items; it += (int64_t)gridDim.x * TPB) {
+        const int64_t cell = it * V, b = cell / N, n = cell - b * N;
+        float in[CI][V], out[CO][V];
+#pragma unroll
+        for (int c = 0; c < CI; ++c) {
+            if (c < p.ci) *reinterpret_cast<T *>(in[c]) = *reinterpret_cast<const T *>(x + (b * p.ci + c) * N + n);
+            else
+#pragma unroll
+                for (int q = 0; q < V; ++q) in[c][q] = 0.f;
+        }
+#pragma unroll
+        for (int o = 0; o < CO; ++o)
+#pragma unroll
+            for (int q = 0; q < V; ++q) out[o][q] = b2[o];
+#pragma unroll 1
+        for (int j = 0; j < chp; j += 2) {
+            float z[2][V];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                for (int q = 0; q < V; ++q) z[h][q] = b1[j + h];
+            }
+#pragma unroll
+            for (int c = 0; c < CI; c += 4)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float4 w = *reinterpret_cast<const float4 *>(w1 + (j + h) * CI + c);
+#pragma unroll
+                    for (int q = 0; q < V; ++q) {
+                        z[h][q] = fmaf(w.x, in[c][q], z[h][q]);
+                        z[h][q] = fmaf(w.y, in[c + 1][q], z[h][q]);
+                        z[h][q] = fmaf(w.z, in[c + 2][q], z[h][q]);
+                        z[h][q] = fmaf(w.w, in[c + 3][q], z[h][q]);
+                    }
+                }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int q = 0; q < V; ++q) z[h][q] = act_of<ACT>(z[h][q], p.w0);
+#pragma unroll
+            for (int o = 0; o < CO; o += 4)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float4 w = *reinterpret_cast<const float4 *>(w2 + (j + h) * CO + o);
+#pragma unroll
+                    for (int q = 0; q < V; ++q) {
+                        out[o][q] = fmaf(w.x, z[h][q], out[o][q]);
+                        out[o + 1][q] = fmaf(w.y, z[h][q], out[o + 1][q]);
+                        out[o + 2][q] = fmaf(w.z, z[h][q], out[o + 2][q]);
+                        out[o + 3][q] = fmaf(w.w, z[h][q], out[o + 3][q]);
+                    }
+                }
+        }
+#pragma unroll
+        for (int o = 0; o < CO; ++o) {
+            if (o >= p.co) break;
+            const int64_t at = (b * p.co + o) * N + n;
+            if (res) {
+                float r[V];
+                *reinterpret_cast<T *>(r) = *reinterpret_cast<const T *>(res + at);
+#pragma unroll
+                for (int q = 0; q < V; ++q) out[o][q] += r[q];
+            }
+            *reinterpret_cast<T *>(y + at) = *reinterpret_cast<const T *>(out[o]);
+        }
+    }
+}
+
+constexpr int BT = 128;                      // threads of the backward kernel = cells of a tile
+constexpr int BTP = BT + 4;                  // row stride of its tiles
+constexpr int HC = 32;                       // hidden units per chunk
+
+// Backward of the same network, a persistent block over tiles of 128 cells,
+// one cell per thread: the hidden values are recomputed (cheaper than keeping
+// two fields per layer), 32 hidden units at a time; their values and
+// gradients meet the inputs and output gradients in shared memory, where the
+// block's threads hold 2 x 4 entries of both weight gradients each.
+template <int CI, int CO, int ACT, int NCH, bool GX>
+__global__ void __launch_bounds__(BT) k_mlp_bwd(const Mlp p, const float *__restrict__ x, const float *__restrict__ g,
+                                                float *__restrict__ gx, int B, int64_t N, float *__restrict__ part)
+{
+    extern __shared__ float4 raw[];
+    constexpr int chp = NCH * HC, N1 = CI / 8, N2 = CO / 8;
+    float *w1 = reinterpret_cast<float *>(raw), *w2 = w1 + chp * CI, *b1 = w2 + chp * CO;
+    float *X = b1 + chp, *G = X + CI * BTP, *H = G + CO * BTP, *GH = H + HC * BTP;
+    stage_weights<CI, CO>(p, chp, w1, w2, b1, nullptr);
+    __syncthreads();
+    const int tid = threadIdx.x, hg = tid >> 3, cg = tid & 7;
+    float a1[NCH][2][N1], a2[NCH][2][N2], s1[NCH][2], s2[N2];
+#pragma unroll
+    for (int k = 0; k < NCH; ++k)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            s1[k][h] = 0.f;
+#pragma unroll
+            for (int c = 0; c < N1; ++c) a1[k][h][c] = 0.f;
+#pragma unroll
+            for (int c = 0; c < N2; ++c) a2[k][h][c] = 0.f;
+        }
+#pragma unroll
+    for (int c = 0; c < N2; ++c) s2[c] = 0.f;
+    const int64_t cells = B * N;
+    for (int64_t c0 = (int64_t)blockIdx.x * BT; c0 < cells; c0 += (int64_t)gridDim.x * BT) {
+        const int64_t cell = c0 + tid;
+        const bool ok = cell < cells;
+        const int64_t b = cell / N, n = cell - b * N;
+        float in[CI], go[CO], gi[GX ? CI : 1];
+#pragma unroll
+        for (int c = 0; c < CI; ++c) {
+            in[c] = ok && c < p.ci ? x[(b * p.ci + c) * N + n] : 0.f;
+            X[c * BTP + tid] = in[c];
+        }
+#pragma unroll
+        for (int o = 0; o < CO; ++o) {
+            go[o] = ok && o < p.co ? g[(b * p.co + o) * N + n] : 0.f;
+            G[o * BTP + tid] = go[o];
+        }
+        if (GX)
+#pragma unroll
+            for (int c = 0; c < CI; ++c) gi[c] = 0.f;
+#pragma unroll
+        for (int k = 0; k < NCH; ++k) {
+#pragma unroll 1
+            for (int jj = 0; jj < HC; jj += 2) {
+                const int j = k * HC + jj;
+                float z[2], gh[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    z[h] = b1[j + h];
+                    gh[h] = 0.f;
+                }
+#pragma unroll
+                for (int c = 0; c < CI; c += 4)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float4 w = *reinterpret_cast<const float4 *>(w1 + (j + h) * CI + c);
+                        z[h] = fmaf(w.x, in[c], z[h]);
+                        z[h] = fmaf(w.y, in[c + 1], z[h]);
+                        z[h] = fmaf(w.z, in[c + 2], z[h]);
+                        z[h] = fmaf(w.w, in[c + 3], z[h]);
+                    }
+#pragma unroll
+                for (int o = 0; o < CO; o += 4)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float4 w = *reinterpret_cast<const float4 *>(w2 + (j + h) * CO + o);
+                        gh[h] = fmaf(w.x, go[o], gh[h]);
+                        gh[h] = fmaf(w.y, go[o + 1], gh[h]);
+                        gh[h] = fmaf(w.z, go[o + 2], gh[h]);
+                        gh[h] = fmaf(w.w, go[o + 3], gh[h]);
+                    }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float hv, dh;
+                    act_both<ACT>(z[h], p.w0, hv, dh);
+                    gh[h] *= dh;
+                    H[(jj + h) * BTP + tid] = hv;
+                    GH[(jj + h) * BTP + tid] = gh[h];
+                }
+                if (GX)
+#pragma unroll
+                    for (int c = 0; c < CI; c += 4)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const float4 w = *reinterpret_cast<const float4 *>(w1 + (j + h) * CI + c);
+                            gi[c] = fmaf(w.x, gh[h], gi[c]);
+                            gi[c + 1] = fmaf(w.y, gh[h], gi[c + 1]);
+                            gi[c + 2] = fmaf(w.z, gh[h], gi[c + 2]);
+                            gi[c + 3] = fmaf(w.w, gh[h], gi[c + 3]);
+                        }
+            }
+            __syncthreads();
+#pragma unroll 2
+            for (int q = 0; q < BT; q += 4) {
+                float4 hv[2], gv[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    gv[h] = *reinterpret_cast<const float4 *>(GH + (2 * hg + h) * BTP + q);
+                    hv[h] = *reinterpret_cast<const float4 *>(H + (2 * hg + h) * BTP + q);
+                    s1[k][h] += (gv[h].x + gv[h].y) + (gv[h].z + gv[h].w);
+                }
+#pragma unroll
+                for (int c = 0; c < N1; ++c) {
+                    const float4 w = *reinterpret_cast<const float4 *>(X + (cg + 8 * c) * BTP + q);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float s = a1[k][h][c];
+                        s = fmaf(gv[h].x, w.x, s);
+                        s = fmaf(gv[h].y, w.y, s);
+                        s = fmaf(gv[h].z, w.z, s);
+                        a1[k][h][c] = fmaf(gv[h].w, w.w, s);
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < N2; ++c) {
+                    const float4 w = *reinterpret_cast<const float4 *>(G + (cg + 8 * c) * BTP + q);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float s = a2[k][h][c];
+                        s = fmaf(hv[h].x, w.x, s);
+                        s = fmaf(hv[h].y, w.y, s);
+                        s = fmaf(hv[h].z, w.z, s);
+                        a2[k][h][c] = fmaf(hv[h].w, w.w, s);
+                    }
+                    if (k == 0) s2[c] += (w.x + w.y) + (w.z + w.w);
+                }
+            }
+            __syncthreads();
+        }
+        if (GX && ok)
+#pragma unroll
+            for (int c = 0; c < CI; ++c)
+                if (c < p.ci) gx[(b * p.ci + c) * N + n] = gi[c];
+    }
+    // this block's sums, in the parameters' order: W1 [ch][ci], b1, W2 [co][ch], b2
+    const int n1 = p.ch * p.ci, n2 = p.co * p.ch;
+    float *d = part + (int64_t)blockIdx.x * (n1 + p.ch + n2 + p.co);
+#pragma unroll
+    for (int k = 0; k < NCH; ++k)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = k * HC + 2 * hg + h;
+            if (j >= p.ch) continue;
+#pragma unroll
+            for (int c = 0; c < N1; ++c)
+                if (cg + 8 * c < p.ci) d[j * p.ci + cg + 8 * c] = a1[k][h][c];
+            if (cg == 0) d[n1 + j] = s1[k][h];
+#pragma unroll
+            for (int c = 0; c < N2; ++c)
+                if (cg + 8 * c < p.co) d[n1 + p.ch + (cg + 8 * c) * p.ch + j] = a2[k][h][c];
+        }
+    if (hg == 0)
+#pragma unroll
+        for (int c = 0; c < N2; ++c)
+            if (cg + 8 * c < p.co) d[n1 + p.ch + n2 + cg + 8 * c] = s2[c];
+}
+
+// out[q] = sum over the parts, 8 interleaved FP64 sums added in order
+__global__ void __launch_bounds__(256) k_sum_parts(const float *__restrict__ part, int P, int n, float *__restrict__ out)
+{
+    __shared__ double sh[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = blockIdx.x * 32 + lane;
+    double s = 0.0;
+    if (q < n)
+        for (int p = w; p < P; p += 8) s += part[(int64_t)p * n + q];
+    sh[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && q < n) {
+        for (int k = 1; k < 8; ++k) s += sh[k][lane];
+        out[q] = (float)s;
+    }
+}
+
+int round4(int v) { return (v + 3) & ~3; }
+
+// smallest stride >= v, a multiple of 4, that leaves `rem` on division by 32
+int stride_for(int v, int rem)
+{
+    v = round4(v);
+    while (v % 32 != rem) v += 4;
+    return v;
+}
+
+}  // namespace
+
+// T: as many lines as leave room for two blocks per SM (long runs along the
+// lines and fewer reads of the weights), 4 lines in one block where they do not.
+bool axis_plan(Axis &a, int L, int m, int rows, int64_t S, int64_t outer, int W)
+{
+    if (W < 1 || W > MAXW) return false;
+    a = Axis{};
+    a.L = L; a.m = m; a.rows = rows; a.S = S; a.outer = outer;
+    a.q = L % 4 == 0 ? 2 : 1;
+    a.nq = a.q == 2 ? L / 4 + 1 : L / 2 + 1;
+    a.mk = (m + a.q - 1) / a.q;
+    a.KG = (a.mk + 3) / 4;
+    a.NG = (a.nq + 3) / 4;
+    for (int T = 16; T >= 4; T /= 2) {
+        a.T = T;
+        a.DS = stride_for(2 * a.q * a.nq * T, T);
+        a.KS = stride_for(W * T, 4);
+        a.smem = sizeof(float) * ((size_t)std::max(W * a.DS, 2 * m * a.KS) + (size_t)2 * m * a.KS);
+        if (a.smem <= SMEM_TWO) return true;
+    }
+    return a.smem <= SMEM_MAX;
+}
+
+void axis_tables(const Axis &a, std::vector<float> &out, size_t count[4])
+{
+    out.clear();
+    auto ang = [&](int k, int n) { return 2.0 * M_PI * (double)(((int64_t)k * n) % a.L) / a.L; };
+    for (int f = 0; f < 4; ++f) {
+        const size_t before = out.size();
+        const bool sine = f & 1;
+        for (int par = 0; par < a.q; ++par) {
+            if (f < 2) {
+                for (int n = 0; n < a.nq; ++n)
+                    for (int kk = 0; kk < 4 * a.KG; ++kk) {
+                        const int k = par + a.q * kk;
+                        out.push_back(k < a.m ? (float)(sine ? std::sin(ang(k, n)) : std::cos(ang(k, n))) : 0.f);
+                    }
+            } else {
+                for (int kk = 0; kk < a.mk; ++kk)
+                    for (int g = 0; g < a.NG; ++g)
+                        for (int j = 0; j < 4; ++j) {
+                            const int k = par + a.q * kk, n = g + j * a.NG;
+                            const bool in = k < a.m && n < a.nq;
+                            out.push_back(in ? (float)(sine ? std::sin(ang(k, n)) : std::cos(ang(k, n))) : 0.f);
+                        }
+            }
+        }
+        count[f] = out.size() - before;
+    }
+}
+
+void spectral(const Axis &a, const float *v, float *u, int B, int W, int64_t N, const float2 *R, const float *wk,
+              const float *ak, float *spec, bool accumulate, cudaStream_t s)
+{
+    const int64_t run = a.rows ? a.outer : a.S;
+    const int tiles = (int)((run + a.T - 1) / a.T);
+    const int64_t blocks = (int64_t)B * tiles * (a.rows ? 1 : a.outer), NL = B * a.lines();
+    if (a.rows)
+        k_spectral<1><<<(unsigned)blocks, TPB, a.smem, s>>>(a, v, u, W, N, R, wk, ak, spec, NL, tiles, accumulate);
+    else
+        k_spectral<0><<<(unsigned)blocks, TPB, a.smem, s>>>(a, v, u, W, N, R, wk, ak, spec, NL, tiles, accumulate);
+}
+
+void pack_r(const PackR &p, int W, cudaStream_t s)
+{
+    const int Wp = round4(W), m = std::max({p.a[0].m, p.a[1].m, p.a[2].m});
+    k_pack_r<<<dim3((unsigned)std::min(gb300::sm_count() * 4, (m * W * Wp + TPB - 1) / TPB), 3), TPB, 0, s>>>(p, W, Wp);
+}
+
+int grad_r_parts(int m, int64_t lines)
+{
+    const int want = std::max(1, 4 * gb300::sm_count() / std::max(1, m));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(want, (lines + GL - 1) / GL));
+}
+
+void grad_r(const float *G, const float *V, int W, int m, int64_t lines, float2 *part, float *gR, cudaStream_t s)
+{
+    const int sp = grad_r_parts(m, lines);
+    k_grad_r<<<m * sp, TPB, 0, s>>>(G, V, W, m, lines, sp, part);
+    k_grad_r_sum<<<(m * W * W + TPB - 1) / TPB, TPB, 0, s>>>(part, W, m, sp, gR);
+}
+
+bool mlp_fits(int ci, int ch, int co) { return ci <= MAXW && co <= MAXW && ch <= 128; }
+
+namespace {
+
+template <int CI, int CO, int ACT>
+void mlp_v(const Mlp &p, const float *x, const float *res, float *y, int B, int64_t N, cudaStream_t s)
+{
+    const int chp = (p.ch + 1) & ~1;
+    const size_t smem = sizeof(float) * (size_t)(chp * (CI + CO) + round4(chp) + CO);
+    const uintptr_t al = (uintptr_t)x | (uintptr_t)res | (uintptr_t)y;
+    const bool two = N % 2 == 0 && (al & 7) == 0;
+    const int64_t items = B * N / (two ? 2 : 1);
+    const int grid = (int)std::min<int64_t>((items + TPB - 1) / TPB, (int64_t)gb300::sm_count() * 2);
+    if (two) k_mlp<CI, CO, ACT, 2><<<grid, TPB, smem, s>>>(p, x, res, y, B, N);
+    else k_mlp<CI, CO, ACT, 1><<<grid, TPB, smem, s>>>(p, x, res, y, B, N);
+}
+
+template <int ACT>
+void mlp_act(const Mlp &p, const float *x, const float *res, float *y, int B, int64_t N, cudaStream_t s)
+{
+    if (p.ci <= 8) mlp_v<8, 32, ACT>(p, x, res, y, B, N, s);
+    else if (p.co <= 8) mlp_v<32, 8, ACT>(p, x, res, y, B, N, s);
+    else mlp_v<32, 32, ACT>(p, x, res, y, B, N, s);
+}
+
+template <int CI, int CO, int ACT, int NCH, bool GX>
+size_t bwd_smem() { return sizeof(float) * (size_t)(NCH * HC * (CI + CO + 1) + (CI + CO + 2 * HC) * BTP); }
+
+int bwd_grid(int64_t cells) { return (int)std::min<int64_t>((cells + BT - 1) / BT, mlp_parts()); }
+
+template <int CI, int CO, int ACT, int NCH, bool GX>
+void bwd_k(const Mlp &p, const float *x, const float *g, float *gx, float *part, int B, int64_t N, cudaStream_t s)
+{
+    k_mlp_bwd<CI, CO, ACT, NCH, GX><<<bwd_grid(B * N), BT, bwd_smem<CI, CO, ACT, NCH, GX>(), s>>>(p, x, g, gx, B, N, part);
+}
+
+template <int CI, int CO, int ACT, bool GX>
+void bwd_n(const Mlp &p, const float *x, const float *g, float *gx, float *part, int B, int64_t N, cudaStream_t s)
+{
+    if (p.ch <= HC) bwd_k<CI, CO, ACT, 1, GX>(p, x, g, gx, part, B, N, s);
+    else if (p.ch <= 2 * HC) bwd_k<CI, CO, ACT, 2, GX>(p, x, g, gx, part, B, N, s);
+    else bwd_k<CI, CO, ACT, 4, GX>(p, x, g, gx, part, B, N, s);
+}
+
+template <int ACT>
+void bwd_act(const Mlp &p, const float *x, const float *g, float *gx, float *part, int B, int64_t N, cudaStream_t s)
+{
+    if (!gx && p.ci <= 8) bwd_n<8, 32, ACT, false>(p, x, g, gx, part, B, N, s);
+    else if (!gx) bwd_n<32, 32, ACT, false>(p, x, g, gx, part, B, N, s);
+    else if (p.co <= 8) bwd_n<32, 8, ACT, true>(p, x, g, gx, part, B, N, s);
+    else bwd_n<32, 32, ACT, true>(p, x, g, gx, part, B, N, s);
+}
+
+template <class K>
+bool big(K k, size_t bytes)
+{
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+}
+
+template <int CI, int CO, int ACT, bool GX>
+bool big_bwd()
+{
+    return big(k_mlp_bwd<CI, CO, ACT, 1, GX>, bwd_smem<CI, CO, ACT, 1, GX>()) &&
+           big(k_mlp_bwd<CI, CO, ACT, 2, GX>, bwd_smem<CI, CO, ACT, 2, GX>()) &&
+           big(k_mlp_bwd<CI, CO, ACT, 4, GX>, bwd_smem<CI, CO, ACT, 4, GX>());
+}
+
+template <int ACT>
+bool big_act()
+{
+    return big_bwd<8, 32, ACT, false>() && big_bwd<32, 32, ACT, false>() && big_bwd<32, 8, ACT, true>() &&
+           big_bwd<32, 32, ACT, true>();
+}
+
+}  // namespace
+
+void mlp(const Mlp &p, const float *x, const float *res, float *y, int B, int64_t N, cudaStream_t s)
+{
+    if (p.act == ACT_SIREN) mlp_act<ACT_SIREN>(p, x, res, y, B, N, s);
+    else mlp_act<ACT_GELU>(p, x, res, y, B, N, s);
+}
+
+int mlp_parts() { return gb300::sm_count() * 3; }
+
+void mlp_bwd(const Mlp &p, const float *x, const float *g, float *gx, float *part, float *gw, int B, int64_t N,
+             cudaStream_t s)
+{
+    if (p.act == ACT_SIREN) bwd_act<ACT_SIREN>(p, x, g, gx, part, B, N, s);
+    else bwd_act<ACT_GELU>(p, x, g, gx, part, B, N, s);
+    const int n = p.ch * p.ci + p.ch + p.co * p.ch + p.co;
+    k_sum_parts<<<(n + 31) / 32, 256, 0, s>>>(part, bwd_grid(B * N), n, gw);
+}
+
+// The dynamic shared-memory limits are per device: set on every creation.
+bool set_attrs()
+{
+    return big(k_spectral<0>, SMEM_MAX) && big(k_spectral<1>, SMEM_MAX) && big_act<ACT_GELU>() && big_act<ACT_SIREN>();
+}
+
+}  // namespace ffno
