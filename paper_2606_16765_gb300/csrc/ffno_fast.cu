@@ -44,309 +44,414 @@ struct Tile {
     int valid;           // lines of this tile that exist
 };
 
-template <int ROWS>
-__device__ __forceinline__ float4 load4(const float *p, const Tile &t, int64_t off, int l, bool vec)
+__device__ __forceinline__ void async16(float *dst, const float *src)
 {
-    if (!ROWS && vec) return l < t.valid ? *reinterpret_cast<const float4 *>(p + off) : f4(0.f);
-    float4 r = f4(0.f);
-    if (l < t.valid) r.x = p[off];
-    if (l + 1 < t.valid) r.y = p[off + t.sl];
-    if (l + 2 < t.valid) r.z = p[off + 2 * t.sl];
-    if (l + 3 < t.valid) r.w = p[off + 3 * t.sl];
-    return r;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
 }
 
+__device__ __forceinline__ void async8(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+__device__ __forceinline__ void async4(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+__device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// copy the four lines into shared memory (this thread's own 16 bytes), zeros
+// past the tile's lines
 template <int ROWS>
-__device__ __forceinline__ void store4(float *p, const Tile &t, int64_t off, int l, bool vec, const float4 &v)
+__device__ __forceinline__ void fetch4(float *dst, const float *p, const Tile &t, int64_t off, int l, bool vec)
 {
     if (!ROWS && vec) {
-        if (l < t.valid) *reinterpret_cast<float4 *>(p + off) = v;
+        if (l < t.valid) async16(dst, p + off);
+        else *reinterpret_cast<float4 *>(dst) = f4(0.f);
         return;
     }
-    if (l < t.valid) p[off] = v.x;
-    if (l + 1 < t.valid) p[off + t.sl] = v.y;
-    if (l + 2 < t.valid) p[off + 2 * t.sl] = v.z;
-    if (l + 3 < t.valid) p[off + 3 * t.sl] = v.w;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (l + q < t.valid) async4(dst + q, p + off + q * t.sl);
+        else dst[q] = 0.f;
 }
 
-// A block: T lines x W channels x L samples.  Phases, a barrier between them:
-//   fold     global -> D [c][class][n][T]: even and odd parts of the lines,
-//            split by the parity of the wave number they serve
+// Store, or add without reading back: one kernel at a time adds to a field, one
+// addition per element, so the sum does not depend on the order of the blocks.
+template <int ROWS>
+__device__ __forceinline__ void store4(float *p, const Tile &t, int64_t off, int l, bool vec, bool add, const float4 &v)
+{
+    if (!ROWS && vec) {
+        if (l >= t.valid) return;
+        if (add) atomicAdd(reinterpret_cast<float4 *>(p + off), v);
+        else *reinterpret_cast<float4 *>(p + off) = v;
+        return;
+    }
+    const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (l + q < t.valid) {
+            if (add) atomicAdd(p + off + q * t.sl, w[q]);
+            else p[off + q * t.sl] = w[q];
+        }
+}
+
+// n / d for n, d < 2^16: mul = ceil(2^32 / d) (0 stands for d = 1)
+__device__ __forceinline__ int fdiv(int n, uint32_t mul) { return mul ? (int)__umulhi((uint32_t)n, mul) : n; }
+
+// V(o) += R(i, o) V(i) for 4 lines and 4 outputs: re, im of the input's lines
+__device__ __forceinline__ void mix4(float4 *gr, float4 *gi, const float4 *w, const float4 &x, const float4 &y)
+{
+    const float c[8] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w};
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+        fma4(gr[o], c[2 * o], x);
+        fma4(gr[o], -c[2 * o + 1], y);
+        fma4(gi[o], c[2 * o + 1], x);
+        fma4(gi[o], c[2 * o], y);
+    }
+}
+
+// A persistent block over tiles of T lines x W channels x L samples.  Phases,
+// a barrier between them:
+//   fold     D [c][class][n][T]: even and odd parts of the lines, split by the
+//            parity of the wave number they serve; each thread folds in place
+//            what it copied itself
 //   forward  V [k][c][T]: thread = 4 wave numbers x 4 lines, real and
 //            imaginary part: 32 multiply-adds per four 16-byte operands
-//   mix      G [k][o][T] over D: thread = 4 lines x 4 outputs (complex), the
-//            weights read once per block from L2
+//   mix      in place on V: thread = 4 lines x 4 outputs (complex); the
+//            threads of one wave number and 4 lines sit in one warp, read all
+//            inputs, then write; the weights come from L2, two steps ahead
 //   inverse  thread = 4 terms x 4 lines of all four symmetric sums, unfolded
 //            into 16 samples and stored
-template <int ROWS>
-__global__ void __launch_bounds__(TPB, 2) k_spectral(const Axis a, const float *__restrict__ v, float *u, int W,
+// D is free after the forward phase: the next tile's copies are issued there
+// and land behind the mixing and the inverse.
+// WC: the width when it is a constant (full unrolling), else 0.
+template <int ROWS, int WC>
+__global__ void __launch_bounds__(TPB, 2) k_spectral(const Axis a, const float *__restrict__ v, float *u, int Wr,
                                                      int64_t N, const float2 *__restrict__ R,
                                                      const float *__restrict__ wk, const float *__restrict__ ak,
-                                                     float *__restrict__ spec, int64_t NL, int tiles, int accumulate)
+                                                     float *__restrict__ spec, int64_t NL, int tiles, int total,
+                                                     int accumulate)
 {
     extern __shared__ float4 raw[];
+    const int W = WC ? WC : Wr;
     float *D = reinterpret_cast<float *>(raw);
-    float *Gre = D, *Gim = D + a.m * a.KS;
-    float *Vre = D + max(W * a.DS, 2 * a.m * a.KS), *Vim = Vre + a.m * a.KS;
+    float *Vre = D + W * a.DS, *Vim = Vre + a.m * a.KS;
     const int T = a.T, TQ = T >> 2, tid = threadIdx.x;
     const int tqs = TQ == 1 ? 0 : (TQ == 2 ? 1 : 2);
-    // the block's lines
-    Tile t;
-    int64_t line0;
-    {
-        int64_t w = blockIdx.x;
+    const bool vec = !ROWS && (a.S & 3) == 0;
+    const int L = a.L, nq = a.nq, cls = nq * T;
+
+    auto lines_of = [&](int64_t w, int64_t &line0) {
+        Tile t;
         const int64_t ti = w % tiles;
         w /= tiles;
         if (ROWS) {
-            const int64_t b = w;
-            t.base = b * W * N + ti * T * a.L;
+            t.base = w * W * N + ti * T * L;
             t.sn = 1;
-            t.sl = a.L;
+            t.sl = L;
             t.valid = (int)min((int64_t)T, a.outer - ti * T);
-            line0 = b * a.outer + ti * T;
+            line0 = w * a.outer + ti * T;
         } else {
             const int64_t o = w % a.outer, b = w / a.outer;
-            t.base = b * W * N + o * a.L * a.S + ti * T;
+            t.base = b * W * N + o * L * a.S + ti * T;
             t.sn = a.S;
             t.sl = 1;
             t.valid = (int)min((int64_t)T, a.S - ti * T);
             line0 = (b * a.outer + o) * a.S + ti * T;
         }
-    }
-    const bool vec = !ROWS && (a.S & 3) == 0;
-    const int L = a.L, nq = a.nq, cls = nq * T;
-
-    // fold
-    for (int idx = tid; idx < W * nq * TQ; idx += TPB) {
-        int j, l, c;
+        return t;
+    };
+    auto place = [&](int idx, int &j, int &l, int &c) {
         if (ROWS) {                                 // neighbouring threads: neighbouring samples
-            j = idx % nq;
-            const int r = idx / nq;
+            const int r = fdiv(idx, a.dnq);
+            j = idx - r * nq;
             l = (r & (TQ - 1)) << 2;
             c = r >> tqs;
         } else {
             l = (idx & (TQ - 1)) << 2;
             const int r = idx >> tqs;
-            j = r % nq;
-            c = r / nq;
+            c = fdiv(r, a.dnq);
+            j = r - c * nq;
         }
-        const int64_t p0 = t.base + (int64_t)c * N + (int64_t)l * t.sl;
-        auto ld = [&](int n) { return load4<ROWS>(v, t, p0 + (int64_t)n * t.sn, l, vec); };
-        float *d = D + c * a.DS + j * T + l;
-        if (a.q == 2) {
-            float4 e0, e1, o0, o1;
-            if (j == 0) {
-                const float4 x = ld(0), y = ld(L / 2);
-                e0 = x + y;
-                e1 = x - y;
-                o0 = o1 = f4(0.f);
-            } else if (4 * j == L) {
-                const float4 x = ld(j), y = ld(L - j);
-                e0 = x + y;
-                o1 = x - y;
-                e1 = o0 = f4(0.f);
-            } else {
-                const float4 x = ld(j), y = ld(L - j), z = ld(L / 2 - j), w = ld(L / 2 + j);
-                const float4 ea = x + y, eb = z + w, oa = x - y, ob = z - w;
-                e0 = ea + eb;
-                e1 = ea - eb;
-                o0 = oa - ob;
-                o1 = oa + ob;
+    };
+    // each thread copies its own (n, L - n, L/2 - n, L/2 + n) into the places
+    // of its four folded values
+    auto fetch = [&](const Tile &t) {
+        for (int idx = tid; idx < W * nq * TQ; idx += TPB) {
+            int j, l, c;
+            place(idx, j, l, c);
+            const int64_t p0 = t.base + (int64_t)c * N + (int64_t)l * t.sl;
+            auto ld = [&](float *dst, int n) { fetch4<ROWS>(dst, v, t, p0 + (int64_t)n * t.sn, l, vec); };
+            float *d = D + c * a.DS + j * T + l;
+            ld(d, j);
+            if (a.q == 2) {
+                ld(d + cls, j == 0 ? L / 2 : L - j);
+                if (j > 0 && 4 * j < L) {
+                    ld(d + 2 * cls, L / 2 - j);
+                    ld(d + 3 * cls, L / 2 + j);
+                }
+            } else if (j > 0 && 2 * j != L) {
+                ld(d + cls, L - j);
             }
-            *reinterpret_cast<float4 *>(d) = e0;
-            *reinterpret_cast<float4 *>(d + cls) = e1;
-            *reinterpret_cast<float4 *>(d + 2 * cls) = o0;
-            *reinterpret_cast<float4 *>(d + 3 * cls) = o1;
-        } else {
-            float4 e = ld(j), o = f4(0.f);
-            if (j > 0 && 2 * j != L) {
-                const float4 y = ld(L - j);
-                o = e - y;
-                e = e + y;
-            }
-            *reinterpret_cast<float4 *>(d) = e;
-            *reinterpret_cast<float4 *>(d + cls) = o;
         }
-    }
-    __syncthreads();
+    };
 
-    // forward: V(k) = wk (sum_n E cos - i sum_n O sin)
-    for (int idx = tid; idx < W * TQ * a.q * a.KG; idx += TPB) {
-        const int kg = idx % a.KG;
-        int r = idx / a.KG;
-        const int par = a.q == 2 ? (r & 1) : 0;
-        r = a.q == 2 ? r >> 1 : r;
-        const int l = (r & (TQ - 1)) << 2, c = r >> tqs;
-        const float *e = D + c * a.DS + par * cls + l, *o = e + a.q * cls;
-        const float4 *ct = a.ctab + (int64_t)par * nq * a.KG + kg, *st = a.stab + (int64_t)par * nq * a.KG + kg;
-        float4 re[4], im[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) re[k] = im[k] = f4(0.f);
-#pragma unroll 4
-        for (int n = 0; n < nq; ++n) {
-            const float4 cw = __ldg(ct + n * a.KG), sw = __ldg(st + n * a.KG);
-            const float4 x = *reinterpret_cast<const float4 *>(e + n * T);
-            const float4 y = *reinterpret_cast<const float4 *>(o + n * T);
-            fma4(re[0], cw.x, x);
-            fma4(re[1], cw.y, x);
-            fma4(re[2], cw.z, x);
-            fma4(re[3], cw.w, x);
-            fma4(im[0], sw.x, y);
-            fma4(im[1], sw.y, y);
-            fma4(im[2], sw.z, y);
-            fma4(im[3], sw.w, y);
-        }
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            const int k = par + a.q * (4 * kg + kk);
-            if (k >= a.m) break;
-            const float w = wk ? wk[k] : 1.f;
-            const float4 vr = mul4(w, re[kk]), vi = mul4(-w, im[kk]);
-            *reinterpret_cast<float4 *>(Vre + k * a.KS + c * T + l) = vr;
-            *reinterpret_cast<float4 *>(Vim + k * a.KS + c * T + l) = vi;
-            if (spec) {
-                const int64_t at = ((int64_t)k * W + c) * NL + line0 + l;
-                float *sr = spec + at, *si = sr + (int64_t)a.m * W * NL;
-                if (l + 4 <= t.valid && (at & 3) == 0 && (NL & 3) == 0) {
-                    *reinterpret_cast<float4 *>(sr) = vr;
-                    *reinterpret_cast<float4 *>(si) = vi;
+    int64_t line0 = 0, line_next = 0;
+    Tile t = lines_of(blockIdx.x, line0), tn = t;
+    fetch(t);
+    for (int w = blockIdx.x; w < total; w += gridDim.x, t = tn, line0 = line_next) {
+        async_wait();
+        for (int idx = tid; idx < W * nq * TQ; idx += TPB) {
+            int j, l, c;
+            place(idx, j, l, c);
+            float4 *d0 = reinterpret_cast<float4 *>(D + c * a.DS + j * T + l);
+            float4 *d1 = d0 + cls / 4, *d2 = d1 + cls / 4, *d3 = d2 + cls / 4;
+            const float4 x = *d0;
+            if (a.q == 2) {
+                const float4 y = *d1, e = x + y, o = x - y;
+                if (j == 0) {                       // x(0), x(L/2)
+                    *d0 = e;
+                    *d1 = o;
+                    *d2 = *d3 = f4(0.f);
+                } else if (4 * j == L) {            // x(L/4), x(3L/4)
+                    *d0 = e;
+                    *d1 = *d2 = f4(0.f);
+                    *d3 = o;
                 } else {
-                    const float *pr = &vr.x, *pi = &vi.x;
-                    for (int q = 0; q < 4 && l + q < t.valid; ++q) {
-                        sr[q] = pr[q];
-                        si[q] = pi[q];
+                    const float4 z = *d2, q = *d3, eb = z + q, ob = z - q;
+                    *d0 = e + eb;
+                    *d1 = e - eb;
+                    *d2 = o - ob;
+                    *d3 = o + ob;
+                }
+            } else if (j > 0 && 2 * j != L) {
+                const float4 y = *d1;
+                *d0 = x + y;
+                *d1 = x - y;
+            } else {
+                *d1 = f4(0.f);
+            }
+        }
+        __syncthreads();
+
+        // forward: V(k) = wk (sum_n E cos - i sum_n O sin)
+        for (int idx = tid; idx < W * TQ * a.q * a.KG; idx += TPB) {
+            int r = fdiv(idx, a.dKG);
+            const int kg = idx - r * a.KG;
+            const int par = a.q == 2 ? (r & 1) : 0;
+            r = a.q == 2 ? r >> 1 : r;
+            const int l = (r & (TQ - 1)) << 2, c = r >> tqs;
+            const float *e = D + c * a.DS + par * cls + l, *o = e + a.q * cls;
+            const float4 *ct = a.ctab + par * nq * a.KG + kg, *st = a.stab + par * nq * a.KG + kg;
+            float4 re[4], im[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) re[k] = im[k] = f4(0.f);
+#pragma unroll 4
+            for (int n = 0; n < nq; ++n) {
+                const float4 cw = __ldg(ct + n * a.KG), sw = __ldg(st + n * a.KG);
+                const float4 x = *reinterpret_cast<const float4 *>(e + n * T);
+                const float4 y = *reinterpret_cast<const float4 *>(o + n * T);
+                fma4(re[0], cw.x, x);
+                fma4(re[1], cw.y, x);
+                fma4(re[2], cw.z, x);
+                fma4(re[3], cw.w, x);
+                fma4(im[0], sw.x, y);
+                fma4(im[1], sw.y, y);
+                fma4(im[2], sw.z, y);
+                fma4(im[3], sw.w, y);
+            }
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                const int k = par + a.q * (4 * kg + kk);
+                if (k >= a.m) break;
+                const float sc = wk ? wk[k] : 1.f;
+                const float4 vr = mul4(sc, re[kk]), vi = mul4(-sc, im[kk]);
+                *reinterpret_cast<float4 *>(Vre + k * a.KS + c * T + l) = vr;
+                *reinterpret_cast<float4 *>(Vim + k * a.KS + c * T + l) = vi;
+                if (spec) {
+                    const int64_t at = ((int64_t)k * W + c) * NL + line0 + l;
+                    float *sr = spec + at, *si = sr + (int64_t)a.m * W * NL;
+                    if (l + 4 <= t.valid && (at & 3) == 0 && (NL & 3) == 0) {
+                        *reinterpret_cast<float4 *>(sr) = vr;
+                        *reinterpret_cast<float4 *>(si) = vi;
+                    } else {
+                        const float pr[4] = {vr.x, vr.y, vr.z, vr.w}, pi[4] = {vi.x, vi.y, vi.z, vi.w};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (l + q < t.valid) {
+                                sr[q] = pr[q];
+                                si[q] = pi[q];
+                            }
                     }
                 }
             }
         }
-    }
-    __syncthreads();
-
-    // mix: G(o) = ak sum_i V(i) R(i, o)
-    const int OG = (W + 3) >> 2;
-    for (int idx = tid; idx < a.m * TQ * OG; idx += TPB) {
-        const int og = idx % OG;
-        int r = idx / OG;
-        const int l = (r & (TQ - 1)) << 2, k = r >> tqs;
-        const float4 *rp = reinterpret_cast<const float4 *>(R + (int64_t)k * W * OG * 4 + og * 4);
-        const float *vr = Vre + k * a.KS + l, *vi = Vim + k * a.KS + l;
-        float4 gr[4], gi[4];
-#pragma unroll
-        for (int o = 0; o < 4; ++o) gr[o] = gi[o] = f4(0.f);
-#pragma unroll 4
-        for (int i = 0; i < W; ++i) {
-            const float4 r01 = __ldg(rp + (int64_t)i * OG * 2), r23 = __ldg(rp + (int64_t)i * OG * 2 + 1);
-            const float4 x = *reinterpret_cast<const float4 *>(vr + i * T);
-            const float4 y = *reinterpret_cast<const float4 *>(vi + i * T);
-            fma4(gr[0], r01.x, x);
-            fma4(gr[0], -r01.y, y);
-            fma4(gi[0], r01.y, x);
-            fma4(gi[0], r01.x, y);
-            fma4(gr[1], r01.z, x);
-            fma4(gr[1], -r01.w, y);
-            fma4(gi[1], r01.w, x);
-            fma4(gi[1], r01.z, y);
-            fma4(gr[2], r23.x, x);
-            fma4(gr[2], -r23.y, y);
-            fma4(gi[2], r23.y, x);
-            fma4(gi[2], r23.x, y);
-            fma4(gr[3], r23.z, x);
-            fma4(gr[3], -r23.w, y);
-            fma4(gi[3], r23.w, x);
-            fma4(gi[3], r23.z, y);
+        __syncthreads();
+        if (w + (int)gridDim.x < total) {
+            tn = lines_of(w + (int)gridDim.x, line_next);
+            fetch(tn);
         }
-        const float w = ak ? ak[k] : 1.f;
-#pragma unroll
-        for (int o = 0; o < 4; ++o) {
-            if (4 * og + o >= W) break;
-            *reinterpret_cast<float4 *>(Gre + k * a.KS + (4 * og + o) * T + l) = mul4(w, gr[o]);
-            *reinterpret_cast<float4 *>(Gim + k * a.KS + (4 * og + o) * T + l) = mul4(w, gi[o]);
-        }
-    }
-    __syncthreads();
 
-    // inverse: u(n) = sum_k (Gre cos - Gim sin)
-    for (int idx = tid; idx < W * TQ * a.NG; idx += TPB) {
-        const int ng = idx % a.NG;
-        int r = idx / a.NG;
-        const int l = (r & (TQ - 1)) << 2, c = r >> tqs;
-        const float *gr = Gre + c * T + l, *gi = Gim + c * T + l;
-        const float4 *ct = a.cinv + ng, *st = a.sinv + ng;
-        const int64_t p0 = t.base + (int64_t)c * N + (int64_t)l * t.sl;
-        auto put = [&](int n, const float4 &x) {
-            const int64_t off = p0 + (int64_t)n * t.sn;
-            store4<ROWS>(u, t, off, l, vec, accumulate ? load4<ROWS>(u, t, off, l, vec) + x : x);
-        };
-        if (a.q == 2) {
-            float4 ce[4], co[4], se[4], so[4];
+        // mix: V(o) <- ak sum_i V(i) R(i, o); OGP lanes (a power of two) share 4 lines
+        const int OG = (W + 3) >> 2, ogs = OG > 4 ? 3 : (OG > 2 ? 2 : (OG > 1 ? 1 : 0)), units = (a.m * TQ) << ogs;
+        for (int i0 = 0; i0 < units; i0 += TPB) {
+            const int idx = i0 + tid, r = idx >> ogs;
+            const int og = idx & ((1 << ogs) - 1);
+            const bool on = idx < units && og < OG;
+            const int l = (r & (TQ - 1)) << 2, k = on ? r >> tqs : 0;
+            const float4 *rp = reinterpret_cast<const float4 *>(R + (int64_t)k * W * OG * 4 + og * 4);
+            float *vr = Vre + k * a.KS + l, *vi = Vim + k * a.KS + l;
+            float4 gr[4], gi[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) ce[j] = co[j] = se[j] = so[j] = f4(0.f);
-            for (int kk = 0; kk < a.mk; ++kk) {
-                const int k0 = 2 * kk, k1 = min(2 * kk + 1, a.m - 1);       // past the end: zero tables
-                const float4 x0 = *reinterpret_cast<const float4 *>(gr + k0 * a.KS);
-                const float4 y0 = *reinterpret_cast<const float4 *>(gi + k0 * a.KS);
-                const float4 x1 = *reinterpret_cast<const float4 *>(gr + k1 * a.KS);
-                const float4 y1 = *reinterpret_cast<const float4 *>(gi + k1 * a.KS);
-                const float4 c0 = __ldg(ct + kk * a.NG), s0 = __ldg(st + kk * a.NG);
-                const float4 c1 = __ldg(ct + (a.mk + kk) * a.NG), s1 = __ldg(st + (a.mk + kk) * a.NG);
-                fma4(ce[0], c0.x, x0);
-                fma4(ce[1], c0.y, x0);
-                fma4(ce[2], c0.z, x0);
-                fma4(ce[3], c0.w, x0);
-                fma4(se[0], s0.x, y0);
-                fma4(se[1], s0.y, y0);
-                fma4(se[2], s0.z, y0);
-                fma4(se[3], s0.w, y0);
-                fma4(co[0], c1.x, x1);
-                fma4(co[1], c1.y, x1);
-                fma4(co[2], c1.z, x1);
-                fma4(co[3], c1.w, x1);
-                fma4(so[0], s1.x, y1);
-                fma4(so[1], s1.y, y1);
-                fma4(so[2], s1.z, y1);
-                fma4(so[3], s1.w, y1);
-            }
+            for (int o = 0; o < 4; ++o) gr[o] = gi[o] = f4(0.f);
+            if (on) {
+                if (WC) {
+                    float4 b[3][2][2];              // two inputs' weights per step, two steps ahead
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int n = ng + j * a.NG;
-                if (n >= nq) break;
-                const float4 p = ce[j] + co[j], m = ce[j] - co[j], s = se[j] + so[j], d = se[j] - so[j];
-                put(n, p - s);
-                if (n == 0) {
-                    put(L / 2, m);
+                    for (int st = 0; st < 2; ++st)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            b[st][h][0] = __ldg(rp + (2 * st + h) * OG * 2);
+                            b[st][h][1] = __ldg(rp + (2 * st + h) * OG * 2 + 1);
+                        }
+#pragma unroll
+                    for (int st = 0; st < WC / 2; ++st) {
+                        if (st + 2 < WC / 2)
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                b[(st + 2) % 3][h][0] = __ldg(rp + (2 * st + 4 + h) * OG * 2);
+                                b[(st + 2) % 3][h][1] = __ldg(rp + (2 * st + 4 + h) * OG * 2 + 1);
+                            }
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            mix4(gr, gi, b[st % 3][h], *reinterpret_cast<const float4 *>(vr + (2 * st + h) * T),
+                                 *reinterpret_cast<const float4 *>(vi + (2 * st + h) * T));
+                    }
                 } else {
-                    put(L - n, p + s);
-                    if (4 * n != L) {
+#pragma unroll 4
+                    for (int i = 0; i < W; ++i) {
+                        const float4 c[2] = {__ldg(rp + i * OG * 2), __ldg(rp + i * OG * 2 + 1)};
+                        mix4(gr, gi, c, *reinterpret_cast<const float4 *>(vr + i * T),
+                             *reinterpret_cast<const float4 *>(vi + i * T));
+                    }
+                }
+            }
+            __syncwarp();
+            if (on) {
+                const float sc = ak ? ak[k] : 1.f;
+#pragma unroll
+                for (int o = 0; o < 4; ++o) {
+                    if (4 * og + o >= W) break;
+                    *reinterpret_cast<float4 *>(vr + (4 * og + o) * T) = mul4(sc, gr[o]);
+                    *reinterpret_cast<float4 *>(vi + (4 * og + o) * T) = mul4(sc, gi[o]);
+                }
+            }
+        }
+        __syncthreads();
+
+        // inverse: u(n) = sum_k (Gre cos - Gim sin)
+        for (int idx = tid; idx < W * TQ * a.NG; idx += TPB) {
+            const int r = fdiv(idx, a.dNG), ng = idx - r * a.NG;
+            const int l = (r & (TQ - 1)) << 2, c = r >> tqs;
+            const float *gr = Vre + c * T + l, *gi = Vim + c * T + l;
+            const float4 *ct = a.cinv + ng, *st = a.sinv + ng;
+            const int64_t p0 = t.base + (int64_t)c * N + (int64_t)l * t.sl;
+            auto put = [&](int n, const float4 &x) {
+                store4<ROWS>(u, t, p0 + (int64_t)n * t.sn, l, vec, accumulate != 0, x);
+            };
+            if (a.q == 2) {
+                float4 ce[4], co[4], se[4], so[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) ce[j] = co[j] = se[j] = so[j] = f4(0.f);
+#pragma unroll 2
+                for (int kk = 0; kk < a.mk; ++kk) {
+                    const int k0 = 2 * kk, k1 = min(2 * kk + 1, a.m - 1);       // past the end: zero tables
+                    const float4 x0 = *reinterpret_cast<const float4 *>(gr + k0 * a.KS);
+                    const float4 y0 = *reinterpret_cast<const float4 *>(gi + k0 * a.KS);
+                    const float4 x1 = *reinterpret_cast<const float4 *>(gr + k1 * a.KS);
+                    const float4 y1 = *reinterpret_cast<const float4 *>(gi + k1 * a.KS);
+                    const float4 c0 = __ldg(ct + kk * a.NG), s0 = __ldg(st + kk * a.NG);
+                    const float4 c1 = __ldg(ct + (a.mk + kk) * a.NG), s1 = __ldg(st + (a.mk + kk) * a.NG);
+                    fma4(ce[0], c0.x, x0);
+                    fma4(ce[1], c0.y, x0);
+                    fma4(ce[2], c0.z, x0);
+                    fma4(ce[3], c0.w, x0);
+                    fma4(se[0], s0.x, y0);
+                    fma4(se[1], s0.y, y0);
+                    fma4(se[2], s0.z, y0);
+                    fma4(se[3], s0.w, y0);
+                    fma4(co[0], c1.x, x1);
+                    fma4(co[1], c1.y, x1);
+                    fma4(co[2], c1.z, x1);
+                    fma4(co[3], c1.w, x1);
+                    fma4(so[0], s1.x, y1);
+                    fma4(so[1], s1.y, y1);
+                    fma4(so[2], s1.z, y1);
+                    fma4(so[3], s1.w, y1);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int n = ng + j * a.NG;
+                    if (4 * n >= L) break;
+                    const float4 p = ce[j] + co[j], m = ce[j] - co[j], s = se[j] + so[j], d = se[j] - so[j];
+                    put(n, p - s);
+                    if (n == 0) {
+                        put(L / 2, m);
+                    } else {
+                        put(L - n, p + s);
                         put(L / 2 - n, m + d);
                         put(L / 2 + n, m - d);
                     }
                 }
-            }
-        } else {
-            float4 ce[4], se[4];
+            } else {
+                float4 ce[4], se[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) ce[j] = se[j] = f4(0.f);
-            for (int kk = 0; kk < a.mk; ++kk) {
-                const float4 x = *reinterpret_cast<const float4 *>(gr + kk * a.KS);
-                const float4 y = *reinterpret_cast<const float4 *>(gi + kk * a.KS);
-                const float4 c0 = __ldg(ct + kk * a.NG), s0 = __ldg(st + kk * a.NG);
-                fma4(ce[0], c0.x, x);
-                fma4(ce[1], c0.y, x);
-                fma4(ce[2], c0.z, x);
-                fma4(ce[3], c0.w, x);
-                fma4(se[0], s0.x, y);
-                fma4(se[1], s0.y, y);
-                fma4(se[2], s0.z, y);
-                fma4(se[3], s0.w, y);
-            }
+                for (int j = 0; j < 4; ++j) ce[j] = se[j] = f4(0.f);
+                for (int kk = 0; kk < a.mk; ++kk) {
+                    const float4 x = *reinterpret_cast<const float4 *>(gr + kk * a.KS);
+                    const float4 y = *reinterpret_cast<const float4 *>(gi + kk * a.KS);
+                    const float4 c0 = __ldg(ct + kk * a.NG), s0 = __ldg(st + kk * a.NG);
+                    fma4(ce[0], c0.x, x);
+                    fma4(ce[1], c0.y, x);
+                    fma4(ce[2], c0.z, x);
+                    fma4(ce[3], c0.w, x);
+                    fma4(se[0], s0.x, y);
+                    fma4(se[1], s0.y, y);
+                    fma4(se[2], s0.z, y);
+                    fma4(se[3], s0.w, y);
+                }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int n = ng + j * a.NG;
-                if (n >= nq) break;
-                put(n, ce[j] - se[j]);
-                if (n > 0 && 2 * n != L) put(L - n, ce[j] + se[j]);
+                for (int j = 0; j < 4; ++j) {
+                    const int n = ng + j * a.NG;
+                    if (n >= nq) break;
+                    put(n, ce[j] - se[j]);
+                    if (n > 0 && 2 * n != L) put(L - n, ce[j] + se[j]);
+                }
             }
         }
+        // the self-symmetric term n = L/4 (its cosines and sines are 0, 1, -1),
+        // one thread per channel and 4 lines
+        if (a.q == 2)
+            for (int idx = TPB - 1 - tid; idx < W * TQ; idx += TPB) {
+                const int l = (idx & (TQ - 1)) << 2, c = idx >> tqs;
+                const float *gr = Vre + c * T + l, *gi = Vim + c * T + l;
+                float4 p = f4(0.f), s = f4(0.f);
+                for (int k = 0; k < a.m; k += 4) {
+                    p = p + *reinterpret_cast<const float4 *>(gr + k * a.KS);
+                    if (k + 2 < a.m) p = p - *reinterpret_cast<const float4 *>(gr + (k + 2) * a.KS);
+                    if (k + 1 < a.m) s = s + *reinterpret_cast<const float4 *>(gi + (k + 1) * a.KS);
+                    if (k + 3 < a.m) s = s - *reinterpret_cast<const float4 *>(gi + (k + 3) * a.KS);
+                }
+                const int64_t p0 = t.base + (int64_t)c * N + (int64_t)l * t.sl;
+                store4<ROWS>(u, t, p0 + (int64_t)(L / 4) * t.sn, l, vec, accumulate != 0, p - s);
+                store4<ROWS>(u, t, p0 + (int64_t)(L - L / 4) * t.sn, l, vec, accumulate != 0, p + s);
+            }
     }
 }
 
@@ -530,30 +635,49 @@ template <int V> struct Vec;
 template <> struct Vec<1> { using T = float; };
 template <> struct Vec<2> { using T = float2; };
 
+constexpr int MT = 128;                      // threads of the forward kernel
+
 // A thread's V cells keep their CI inputs and CO outputs in registers; the
 // weights are broadcast from shared memory, so the kernel is bound by the
-// multiply-adds and the activation.
+// multiply-adds and the activation.  Each thread copies its next cells' inputs
+// into its own places of shared memory while it computes (no barrier: nobody
+// else reads them), which 12 warps per SM would not hide otherwise.
 template <int CI, int CO, int ACT, int V>
-__global__ void __launch_bounds__(TPB) k_mlp(const Mlp p, const float *__restrict__ x, const float *res, float *y,
-                                             int B, int64_t N)
+__global__ void __launch_bounds__(MT, 3) k_mlp(const Mlp p, const float *__restrict__ x, const float *res, float *y,
+                                               int B, int64_t N)
 {
     extern __shared__ float4 raw[];
+    using T = typename Vec<V>::T;
     const int chp = (p.ch + 1) & ~1;
     float *w1 = reinterpret_cast<float *>(raw), *w2 = w1 + chp * CI, *b1 = w2 + chp * CO, *b2 = b1 + ((chp + 3) & ~3);
+    T *next = reinterpret_cast<T *>(b2 + CO) + threadIdx.x;
     stage_weights<CI, CO>(p, chp, w1, w2, b1, b2);
     __syncthreads();
-    using T = typename Vec<V>::T;
-    const int64_t items = B * N / V;
-    for (int64_t it = (int64_t)blockIdx.x * TPB + threadIdx.x; it < items; it += (int64_t)gridDim.x * TPB) {
+    const int64_t items = B * N / V, step = (int64_t)gridDim.x * MT;
+    auto fetch = [&](int64_t it) {
+        if (it >= items) return;
+        const int64_t cell = it * V, b = cell / N, n = cell - b * N;
+        const float *src = x + b * p.ci * N + n;
+#pragma unroll 8
+        for (int c = 0; c < p.ci; ++c, src += N) {
+            if (V == 2) async8(next + c * MT, src);
+            else async4(next + c * MT, src);
+        }
+    };
+    int64_t it = (int64_t)blockIdx.x * MT + threadIdx.x;
+    fetch(it);
+    for (; it < items; it += step) {
         const int64_t cell = it * V, b = cell / N, n = cell - b * N;
         float in[CI][V], out[CO][V];
+        async_wait();
 #pragma unroll
         for (int c = 0; c < CI; ++c) {
-            if (c < p.ci) *reinterpret_cast<T *>(in[c]) = *reinterpret_cast<const T *>(x + (b * p.ci + c) * N + n);
+            if (c < p.ci) *reinterpret_cast<T *>(in[c]) = next[c * MT];
             else
 #pragma unroll
                 for (int q = 0; q < V; ++q) in[c][q] = 0.f;
         }
+        fetch(it + step);
 #pragma unroll
         for (int o = 0; o < CO; ++o)
 #pragma unroll
@@ -597,18 +721,25 @@ __global__ void __launch_bounds__(TPB) k_mlp(const Mlp p, const float *__restric
                     }
                 }
         }
+        float *dst = y + b * p.co * N + n;
+        if (res) {                               // `in` is free: sixteen residuals in flight at once
+            const float *r = res + b * p.co * N + n;
 #pragma unroll
-        for (int o = 0; o < CO; ++o) {
-            if (o >= p.co) break;
-            const int64_t at = (b * p.co + o) * N + n;
-            if (res) {
-                float r[V];
-                *reinterpret_cast<T *>(r) = *reinterpret_cast<const T *>(res + at);
+            for (int o = 0; o < CO; o += 16) {
+                float v[16][V];
 #pragma unroll
-                for (int q = 0; q < V; ++q) out[o][q] += r[q];
+                for (int k = 0; k < 16 && o + k < CO; ++k, r += N)
+                    if (o + k < p.co) *reinterpret_cast<T *>(v[k]) = *reinterpret_cast<const T *>(r);
+#pragma unroll
+                for (int k = 0; k < 16 && o + k < CO; ++k)
+                    if (o + k < p.co)
+#pragma unroll
+                        for (int q = 0; q < V; ++q) out[o + k][q] += v[k][q];
             }
-            *reinterpret_cast<T *>(y + at) = *reinterpret_cast<const T *>(out[o]);
         }
+#pragma unroll
+        for (int o = 0; o < CO; ++o, dst += N)
+            if (o < p.co) *reinterpret_cast<T *>(dst) = *reinterpret_cast<const T *>(out[o]);
     }
 }
 
@@ -820,15 +951,19 @@ bool axis_plan(Axis &a, int L, int m, int rows, int64_t S, int64_t outer, int W)
     a.nq = a.q == 2 ? L / 4 + 1 : L / 2 + 1;
     a.mk = (m + a.q - 1) / a.q;
     a.KG = (a.mk + 3) / 4;
-    a.NG = (a.nq + 3) / 4;
+    a.NG = a.q == 2 ? (L / 4 + 3) / 4 : (a.nq + 3) / 4;
+    auto recip = [](int d) { return d > 1 ? (uint32_t)((((uint64_t)1 << 32) + d - 1) / d) : 0u; };
+    a.dnq = recip(a.nq);
+    a.dKG = recip(a.KG);
+    a.dNG = recip(a.NG);
     for (int T = 16; T >= 4; T /= 2) {
         a.T = T;
         a.DS = stride_for(2 * a.q * a.nq * T, T);
         a.KS = stride_for(W * T, 4);
-        a.smem = sizeof(float) * ((size_t)std::max(W * a.DS, 2 * m * a.KS) + (size_t)2 * m * a.KS);
+        a.smem = sizeof(float) * ((size_t)W * a.DS + (size_t)2 * m * a.KS);
         if (a.smem <= SMEM_TWO) return true;
     }
-    return a.smem <= SMEM_MAX;
+    return a.smem <= SMEM_MAX && (int64_t)W * a.nq * 4 < 65536;
 }
 
 void axis_tables(const Axis &a, std::vector<float> &out, size_t count[4])
@@ -864,11 +999,11 @@ void spectral(const Axis &a, const float *v, float *u, int B, int W, int64_t N, 
 {
     const int64_t run = a.rows ? a.outer : a.S;
     const int tiles = (int)((run + a.T - 1) / a.T);
-    const int64_t blocks = (int64_t)B * tiles * (a.rows ? 1 : a.outer), NL = B * a.lines();
-    if (a.rows)
-        k_spectral<1><<<(unsigned)blocks, TPB, a.smem, s>>>(a, v, u, W, N, R, wk, ak, spec, NL, tiles, accumulate);
-    else
-        k_spectral<0><<<(unsigned)blocks, TPB, a.smem, s>>>(a, v, u, W, N, R, wk, ak, spec, NL, tiles, accumulate);
+    const int64_t total = (int64_t)B * tiles * (a.rows ? 1 : a.outer), NL = B * a.lines();
+    const int grid = (int)std::min<int64_t>(total, (int64_t)gb300::sm_count() * (a.smem <= SMEM_TWO ? 2 : 1));
+    auto k = a.rows ? (W == MAXW ? k_spectral<1, MAXW> : k_spectral<1, 0>)
+                    : (W == MAXW ? k_spectral<0, MAXW> : k_spectral<0, 0>);
+    k<<<grid, TPB, a.smem, s>>>(a, v, u, W, N, R, wk, ak, spec, NL, tiles, (int)total, accumulate);
 }
 
 void pack_r(const PackR &p, int W, cudaStream_t s)
@@ -898,13 +1033,13 @@ template <int CI, int CO, int ACT>
 void mlp_v(const Mlp &p, const float *x, const float *res, float *y, int B, int64_t N, cudaStream_t s)
 {
     const int chp = (p.ch + 1) & ~1;
-    const size_t smem = sizeof(float) * (size_t)(chp * (CI + CO) + round4(chp) + CO);
+    const size_t smem = sizeof(float) * (size_t)(chp * (CI + CO) + round4(chp) + CO + 2 * CI * MT);
     const uintptr_t al = (uintptr_t)x | (uintptr_t)res | (uintptr_t)y;
     const bool two = N % 2 == 0 && (al & 7) == 0;
     const int64_t items = B * N / (two ? 2 : 1);
-    const int grid = (int)std::min<int64_t>((items + TPB - 1) / TPB, (int64_t)gb300::sm_count() * 2);
-    if (two) k_mlp<CI, CO, ACT, 2><<<grid, TPB, smem, s>>>(p, x, res, y, B, N);
-    else k_mlp<CI, CO, ACT, 1><<<grid, TPB, smem, s>>>(p, x, res, y, B, N);
+    const int grid = (int)std::min<int64_t>((items + MT - 1) / MT, (int64_t)gb300::sm_count() * 3);
+    if (two) k_mlp<CI, CO, ACT, 2><<<grid, MT, smem, s>>>(p, x, res, y, B, N);
+    else k_mlp<CI, CO, ACT, 1><<<grid, MT, smem, s>>>(p, x, res, y, B, N);
 }
 
 template <int ACT>
@@ -957,10 +1092,17 @@ bool big_bwd()
            big(k_mlp_bwd<CI, CO, ACT, 4, GX>, bwd_smem<CI, CO, ACT, 4, GX>());
 }
 
+template <int CI, int CO, int ACT>
+bool big_mlp()
+{
+    constexpr size_t most = sizeof(float) * (size_t)(128 * (CI + CO + 1) + CO + 2 * CI * MT);
+    return big(k_mlp<CI, CO, ACT, 1>, most) && big(k_mlp<CI, CO, ACT, 2>, most);
+}
+
 template <int ACT>
 bool big_act()
 {
-    return big_bwd<8, 32, ACT, false>() && big_bwd<32, 32, ACT, false>() && big_bwd<32, 8, ACT, true>() &&
+    return big_mlp<8, 32, ACT>() && big_mlp<32, 8, ACT>() && big_mlp<32, 32, ACT>() && big_bwd<8, 32, ACT, false>() && big_bwd<32, 32, ACT, false>() && big_bwd<32, 8, ACT, true>() &&
            big_bwd<32, 32, ACT, true>();
 }
 
@@ -986,7 +1128,8 @@ void mlp_bwd(const Mlp &p, const float *x, const float *g, float *gx, float *par
 // The dynamic shared-memory limits are per device: set on every creation.
 bool set_attrs()
 {
-    return big(k_spectral<0>, SMEM_MAX) && big(k_spectral<1>, SMEM_MAX) && big_act<ACT_GELU>() && big_act<ACT_SIREN>();
+    return big(k_spectral<0, 0>, SMEM_MAX) && big(k_spectral<1, 0>, SMEM_MAX) &&
+           big(k_spectral<0, MAXW>, SMEM_MAX) && big(k_spectral<1, MAXW>, SMEM_MAX) && big_act<ACT_GELU>() && big_act<ACT_SIREN>();
 }
 
 }  // namespace ffno

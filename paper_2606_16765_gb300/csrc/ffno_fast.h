@@ -24,6 +24,7 @@ struct Axis {
     int T;                               // lines per block
     int q, nq;                           // parities, terms per folded sum
     int mk, KG, NG;                      // wave numbers per parity, groups of 4 of them, groups of 4 terms
+    uint32_t dnq, dKG, dNG;              // reciprocals of nq, KG, NG
     int DS, KS;                          // shared-memory strides: folded channel, wave number
     size_t smem;
     const float4 *ctab, *stab;           // [q][nq][KG] cos, sin of 4 wave numbers
