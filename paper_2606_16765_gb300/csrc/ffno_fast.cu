@@ -9,6 +9,7 @@
 //                accumulated per block and summed in a fixed order
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "ffno_fast.h"
 #include "sm_count.h"
@@ -116,6 +117,72 @@ __device__ __forceinline__ void mix4(float4 *gr, float4 *gi, const float4 *w, co
     }
 }
 
+// Channel mixing of a tile in place: V [k][c][T], V(o) <- ak sum_i V(i) R(i, o).
+// Thread = 4 lines x 4 outputs (complex), 64 multiply-adds per two operands
+// from shared memory and two from L2 (read two steps ahead); the lanes of one
+// wave number and 4 lines (a power of two of them) sit in one warp, read all
+// inputs, then write.  WC: the width when it is a constant, else 0.
+template <int WC>
+__device__ __forceinline__ void mix_phase(float *Vre, float *Vim, int m, int KS, int T, int W,
+                                          const float2 *__restrict__ R, const float *__restrict__ ak)
+{
+    const int TQ = T >> 2, tqs = TQ == 1 ? 0 : (TQ == 2 ? 1 : 2);
+    const int OG = (W + 3) >> 2, ogs = OG > 4 ? 3 : (OG > 2 ? 2 : (OG > 1 ? 1 : 0)), units = (m * TQ) << ogs;
+    for (int i0 = 0; i0 < units; i0 += TPB) {
+        const int idx = i0 + (int)threadIdx.x, r = idx >> ogs;
+        const int og = idx & ((1 << ogs) - 1);
+        const bool on = idx < units && og < OG;
+        const int l = (r & (TQ - 1)) << 2, k = on ? r >> tqs : 0;
+        const float4 *rp = reinterpret_cast<const float4 *>(R + (int64_t)k * W * OG * 4) + og;
+        float *vr = Vre + k * KS + l, *vi = Vim + k * KS + l;
+        float4 gr[4], gi[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) gr[o] = gi[o] = f4(0.f);
+        if (on) {
+            if (WC) {
+                float4 b[3][2][2];              // two inputs' weights per step, two steps ahead
+#pragma unroll
+                for (int st = 0; st < 2; ++st)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        b[st][h][0] = __ldg(rp + (2 * st + h) * OG * 2);
+                        b[st][h][1] = __ldg(rp + (2 * st + h) * OG * 2 + OG);
+                    }
+#pragma unroll
+                for (int st = 0; st < WC / 2; ++st) {
+                    if (st + 2 < WC / 2)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            b[(st + 2) % 3][h][0] = __ldg(rp + (2 * st + 4 + h) * OG * 2);
+                            b[(st + 2) % 3][h][1] = __ldg(rp + (2 * st + 4 + h) * OG * 2 + OG);
+                        }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        mix4(gr, gi, b[st % 3][h], *reinterpret_cast<const float4 *>(vr + (2 * st + h) * T),
+                             *reinterpret_cast<const float4 *>(vi + (2 * st + h) * T));
+                }
+            } else {
+#pragma unroll 4
+                for (int i = 0; i < W; ++i) {
+                    const float4 c[2] = {__ldg(rp + i * OG * 2), __ldg(rp + i * OG * 2 + OG)};
+                    mix4(gr, gi, c, *reinterpret_cast<const float4 *>(vr + i * T),
+                         *reinterpret_cast<const float4 *>(vi + i * T));
+                }
+            }
+        }
+        __syncwarp();
+        if (on) {
+            const float sc = ak ? ak[k] : 1.f;
+#pragma unroll
+            for (int o = 0; o < 4; ++o) {
+                if (4 * og + o >= W) break;
+                *reinterpret_cast<float4 *>(vr + (4 * og + o) * T) = mul4(sc, gr[o]);
+                *reinterpret_cast<float4 *>(vi + (4 * og + o) * T) = mul4(sc, gi[o]);
+            }
+        }
+    }
+}
+
 // A persistent block over tiles of T lines x W channels x L samples.  Phases,
 // a barrier between them:
 //   fold     D [c][class][n][T]: even and odd parts of the lines, split by the
@@ -123,9 +190,7 @@ __device__ __forceinline__ void mix4(float4 *gr, float4 *gi, const float4 *w, co
 //            what it copied itself
 //   forward  V [k][c][T]: thread = 4 wave numbers x 4 lines, real and
 //            imaginary part: 32 multiply-adds per four 16-byte operands
-//   mix      in place on V: thread = 4 lines x 4 outputs (complex); the
-//            threads of one wave number and 4 lines sit in one warp, read all
-//            inputs, then write; the weights come from L2, two steps ahead
+//   mix      in place on V
 //   inverse  thread = 4 terms x 4 lines of all four symmetric sums, unfolded
 //            into 16 samples and stored
 // D is free after the forward phase: the next tile's copies are issued there
@@ -298,61 +363,7 @@ __global__ void __launch_bounds__(TPB, 2) k_spectral(const Axis a, const float *
             fetch(tn);
         }
 
-        // mix: V(o) <- ak sum_i V(i) R(i, o); OGP lanes (a power of two) share 4 lines
-        const int OG = (W + 3) >> 2, ogs = OG > 4 ? 3 : (OG > 2 ? 2 : (OG > 1 ? 1 : 0)), units = (a.m * TQ) << ogs;
-        for (int i0 = 0; i0 < units; i0 += TPB) {
-            const int idx = i0 + tid, r = idx >> ogs;
-            const int og = idx & ((1 << ogs) - 1);
-            const bool on = idx < units && og < OG;
-            const int l = (r & (TQ - 1)) << 2, k = on ? r >> tqs : 0;
-            const float4 *rp = reinterpret_cast<const float4 *>(R + (int64_t)k * W * OG * 4 + og * 4);
-            float *vr = Vre + k * a.KS + l, *vi = Vim + k * a.KS + l;
-            float4 gr[4], gi[4];
-#pragma unroll
-            for (int o = 0; o < 4; ++o) gr[o] = gi[o] = f4(0.f);
-            if (on) {
-                if (WC) {
-                    float4 b[3][2][2];              // two inputs' weights per step, two steps ahead
-#pragma unroll
-                    for (int st = 0; st < 2; ++st)
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            b[st][h][0] = __ldg(rp + (2 * st + h) * OG * 2);
-                            b[st][h][1] = __ldg(rp + (2 * st + h) * OG * 2 + 1);
-                        }
-#pragma unroll
-                    for (int st = 0; st < WC / 2; ++st) {
-                        if (st + 2 < WC / 2)
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                b[(st + 2) % 3][h][0] = __ldg(rp + (2 * st + 4 + h) * OG * 2);
-                                b[(st + 2) % 3][h][1] = __ldg(rp + (2 * st + 4 + h) * OG * 2 + 1);
-                            }
-#pragma unroll
-                        for (int h = 0; h < 2; ++h)
-                            mix4(gr, gi, b[st % 3][h], *reinterpret_cast<const float4 *>(vr + (2 * st + h) * T),
-                                 *reinterpret_cast<const float4 *>(vi + (2 * st + h) * T));
-                    }
-                } else {
-#pragma unroll 4
-                    for (int i = 0; i < W; ++i) {
-                        const float4 c[2] = {__ldg(rp + i * OG * 2), __ldg(rp + i * OG * 2 + 1)};
-                        mix4(gr, gi, c, *reinterpret_cast<const float4 *>(vr + i * T),
-                             *reinterpret_cast<const float4 *>(vi + i * T));
-                    }
-                }
-            }
-            __syncwarp();
-            if (on) {
-                const float sc = ak ? ak[k] : 1.f;
-#pragma unroll
-                for (int o = 0; o < 4; ++o) {
-                    if (4 * og + o >= W) break;
-                    *reinterpret_cast<float4 *>(vr + (4 * og + o) * T) = mul4(sc, gr[o]);
-                    *reinterpret_cast<float4 *>(vi + (4 * og + o) * T) = mul4(sc, gi[o]);
-                }
-            }
-        }
+        mix_phase<WC>(Vre, Vim, a.m, a.KS, T, W, R, ak);
         __syncthreads();
 
         // inverse: u(n) = sum_k (Gre cos - Gim sin)
@@ -455,14 +466,330 @@ __global__ void __launch_bounds__(TPB, 2) k_spectral(const Axis a, const float *
     }
 }
 
-// R [i][o][m] -> rf [m][i][Wp] and the conjugate transpose ra [m][o][Wp]
+// ---------------------------------------------------------------------------
+// the same for the usual lengths, with the transform in registers
+// ---------------------------------------------------------------------------
+// cos(2 pi j / n) and sin(2 pi j / n) from their Taylor series at the argument
+// reduced to [0, pi/4] (double; 20 terms leave less than 1e-20)
+constexpr double taylor(double x, bool sine)
+{
+    double t = sine ? x : 1.0, s = t;
+    for (int k = sine ? 2 : 1; k < 40; k += 2) {
+        t *= -x * x / (k * (k + 1.0));
+        s += t;
+    }
+    return s;
+}
+constexpr double sincos_of(int j, int n, bool sine)
+{
+    j %= n;
+    if (sine) return 2 * j > n ? -sincos_of(n - j, n, true)
+                   : 4 * j > n ? (8 * j > 3 * n ? taylor(2 * M_PI * (n - 2 * j) / (2.0 * n), true)
+                                                : taylor(2 * M_PI * (4 * j - n) / (4.0 * n), false))
+                   : 8 * j > n ? taylor(2 * M_PI * (n - 4 * j) / (4.0 * n), false)
+                               : taylor(2 * M_PI * j / n, true);
+    return 2 * j > n ? sincos_of(n - j, n, false)
+         : 4 * j > n ? -(8 * j > 3 * n ? taylor(2 * M_PI * (n - 2 * j) / (2.0 * n), false)
+                                       : taylor(2 * M_PI * (4 * j - n) / (4.0 * n), true))
+         : 8 * j > n ? taylor(2 * M_PI * (n - 4 * j) / (4.0 * n), true)
+                     : taylor(2 * M_PI * j / n, false);
+}
+
+template <int A, int B, int STEP = 1, class F>
+__device__ __forceinline__ void each(const F &f)
+{
+    if constexpr (A < B) {
+        f(std::integral_constant<int, A>());
+        each<A + STEP, B, STEP>(f);
+    }
+}
+
+// s += c x with the constant c (nothing where it is 0)
+template <int J, int N, bool SINE>
+__device__ __forceinline__ void cfma(float &s, float x)
+{
+    constexpr double d = sincos_of(J, N, SINE);
+    constexpr float c = d < 1e-12 && d > -1e-12 ? 0.f : (float)d;
+    if constexpr (c == 1.f) s += x;
+    else if constexpr (c == -1.f) s -= x;
+    else if constexpr (c != 0.f) s = fmaf(c, x, s);
+}
+
+// The wave numbers of parity PAR (-1: all) below M of one line whose folded
+// samples are E0, E1 (even parts), O0, O1 (odd parts): st(k, re, im).
+template <int L, int M, int PAR, class F>
+__device__ __forceinline__ void forward_line(const float *E, const float *O, const F &st)
+{
+    each<0, M>([&](auto kc) {
+        constexpr int k = kc;
+        if constexpr (PAR < 0 || (k & 1) == PAR) {
+            constexpr int Q = L / 4 + 1, off = PAR < 0 ? (k & 1) * Q : 0;
+            float re = 0.f, im = 0.f;
+            each<0, Q>([&](auto nc) {
+                constexpr int n = nc;
+                cfma<(k * n) % L, L, false>(re, E[off + n]);
+                cfma<(k * n) % L, L, true>(im, O[off + n]);
+            });
+            st(kc, re, im);
+        }
+    });
+}
+
+// The samples n, L - n, L/2 - n, L/2 + n of one line for FIRST <= n < LAST
+// (n <= L/4) from its wave numbers: put(index, value), in this order.
+template <int L, int M, int FIRST, int LAST, class F>
+__device__ __forceinline__ void inverse_line(const float *re, const float *im, const F &put)
+{
+    each<FIRST, LAST>([&](auto nc) {
+        constexpr int n = nc;
+        float ce = 0.f, co = 0.f, se = 0.f, so = 0.f;
+        each<0, M>([&](auto kc) {
+            constexpr int k = kc;
+            if constexpr (k & 1) {
+                cfma<(k * n) % L, L, false>(co, re[k]);
+                cfma<(k * n) % L, L, true>(so, im[k]);
+            } else {
+                cfma<(k * n) % L, L, false>(ce, re[k]);
+                cfma<(k * n) % L, L, true>(se, im[k]);
+            }
+        });
+        const float p = ce + co, s = se + so;
+        put(nc, p - s);
+        if constexpr (n > 0) put(std::integral_constant<int, L - n>(), p + s);
+        if constexpr (n == 0) put(std::integral_constant<int, L / 2>(), ce - co);
+        if constexpr (n > 0 && 4 * n != L) {
+            const float m = ce - co, d = se - so;
+            put(std::integral_constant<int, L / 2 - n>(), m + d);
+            put(std::integral_constant<int, L / 2 + n>(), m - d);
+        }
+    });
+}
+
+__device__ __forceinline__ void put1(float *p, float v, bool add)
+{
+    if (add) atomicAdd(p, v);
+    else *p = v;
+}
+
+__device__ __forceinline__ void put4(float *p, const float4 &v, bool add)
+{
+    if (add) atomicAdd(reinterpret_cast<float4 *>(p), v);
+    else *reinterpret_cast<float4 *>(p) = v;
+}
+
+// One thread per line (c, t), its samples in registers: the transforms'
+// cosines are immediate operands, so they take one instruction per
+// multiply-add and shared memory carries the samples and spectra once (the
+// tabulated kernel above is bound by shared-memory reads: 32 multiply-adds per
+// four 16-byte operands).  The next tile's samples are copied behind the
+// mixing and the inverse.
+//   ROWS = 0 (samples S apart): X [c][n][8 lines]; stores run along the lines
+//   ROWS = 1 (contiguous samples): X [c, row][L + 4], read 16 bytes at a time;
+//     a line is shared by two threads (wave numbers of even and odd parity;
+//     the lower and the upper half of the terms back, 16 bytes per store)
+template <int L, int M, int ROWS>
+__global__ void __launch_bounds__(TPB, 2) k_spectral_reg(const Axis a, const float *__restrict__ v, float *u, int W,
+                                                         int64_t N, const float2 *__restrict__ R,
+                                                         const float *__restrict__ wk, const float *__restrict__ ak,
+                                                         float *__restrict__ spec, int64_t NL, int tiles, int total,
+                                                         int accumulate)
+{
+    extern __shared__ float4 raw[];
+    constexpr int T = ROWS ? 4 : 8, TS = ROWS ? 2 : 3, P = L + 4, CS = L * T + 8, Q = L / 4 + 1, H = L / 8;
+    const int tid = threadIdx.x;
+    float *X = reinterpret_cast<float *>(raw), *Vre = X + W * (ROWS ? T * P : CS), *Vim = Vre + a.m * a.KS;
+    const int64_t plane = (int64_t)a.m * W * NL;
+    const bool vec = ROWS || (a.S & 3) == 0, add = accumulate != 0;
+
+    auto lines_of = [&](int w, int64_t &line0) {
+        Tile t;
+        const int64_t ti = w % tiles, ob = w / tiles;
+        if (ROWS) {
+            t.base = ob * W * N + ti * T * L;
+            t.valid = (int)min((int64_t)T, a.outer - ti * T);
+            line0 = ob * a.outer + ti * T;
+        } else {
+            const int64_t o = ob % a.outer, b = ob / a.outer;
+            t.base = b * W * N + o * L * a.S + ti * T;
+            t.valid = (int)min((int64_t)T, a.S - ti * T);
+            line0 = ob * a.S + ti * T;
+        }
+        t.sn = a.S;
+        t.sl = 1;
+        return t;
+    };
+    auto fetch = [&](const Tile &t) {
+        if (ROWS) {                                  // 16 bytes along a row
+            for (int idx = tid; idx < W * T * (L / 4); idx += TPB) {
+                const int x = (idx % (L / 4)) * 4, r = idx / (L / 4);
+                if ((r & (T - 1)) < t.valid)
+                    async16(X + r * P + x, v + t.base + (int64_t)(r >> TS) * N + (r & (T - 1)) * L + x);
+            }
+        } else {                                     // 16 bytes along the lines
+            for (int idx = tid; idx < W * L * (T / 4); idx += TPB) {
+                const int l = (idx & (T / 4 - 1)) * 4, r = idx / (T / 4), n = r % L, c = r / L;
+                fetch4<0>(X + c * CS + n * T + l, v, t, t.base + (int64_t)c * N + n * a.S + l, l, vec);
+            }
+        }
+    };
+
+    int64_t line0 = 0, line_next = 0;
+    Tile t = lines_of(blockIdx.x, line0), tn = t;
+    fetch(t);
+    for (int w = blockIdx.x; w < total; w += gridDim.x, t = tn, line0 = line_next) {
+        async_wait();
+        __syncthreads();
+
+        // forward: one line, or one parity of a line, per thread
+        constexpr int SPLIT = ROWS ? 2 : 1;
+        for (int i0 = 0; i0 < W * T * SPLIT; i0 += TPB) {
+            // the parity is uniform over half a block
+            const int par = ROWS ? tid / (TPB / 2) : 0;
+            const int ln = ROWS ? i0 / 2 + tid % (TPB / 2) : i0 + tid;
+            const int c = ln >> TS, l = ln & (T - 1);
+            if (ln >= W * T) continue;
+            const bool ok = l < t.valid;
+            auto out = [&](auto kc, float re, float im) {
+                constexpr int k = kc;
+                if (k < a.m) {
+                    const float sc = wk ? wk[k] : 1.f;
+                    const float x = ok ? sc * re : 0.f, y = ok ? -sc * im : 0.f;
+                    Vre[k * a.KS + ln] = x;
+                    Vim[k * a.KS + ln] = y;
+                    if (spec && ok) {
+                        float *s = spec + ((int64_t)k * W + c) * NL + line0 + l;
+                        s[0] = x;
+                        s[plane] = y;
+                    }
+                }
+            };
+            float x[L];
+            if constexpr (ROWS) {
+                const float4 *src = reinterpret_cast<const float4 *>(X + ln * P);
+#pragma unroll
+                for (int n = 0; n < L / 4; ++n) {
+                    const float4 q = src[n];
+                    x[4 * n] = q.x;
+                    x[4 * n + 1] = q.y;
+                    x[4 * n + 2] = q.z;
+                    x[4 * n + 3] = q.w;
+                }
+                float E[Q], O[Q];
+                const float sg = par ? -1.f : 1.f;
+#pragma unroll
+                for (int n = 0; n < Q; ++n) {
+                    if (n == 0) {
+                        E[0] = fmaf(sg, x[L / 2], x[0]);
+                        O[0] = 0.f;
+                    } else if (4 * n == L) {
+                        E[n] = par ? 0.f : x[n] + x[L - n];
+                        O[n] = par ? x[n] - x[L - n] : 0.f;
+                    } else {
+                        E[n] = fmaf(sg, x[L / 2 - n] + x[L / 2 + n], x[n] + x[L - n]);
+                        O[n] = fmaf(-sg, x[L / 2 - n] - x[L / 2 + n], x[n] - x[L - n]);
+                    }
+                }
+                if (par) forward_line<L, M, 1>(E, O, out);
+                else forward_line<L, M, 0>(E, O, out);
+            } else {
+                float E[2 * Q], O[2 * Q];
+                const float *src = X + c * CS + l;
+#pragma unroll
+                for (int n = 0; n < L; ++n) x[n] = src[n * T];
+#pragma unroll
+                for (int n = 0; n < Q; ++n) {
+                    if (n == 0) {
+                        E[0] = x[0] + x[L / 2];
+                        E[Q] = x[0] - x[L / 2];
+                        O[0] = O[Q] = 0.f;
+                    } else if (4 * n == L) {
+                        E[n] = x[n] + x[L - n];
+                        O[Q + n] = x[n] - x[L - n];
+                        E[Q + n] = O[n] = 0.f;
+                    } else {
+                        const float ea = x[n] + x[L - n], eb = x[L / 2 - n] + x[L / 2 + n];
+                        const float oa = x[n] - x[L - n], ob = x[L / 2 - n] - x[L / 2 + n];
+                        E[n] = ea + eb;
+                        E[Q + n] = ea - eb;
+                        O[n] = oa - ob;
+                        O[Q + n] = oa + ob;
+                    }
+                }
+                forward_line<L, M, -1>(E, O, out);
+            }
+        }
+        __syncthreads();
+        if (w + (int)gridDim.x < total) {
+            tn = lines_of(w + (int)gridDim.x, line_next);
+            fetch(tn);
+        }
+        if (W == MAXW) mix_phase<MAXW>(Vre, Vim, a.m, a.KS, T, W, R, ak);
+        else mix_phase<0>(Vre, Vim, a.m, a.KS, T, W, R, ak);
+        __syncthreads();
+
+        // inverse
+        for (int i0 = 0; i0 < W * T * SPLIT; i0 += TPB) {
+            const int par = ROWS ? tid / (TPB / 2) : 0;
+            const int ln = ROWS ? i0 / 2 + tid % (TPB / 2) : i0 + tid;
+            const int c = ln >> TS, l = ln & (T - 1);
+            if (ln >= W * T || l >= t.valid) continue;
+            float re[M], im[M];
+#pragma unroll
+            for (int k = 0; k < M; ++k) {
+                re[k] = k < a.m ? Vre[k * a.KS + ln] : 0.f;
+                im[k] = k < a.m ? Vim[k * a.KS + ln] : 0.f;
+            }
+            if constexpr (ROWS) {
+                // the terms below L/8 give the samples within L/8 of 0 and L/2,
+                // the others those around L/4 and 3L/4; 16 bytes are stored
+                // once their four samples are there
+                float *dst = u + t.base + (int64_t)c * N + (int64_t)l * L;
+                float x[L];
+                auto run = [&](auto fc, auto lc) {
+                    constexpr int F = fc, E = lc;
+                    inverse_line<L, M, F, E>(re, im, [&](auto nc, float val) {
+                        constexpr int n = nc;
+                        x[n] = val;
+                    });
+                    each<0, L / 4>([&](auto qc) {
+                        constexpr int q = 4 * qc;
+                        // the term that gives sample n: its distance to the nearest multiple of L/2
+                        constexpr auto term = [](int n) { const int r = n % (L / 2); return r > L / 4 ? L / 2 - r : r; };
+                        constexpr bool all = term(q) >= F && term(q) < E && term(q + 1) >= F && term(q + 1) < E &&
+                                             term(q + 2) >= F && term(q + 2) < E && term(q + 3) >= F && term(q + 3) < E;
+                        if constexpr (all) {
+                            put4(dst + q, make_float4(x[q], x[q + 1], x[q + 2], x[q + 3]), add);
+                        } else {
+                            each<0, 4>([&](auto ic) {
+                                constexpr int n = q + ic;
+                                if constexpr (term(n) >= F && term(n) < E) put1(dst + n, x[n], add);
+                            });
+                        }
+                    });
+                };
+                if (par) run(std::integral_constant<int, H>(), std::integral_constant<int, Q>());
+                else run(std::integral_constant<int, 0>(), std::integral_constant<int, H>());
+            } else {
+                float *dst = u + t.base + (int64_t)c * N + l;
+                if (add) inverse_line<L, M, 0, Q>(re, im, [&](auto nc, float val) { constexpr int n = nc; atomicAdd(dst + n * a.S, val); });
+                else inverse_line<L, M, 0, Q>(re, im, [&](auto nc, float val) { constexpr int n = nc; dst[n * a.S] = val; });
+            }
+        }
+    }
+}
+
+// R [i][o][m] -> rf [m][i] and the conjugate transpose ra [m][o], each row of
+// Wp entries in the order the mixing reads them: entries 4g, 4g + 1 of every
+// group g, then entries 4g + 2, 4g + 3 (neighbouring lanes read neighbouring
+// 16 bytes)
 __global__ void k_pack_r(const PackR pr, int W, int Wp)
 {
     const float *R = pr.a[blockIdx.y].R;
     float2 *rf = pr.a[blockIdx.y].rf, *ra = pr.a[blockIdx.y].ra;
     const int m = pr.a[blockIdx.y].m, n = m * W * Wp;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        const int p = t % Wp, r = (t / Wp) % W, k = t / (Wp * W);
+        const int e = t % Wp, r = (t / Wp) % W, k = t / (Wp * W);
+        const int half = e / (Wp / 2), x = e % (Wp / 2), p = (x >> 1) * 4 + half * 2 + (x & 1);
         float2 f = make_float2(0.f, 0.f), g = f;
         if (p < W) {
             const int64_t j = (((int64_t)r * W + p) * m + k) * 2, h = (((int64_t)p * W + r) * m + k) * 2;
@@ -940,6 +1267,30 @@ int stride_for(int v, int rem)
 
 }  // namespace
 
+namespace {
+
+typedef void (*SpecKernel)(Axis, const float *, float *, int, int64_t, const float2 *, const float *, const float *,
+                           float *, int64_t, int, int, int);
+
+// the register kernel of a length, or null: the lengths of the surrogate grids
+// (samples S apart: a line fits a thread's registers up to 64)
+SpecKernel k_reg(const Axis &a)
+{
+    switch (a.m > 32 ? 0 : a.L * 2 + (a.m > 16)) {
+    case 64: return a.rows ? k_spectral_reg<32, 16, 1> : k_spectral_reg<32, 16, 0>;
+    case 96: return a.rows ? k_spectral_reg<48, 16, 1> : k_spectral_reg<48, 16, 0>;
+    case 128: return a.rows ? k_spectral_reg<64, 16, 1> : k_spectral_reg<64, 16, 0>;
+    case 129: return a.rows ? k_spectral_reg<64, 32, 1> : nullptr;
+    case 192:
+    case 193: return a.rows ? k_spectral_reg<96, 32, 1> : nullptr;
+    case 256:
+    case 257: return a.rows ? k_spectral_reg<128, 32, 1> : nullptr;
+    default: return nullptr;
+    }
+}
+
+}  // namespace
+
 // T: as many lines as leave room for two blocks per SM (long runs along the
 // lines and fewer reads of the weights), 4 lines in one block where they do not.
 bool axis_plan(Axis &a, int L, int m, int rows, int64_t S, int64_t outer, int W)
@@ -956,6 +1307,14 @@ bool axis_plan(Axis &a, int L, int m, int rows, int64_t S, int64_t outer, int W)
     a.dnq = recip(a.nq);
     a.dKG = recip(a.KG);
     a.dNG = recip(a.NG);
+    if (k_reg(a)) {
+        a.reg = 1;
+        a.T = rows ? 4 : 8;
+        a.KS = stride_for(W * a.T, 0) + 4;
+        a.smem = sizeof(float) * ((size_t)2 * m * a.KS + (size_t)W * (rows ? a.T * (L + 4) : a.T * L + 8));
+        if (a.smem <= SMEM_TWO) return true;
+        a.reg = 0;
+    }
     for (int T = 16; T >= 4; T /= 2) {
         a.T = T;
         a.DS = stride_for(2 * a.q * a.nq * T, T);
@@ -1001,6 +1360,10 @@ void spectral(const Axis &a, const float *v, float *u, int B, int W, int64_t N, 
     const int tiles = (int)((run + a.T - 1) / a.T);
     const int64_t total = (int64_t)B * tiles * (a.rows ? 1 : a.outer), NL = B * a.lines();
     const int grid = (int)std::min<int64_t>(total, (int64_t)gb300::sm_count() * (a.smem <= SMEM_TWO ? 2 : 1));
+    if (a.reg) {
+        k_reg(a)<<<grid, TPB, a.smem, s>>>(a, v, u, W, N, R, wk, ak, spec, NL, tiles, (int)total, accumulate);
+        return;
+    }
     auto k = a.rows ? (W == MAXW ? k_spectral<1, MAXW> : k_spectral<1, 0>)
                     : (W == MAXW ? k_spectral<0, MAXW> : k_spectral<0, 0>);
     k<<<grid, TPB, a.smem, s>>>(a, v, u, W, N, R, wk, ak, spec, NL, tiles, (int)total, accumulate);
@@ -1128,6 +1491,14 @@ void mlp_bwd(const Mlp &p, const float *x, const float *g, float *gx, float *par
 // The dynamic shared-memory limits are per device: set on every creation.
 bool set_attrs()
 {
+    for (int L : {32, 48, 64, 96, 128})
+        for (int m : {16, 32})
+            for (int rows : {0, 1}) {
+                Axis a{};
+                a.L = L; a.m = m; a.rows = rows;
+                SpecKernel k = k_reg(a);
+                if (k && !big(k, SMEM_TWO)) return false;
+            }
     return big(k_spectral<0, 0>, SMEM_MAX) && big(k_spectral<1, 0>, SMEM_MAX) &&
            big(k_spectral<0, MAXW>, SMEM_MAX) && big(k_spectral<1, MAXW>, SMEM_MAX) && big_act<ACT_GELU>() && big_act<ACT_SIREN>();
 }

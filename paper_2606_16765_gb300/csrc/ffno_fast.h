@@ -21,6 +21,7 @@ struct Axis {
     int L, m;
     int rows;                            // 1: the samples are contiguous (x); 0: S apart
     int64_t S, outer;                    // lines: outer x S (rows: outer, S = 1)
+    int reg;                             // 1: a register kernel exists for this length
     int T;                               // lines per block
     int q, nq;                           // parities, terms per folded sum
     int mk, KG, NG;                      // wave numbers per parity, groups of 4 of them, groups of 4 terms
@@ -47,7 +48,7 @@ void spectral(const Axis &a, const float *v, float *u, int B, int W, int64_t N, 
               const float *ak, float *spec, bool accumulate, cudaStream_t s);
 
 // R [i][o][m] complex (parameter layout, floats) of the three axes ->
-// rf [m][i][Wp], ra [m][o][Wp] conjugated
+// rf [m][i][Wp], ra [m][o][Wp] conjugated (rows in the order the mixing reads)
 struct PackR {
     struct { const float *R; int m; float2 *rf, *ra; } a[3];
 };
