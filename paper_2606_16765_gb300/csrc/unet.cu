@@ -32,6 +32,7 @@
 #include <cstddef>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -92,27 +93,54 @@ __global__ void k_pack_input(const float *__restrict__ x, int64_t N, int B, int 
     }
 }
 
+// 4 values per thread (n a multiple of 4: channel counts are multiples of 32);
+// s may sit on any float, d is scratch
 __global__ void k_f2bf(const float *__restrict__ s, bf16 *__restrict__ d, int64_t n)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        d[i] = __float2bfloat16_rn(s[i]);
+    const bool al = (reinterpret_cast<uintptr_t>(s) & 15) == 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / 4; i += (int64_t)gridDim.x * blockDim.x) {
+        const float4 v = al ? reinterpret_cast<const float4 *>(s)[i]
+                            : make_float4(s[4 * i], s[4 * i + 1], s[4 * i + 2], s[4 * i + 3]);
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        reinterpret_cast<uint2 *>(d)[i] = make_uint2(*reinterpret_cast<const uint32_t *>(&a),
+                                                     *reinterpret_cast<const uint32_t *>(&b));
+    }
 }
 
 // w [o][i][27] FP32 -> wf [27][o][ip] (i < cin, zeros above) and, if given,
-// wb [26 - d][ip][o] (the same values with the taps reversed, transposed).
-__global__ void k_pack_w(const float *__restrict__ w, int cout, int cin, int ip, bf16 *__restrict__ wf,
-                         bf16 *__restrict__ wb)
+// wb [26 - d][ip][o] (the same values with the taps reversed, transposed);
+// either may be null.  A block takes 16 x 16 (o, i) pairs through shared
+// memory: w is read along its rows and both results are written in 32-byte
+// runs (reading every 27th float took 16.8 us for 512 x 256 channels).
+constexpr int PW = 16;
+__global__ void __launch_bounds__(TPB) k_pack_w(const float *__restrict__ w, int cout, int cin, int ip,
+                                                bf16 *__restrict__ wf, bf16 *__restrict__ wb)
 {
-    const int64_t n = (int64_t)27 * cout * ip;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        const int d = (int)(k / ((int64_t)cout * ip));
-        const int r = (int)(k % ((int64_t)cout * ip));
-        const int o = r / ip, i = r % ip;
-        const bf16 v = __float2bfloat16_rn(i < cin ? w[((int64_t)o * cin + i) * 27 + d] : 0.f);
-        wf[k] = v;
-        if (wb) wb[((int64_t)(26 - d) * ip + i) * cout + o] = v;
+    __shared__ bf16 sh[PW][PW][28];
+    const int tiles_i = (ip + PW - 1) / PW;
+    const int o0 = (int)(blockIdx.x / tiles_i) * PW, i0 = (int)(blockIdx.x % tiles_i) * PW;
+    static_assert(PW * PW == TPB, "27 values per thread");
+    float v[27];                                   // all reads in flight at once
+#pragma unroll
+    for (int q = 0; q < 27; ++q) {
+        const int k = q * TPB + (int)threadIdx.x, d = k % 27, i = (k / 27) % PW, o = k / (27 * PW);
+        v[q] = o0 + o < cout && i0 + i < cin ? w[((int64_t)(o0 + o) * cin + i0 + i) * 27 + d] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < 27; ++q) {
+        const int k = q * TPB + (int)threadIdx.x;
+        sh[k / (27 * PW)][(k / 27) % PW][k % 27] = __float2bfloat16_rn(v[q]);
+    }
+    __syncthreads();
+#pragma unroll 9
+    for (int k = threadIdx.x; k < PW * PW * 27; k += TPB) {
+        const int x = k % PW, y = (k / PW) % PW, d = k / (PW * PW);
+        if (wf && o0 + y < cout && i0 + x < ip) wf[((int64_t)d * cout + o0 + y) * ip + i0 + x] = sh[y][x][d];
+        if (wb && o0 + x < cout && i0 + y < ip) wb[((int64_t)(26 - d) * ip + i0 + y) * cout + o0 + x] = sh[x][y][d];
     }
 }
+
+int pack_grid(int cout, int ip) { return ((cout + PW - 1) / PW) * ((ip + PW - 1) / PW); }
 
 // gwt [(d * ip + i)][o] -> gw [o][i][d]
 __global__ void k_wg_convert(const float *__restrict__ gwt, int cin, int ip, int cout, float *__restrict__ gw)
@@ -682,7 +710,7 @@ double normal(uint64_t &s)
 lbm_status pack_weights(unet_ctx *u)
 {
     for (Blk &b : u->blk)
-        k_pack_w<<<grid_for((int64_t)27 * b.cout * b.ip), TPB, 0, u->s>>>(u->params + b.ow, b.cout, b.cin, b.ip, b.wf,
+        k_pack_w<<<pack_grid(b.cout, b.ip), TPB, 0, u->s>>>(u->params + b.ow, b.cout, b.cin, b.ip, b.wf,
                                                                           b.wb);
     UCK(cudaGetLastError());
     return LBM_OK;
@@ -1129,16 +1157,53 @@ extern "C" const char *unet_last_error(const unet_ctx *u) { return u ? u->err.c_
 // ---------------------------------------------------------------------------
 namespace {
 
+// Scratch of one call, from a stream-ordered pool of the device that keeps up
+// to a gigabyte between calls (more goes back to the device at the next
+// synchronisation): cudaMalloc and cudaFree of the converted operands took
+// 0.26 to 0.38 ms per call.  Pools are created once per device under a lock;
+// the driver serialises their use by threads and orders it by stream.
+constexpr int MAX_DEV = 64;
+
+cudaMemPool_t op_pool()
+{
+    static std::mutex lock;
+    static cudaMemPool_t pool[MAX_DEV];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= MAX_DEV) return nullptr;
+    std::lock_guard<std::mutex> hold(lock);
+    if (!pool[dev]) {
+        cudaMemPoolProps pr{};
+        pr.allocType = cudaMemAllocationTypePinned;
+        pr.location.type = cudaMemLocationTypeDevice;
+        pr.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        uint64_t keep = (uint64_t)1 << 30;
+        if (cudaMemPoolCreate(&p, &pr) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+        pool[dev] = p;
+    }
+    return pool[dev];
+}
+
 struct OpScratch {
+    cudaStream_t s;
     std::vector<void *> p;
+    explicit OpScratch(cudaStream_t st) : s(st) {}
     ~OpScratch()
     {
-        for (void *q : p) cudaFree(q);
+        for (void *q : p) cudaFreeAsync(q, s);
     }
     template <class T> T *get(size_t n)
     {
+        const cudaMemPool_t pool = op_pool();
         void *q = nullptr;
-        if (cudaMalloc(&q, std::max<size_t>(n * sizeof(T), 16)) != cudaSuccess) return nullptr;
+        if (!pool || cudaMallocFromPoolAsync(&q, std::max<size_t>(n * sizeof(T), 16), pool, s) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
         p.push_back(q);
         return static_cast<T *>(q);
     }
@@ -1165,14 +1230,14 @@ lbm_status op_check(const void *a, const void *b, const void *c, int32_t B, int3
 
 lbm_status op_finish(cudaStream_t s, int *status)
 {
+    int st = 0;
     cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&st, status, sizeof st, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         g_unet_err = std::string("convolution: ") + cudaGetErrorString(e);
         return LBM_ERR_CUDA;
     }
-    int st = 0;
-    if (cudaMemcpy(&st, status, sizeof st, cudaMemcpyDeviceToHost) != cudaSuccess) return LBM_ERR_CUDA;
     if (st) {
         g_unet_err = "a bounded wait of a tensor-core kernel gave up (code " + std::to_string(st) + ")";
         return LBM_ERR_TIMEOUT;
@@ -1189,13 +1254,13 @@ extern "C" lbm_status unet_conv3_forward(const float *x, const float *w, float *
     if (st != LBM_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int64_t n = (int64_t)B * nx * ny * nz;
-    OpScratch sc;
+    OpScratch sc(s);
     bf16 *xb = sc.get<bf16>(n * cin), *wf = sc.get<bf16>((size_t)27 * cin * cout);
     int *status = sc.get<int>(1);
     if (!xb || !wf || !status) return LBM_ERR_OOM;
     cudaMemsetAsync(status, 0, sizeof(int), s);
-    k_f2bf<<<grid_for(n * cin), TPB, 0, s>>>(x, xb, n * cin);
-    k_pack_w<<<grid_for((int64_t)27 * cout * cin), TPB, 0, s>>>(w, cout, cin, cin, wf, nullptr);
+    k_f2bf<<<grid_for(n * cin / 4), TPB, 0, s>>>(x, xb, n * cin);
+    k_pack_w<<<pack_grid(cout, cin), TPB, 0, s>>>(w, cout, cin, cin, wf, nullptr);
     unet::ConvPlan p;
     const char *e = nullptr;
     if (!unet::conv_plan(p, xb, cin, cin, nx, ny, nz, B, wf, cout, 27, cout, 0, gb300::sm_count(), &e)) {
@@ -1214,14 +1279,13 @@ extern "C" lbm_status unet_conv3_backward_data(const float *gy, const float *w, 
     if (st != LBM_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int64_t n = (int64_t)B * nx * ny * nz;
-    OpScratch sc;
-    bf16 *gb = sc.get<bf16>(n * cout), *wf = sc.get<bf16>((size_t)27 * cin * cout),
-         *wb = sc.get<bf16>((size_t)27 * cin * cout);
+    OpScratch sc(s);
+    bf16 *gb = sc.get<bf16>(n * cout), *wb = sc.get<bf16>((size_t)27 * cin * cout);
     int *status = sc.get<int>(1);
-    if (!gb || !wf || !wb || !status) return LBM_ERR_OOM;
+    if (!gb || !wb || !status) return LBM_ERR_OOM;
     cudaMemsetAsync(status, 0, sizeof(int), s);
-    k_f2bf<<<grid_for(n * cout), TPB, 0, s>>>(gy, gb, n * cout);
-    k_pack_w<<<grid_for((int64_t)27 * cout * cin), TPB, 0, s>>>(w, cout, cin, cin, wf, wb);
+    k_f2bf<<<grid_for(n * cout / 4), TPB, 0, s>>>(gy, gb, n * cout);
+    k_pack_w<<<pack_grid(cout, cin), TPB, 0, s>>>(w, cout, cin, cin, nullptr, wb);
     unet::ConvPlan p;
     const char *e = nullptr;
     if (!unet::conv_plan(p, gb, cout, cout, nx, ny, nz, B, wb, cin, 27, cin, 0, gb300::sm_count(), &e)) {
@@ -1240,15 +1304,15 @@ extern "C" lbm_status unet_conv3_backward_weights(const float *x, const float *g
     if (st != LBM_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int64_t n = (int64_t)B * nx * ny * nz;
-    OpScratch sc;
+    OpScratch sc(s);
     bf16 *xb = sc.get<bf16>(n * cin), *gb = sc.get<bf16>(n * cout);
     float *gwt = sc.get<float>((size_t)27 * cin * cout);
     int *status = sc.get<int>(1);
     if (!xb || !gb || !gwt || !status) return LBM_ERR_OOM;
     cudaMemsetAsync(status, 0, sizeof(int), s);
     cudaMemsetAsync(gwt, 0, sizeof(float) * 27 * (size_t)cin * cout, s);
-    k_f2bf<<<grid_for(n * cin), TPB, 0, s>>>(x, xb, n * cin);
-    k_f2bf<<<grid_for(n * cout), TPB, 0, s>>>(gy, gb, n * cout);
+    k_f2bf<<<grid_for(n * cin / 4), TPB, 0, s>>>(x, xb, n * cin);
+    k_f2bf<<<grid_for(n * cout / 4), TPB, 0, s>>>(gy, gb, n * cout);
     unet::WgradPlan p;
     const char *e = nullptr;
     if (!unet::wgrad_plan(p, xb, cin, cin, gb, cout, cout, nx, ny, nz, B, gb300::sm_count(), &e)) {
