@@ -13,6 +13,11 @@
 // multiple of 64).  The input gradient is the same product with the weights
 // transposed and the taps reversed.
 //
+// Where the input has 32 or 64 channels on a large grid, those 27 shifted
+// copies are what the kernel waits for (8 KB of cells for two products): the
+// halo kernel below keeps a block of cells with its halo in shared memory
+// instead and takes every tap's operand from it.
+//
 // Weight gradient: G[(tap, i)][o] = sum over cells of X[cell + tap - 1][i] *
 // GZ[cell][o]: M = 128 (tap, input-channel) rows taken as four 32-channel
 // atoms, N = output channels, K = cells.  Here both operands are MN-major: the
@@ -29,6 +34,7 @@
 // copies in flight and the issued products are waited for (bounded again),
 // tensor memory is freed and the kernel returns.
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -387,6 +393,256 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
 }
 
 // ---------------------------------------------------------------------------
+// forward / input-gradient convolution from a halo block
+// ---------------------------------------------------------------------------
+// A block of bz x sy rows of X cells with its halo lies in shared memory as
+// [8-channel group][plane][row][P = X + 2 cells][16 bytes]: the unswizzled
+// K-major operand layout whose 8-row groups are 128 bytes apart, so that any
+// run of 128 cells is an A tile and a tap is an offset of the start address
+// by whole cells (16 bytes).  A plane's rows are one run of sy P cells cut
+// into tiles of 128 (one row each where X = 128); the two cells between rows
+// give results that are not stored.  Each input cell is fetched
+// (bz + 2)(sy + 2) / (bz sy) times instead of 27, and a tap's weights serve
+// all the block's tiles.  The products of an output are added in the order of
+// the kernel above (tap, channel chunk, 16 channels): the same bits.
+// Ten warps: four fetch the block (16-byte copies, zeros outside the grid),
+// one the weights (tensor map, a ring of stages), one issues, four store.  A
+// plane is handed back as soon as no later tap reads it.
+constexpr int HT = 320;
+
+struct HCtl {
+    uint64_t *afull, *aempty, *full, *empty, *accf, *acce, *drain;
+    uint32_t *tslot;
+    volatile int *abort;
+};
+
+constexpr int HPL = 6;                       // most planes of a block (bz + 2)
+
+__device__ __forceinline__ HCtl hctl_at(unsigned char *p, int S)
+{
+    HCtl c;
+    uint64_t *b = reinterpret_cast<uint64_t *>(p);
+    c.afull = b;
+    c.aempty = b + HPL;
+    c.accf = b + 2 * HPL;
+    c.acce = b + 2 * HPL + 2;
+    c.drain = b + 2 * HPL + 4;
+    c.full = b + 2 * HPL + 5;
+    c.empty = c.full + S;
+    c.tslot = reinterpret_cast<uint32_t *>(c.empty + S);
+    c.abort = reinterpret_cast<volatile int *>(c.tslot + 1);
+    return c;
+}
+
+// unswizzled K-major: `lbo` bytes between 8-channel groups, 128 between 8-row groups
+__device__ __forceinline__ uint64_t desc_plain(uint32_t addr, uint32_t lbo)
+{
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) |
+           ((uint64_t)1 << 46);
+}
+
+struct HItem {
+    int b, z0, y0, n0;
+};
+
+__device__ __forceinline__ HItem hitem(const HaloArgs &a, int64_t w)
+{
+    HItem it;
+    it.n0 = (int)(w % a.nntiles) * a.ntile;
+    w /= a.nntiles;
+    it.y0 = (int)(w % a.ty) * a.sy;
+    w /= a.ty;
+    it.z0 = (int)(w % a.tz) * a.bz;
+    it.b = (int)(w / a.tz);
+    return it;
+}
+
+template <int CK, class TO>
+__global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__restrict__ x,
+                                                     const __grid_constant__ CUtensorMap wmap, const HaloArgs a,
+                                                     TO *__restrict__ out, int *status)
+{
+    extern __shared__ unsigned char raw[];
+    unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+    const int S = a.stages;
+    unsigned char *sB = sm, *sA = sm + (size_t)S * a.b_bytes;
+    const HCtl c = hctl_at(sA + a.a_bytes, S);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, planes = a.bz + 2;
+    if (threadIdx.x == 0) {
+        for (int p = 0; p < planes; ++p) {
+            mbar_init(saddr(&c.afull[p]), 128);
+            mbar_init(saddr(&c.aempty[p]), 1);
+        }
+        for (int s = 0; s < S; ++s) {
+            mbar_init(saddr(&c.full[s]), 1);
+            mbar_init(saddr(&c.empty[s]), 1);
+        }
+        for (int q = 0; q < 2; ++q) {
+            mbar_init(saddr(&c.accf[q]), 1);
+            mbar_init(saddr(&c.acce[q]), 128);
+        }
+        mbar_init(saddr(c.drain), 1);
+        *c.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 5) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(saddr(c.tslot)),
+                     "r"(a.tmem_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    // zeros once: the cells beside every row stay zero
+    for (uint32_t q = threadIdx.x; q < a.a_bytes / 16; q += HT) reinterpret_cast<uint4 *>(sA)[q] = make_uint4(0, 0, 0, 0);
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    tc_before();
+    __syncthreads();
+    tc_after();
+    const uint32_t tmem = *c.tslot;
+    const int rows = a.sy + 2, P = a.X + 2, nk = 27 * a.kchunks;
+
+    if (warp < 4) {
+        // 16 bytes (8 channels of a cell) per copy
+        const int G = a.C / 8, per_row = a.X * G;
+        uint32_t n = 0;
+        bool ok = true;
+        for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x, ++n) {
+            const HItem it = hitem(a, w);
+            for (int p = 0; p < planes; ++p) {
+                if (!wait_bar(saddr(&c.aempty[p]), (n & 1) ^ 1, c.abort)) {
+                    fail(c.abort, status, 6);
+                    ok = false;
+                    break;
+                }
+                const int z = it.z0 + p - 1;
+                for (int r = 0; r < rows; ++r) {
+                    const int y = it.y0 + r - 1;
+                    const bool in = z >= 0 && z < a.Z && y >= 0 && y < a.Y;
+                    const __nv_bfloat16 *src = x + (((int64_t)it.b * a.Z + (in ? z : 0)) * a.Y + (in ? y : 0)) * a.X * a.C;
+                    const uint32_t dst = saddr(sA) + (uint32_t)(((p * rows + r) * P + 1) * 16);
+                    for (int q = (int)threadIdx.x; q < per_row; q += 128) {
+                        const int g = q & (G - 1), cell = q / G;
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst + g * a.lbo + cell * 16),
+                                     "l"(src + (int64_t)cell * a.C + g * 8), "r"(in ? 16 : 0)
+                                     : "memory");
+                    }
+                }
+                asm volatile("cp.async.wait_all;\n" ::: "memory");
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                mbar_arrive(saddr(&c.afull[p]));
+            }
+        }
+    } else if (warp == 4) {
+        if (lane == 0) {
+            uint32_t it = 0;
+            bool ok = true;
+            for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x) {
+                const int n0 = hitem(a, w).n0;
+                for (int tap = 0; ok && tap < 27; ++tap)
+                    for (int kc = 0; kc < a.kchunks; ++kc) {
+                        const uint32_t s = it % S;
+                        if (!wait_bar(saddr(&c.empty[s]), ((it / S) & 1) ^ 1, c.abort)) {
+                            fail(c.abort, status, 1);
+                            ok = false;
+                            break;
+                        }
+                        const uint32_t fb = saddr(&c.full[s]);
+                        mbar_expect_tx(fb, a.b_bytes);
+                        tma3(saddr(sB + (size_t)s * a.b_bytes), &wmap, kc * CK, n0, tap, fb);
+                        ++it;
+                    }
+            }
+            for (uint32_t j = it > (uint32_t)S ? it - S : 0; j < it; ++j)
+                if (!wait_bar(saddr(&c.full[j % S]), (j / S) & 1, nullptr)) atomicCAS(status, 0, 3);
+        }
+    } else if (warp == 5) {
+        if (lane == 0) {
+            uint32_t it = 0, n = 0;
+            bool ok = true;
+            const uint64_t a0 = desc_plain(saddr(sA), a.lbo);
+            for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x, ++n) {
+                const uint32_t set = a.sets == 2 ? n & 1 : 0, use = a.sets == 2 ? n >> 1 : n;
+                if (!wait_bar(saddr(&c.acce[set]), (use & 1) ^ 1, c.abort)) {
+                    fail(c.abort, status, 2);
+                    break;
+                }
+                tc_after();
+                const uint32_t d0 = tmem + set * (uint32_t)(a.ntiles * a.ntile);
+                int have = 0;                                  // planes that have arrived
+                for (int q = 0; ok && q < nk; ++q) {
+                    const int tap = q / a.kchunks, kc = q % a.kchunks;
+                    const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
+                    for (; have < dz + a.bz; ++have)
+                        if (!wait_bar(saddr(&c.afull[have]), n & 1, c.abort)) {
+                            fail(c.abort, status, 7);
+                            ok = false;
+                            break;
+                        }
+                    const uint32_t s = it % S;
+                    if (!ok || !wait_bar(saddr(&c.full[s]), (it / S) & 1, c.abort)) {
+                        fail(c.abort, status, 2);
+                        ok = false;
+                        break;
+                    }
+                    tc_after();
+                    const uint64_t bd = desc_k(saddr(sB + (size_t)s * a.b_bytes), CK * 2);
+                    uint32_t d = d0;
+                    for (int zo = 0; zo < a.bz; ++zo) {
+                        uint64_t ad = a0 + (uint64_t)(((zo + dz) * rows + dy) * P + dx) + (uint64_t)(kc * (CK / 8)) * (a.lbo >> 4);
+                        for (int t = 0; t < a.ptiles; ++t, d += (uint32_t)a.ntile, ad += (uint64_t)a.tstep)
+#pragma unroll
+                            for (int k = 0; k < CK / 16; ++k)
+                                umma(d, ad + (uint64_t)(2 * k) * (a.lbo >> 4), bd + 2 * k, a.idesc, (q > 0 || k > 0) ? 1u : 0u);
+                    }
+                    commit(saddr(&c.empty[s]));
+                    ++it;
+                    // planes 0 and 1 have no reader after the last tap of dz = 0 and 1
+                    if (kc == a.kchunks - 1 && (tap == 8 || tap == 17)) commit(saddr(&c.aempty[dz]));
+                }
+                if (!ok) break;
+                for (int p = 2; p < planes; ++p) commit(saddr(&c.aempty[p]));
+                commit(saddr(&c.accf[set]));
+            }
+            commit(saddr(c.drain));
+            if (!wait_bar(saddr(c.drain), 0, nullptr)) atomicCAS(status, 0, 4);
+        }
+    } else {
+        const int quad = warp & 3, row = quad * 32 + lane;
+        uint32_t n = 0;
+        for (int64_t w = blockIdx.x; w < a.nwork; w += gridDim.x, ++n) {
+            const uint32_t set = a.sets == 2 ? n & 1 : 0, use = a.sets == 2 ? n >> 1 : n;
+            if (!wait_bar(saddr(&c.accf[set]), use & 1, c.abort)) {
+                fail(c.abort, status, 5);
+                break;
+            }
+            tc_after();
+            const HItem it = hitem(a, w);
+            const uint32_t base = tmem + ((uint32_t)(quad * 32) << 16) + set * (uint32_t)(a.ntiles * a.ntile);
+            for (int t = 0; t < a.ntiles; ++t) {
+                const int zo = t / a.ptiles, j = (t % a.ptiles) * a.tstep + row, ry = j / P, rx = j - ry * P;
+                const int z = it.z0 + zo, y = it.y0 + ry;
+                const bool valid = rx < a.X && ry < a.sy && z < a.Z && y < a.Y;
+                TO *dst = out + ((((int64_t)it.b * a.Z + (valid ? z : 0)) * a.Y + (valid ? y : 0)) * a.X + (valid ? rx : 0)) * a.ldo +
+                          a.ooff + it.n0;
+                for (int cc = 0; cc < a.ntile; cc += 16) {
+                    float v[16];
+                    tmem_ld16(base + (uint32_t)(t * a.ntile + cc), v);
+                    if (valid) store16(dst + cc, v);
+                }
+            }
+            tc_before();
+            mbar_arrive(saddr(&c.acce[set]));
+        }
+    }
+    tc_before();
+    __syncthreads();
+    tc_after();
+    if (warp == 5) {
+        __syncwarp();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
+    }
+}
+
+// ---------------------------------------------------------------------------
 // weight gradient
 // ---------------------------------------------------------------------------
 struct WItem {
@@ -593,6 +849,8 @@ size_t ctl_bytes(int S) { return (size_t)(2 * S + 5) * 8 + 16; }
 
 }  // namespace
 
+static bool halo_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, int sms);
+
 bool conv_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, const void *w, int N,
                int ntaps, int ldo, int ooff, int sms, const char **err)
 {
@@ -635,7 +893,79 @@ bool conv_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z
     const cuuint64_t wstr[2] = {(cuuint64_t)k * 2, (cuuint64_t)k * 2 * N};
     const cuuint32_t wbox[3] = {(cuuint32_t)p.ck, (cuuint32_t)a.ntile, 1};
     if (!encode(p.wmap, 3, w, wdims, wstr, wbox, sw)) return bad("conv: weight tensor map rejected");
+    p.halo = false;
+    if (ntaps == 27) halo_plan(p, act, lda, k, X, Y, Z, B, sms);
     return true;
+}
+
+// The halo kernel's block: rows and planes that need the fewest cycles per
+// cell, from the products (an M = 128 tile reads its A rows at 128 bytes a
+// cycle: 32 + N / 4 cycles, or N / 2 where the products themselves take
+// longer) and the bytes fetched (about 50 a cycle on one SM, partly behind the
+// products); taken where that is at most 0.8 of the shifted copies' cost (27
+// taps of cells and weights at the 16.6 bytes a cycle and SM that all SMs
+// together reach).  lda = k: the block's cells are whole runs of channels.
+static bool halo_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, int sms)
+{
+    if (lda != k || (k != 32 && k != 64) || X < 16 || X > 128 || (reinterpret_cast<uintptr_t>(act) & 15)) return false;
+    const ConvArgs &o = p.a;
+    HaloArgs best{};
+    double best_cost = 1e300;
+    const int P = X + 2;
+    for (int bz = 1; bz <= std::min(4, Z); ++bz)
+        for (int sy = 1; sy <= Y; ++sy) {
+            HaloArgs a{};
+            a.bz = bz;
+            a.sy = sy;
+            a.tstep = X == 128 ? P : 128;
+            a.ptiles = X == 128 ? sy : (sy * P - 2 + 127) / 128;
+            a.ntiles = bz * a.ptiles;
+            if (a.ntiles * o.ntile > 512) continue;
+            a.sets = 2 * a.ntiles * o.ntile <= 512 ? 2 : 1;
+            const int cells = (bz + 2) * (sy + 2) * P + 130;           // and what the last tile reads past them
+            a.lbo = (uint32_t)cells * 16;
+            a.a_bytes = a.lbo * (uint32_t)(k / 8);
+            a.b_bytes = o.b_bytes;
+            const size_t room = SMEM_MAX - 1024 - 512;
+            if (a.a_bytes + 3 * (size_t)a.b_bytes > room) continue;
+            a.stages = (int)std::min<size_t>(8, (room - a.a_bytes) / a.b_bytes);
+            a.ty = (Y + sy - 1) / sy;
+            a.tz = (Z + bz - 1) / bz;
+            a.nwork = (int64_t)B * a.tz * a.ty * o.nntiles;
+            const double mma = (double)a.ntiles * 27 * (k / 16) * std::max(o.ntile / 2.0, 32.0 + o.ntile / 4.0);
+            const double load = ((double)cells * k * 2 + 27.0 * k * o.ntile * 2) / 50.0;
+            const double waves = std::ceil((double)a.nwork / std::max(1, sms));
+            const double cost = waves * (mma + 0.6 * load);
+            if (cost < best_cost) {
+                best_cost = cost;
+                best = a;
+            }
+        }
+    const double copies = std::ceil((double)o.nwork / std::max(1, sms)) * 27.0 * (256.0 * k + 2.0 * o.ntile * k) / 16.6;
+    if (best_cost > 0.8 * copies) return false;
+    HaloArgs &h = p.h;
+    h = best;
+    h.X = X; h.Y = Y; h.Z = Z; h.B = B;
+    h.C = k;
+    h.kchunks = o.kchunks;
+    h.ntile = o.ntile; h.nntiles = o.nntiles;
+    h.ldo = o.ldo; h.ooff = o.ooff;
+    h.idesc = o.idesc;
+    h.tmem_cols = 32;
+    while (h.tmem_cols < (uint32_t)(h.sets * h.ntiles * h.ntile)) h.tmem_cols <<= 1;
+    p.act = act;
+    p.halo = true;
+    p.smem = std::max(SMEM_ONE_CTA, 1024 + (size_t)h.stages * h.b_bytes + h.a_bytes + (size_t)(2 * HPL + 5 + 2 * h.stages) * 8 + 16);
+    p.grid = (int)std::min<int64_t>(h.nwork, std::max(1, sms));
+    return true;
+}
+
+template <int CK>
+static void launch_halo(const ConvPlan &p, const CUtensorMap &wm, void *out, bool out_f32, int *status, cudaStream_t s)
+{
+    const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(p.act);
+    if (out_f32) k_conv_halo<CK, float><<<p.grid, HT, p.smem, s>>>(x, wm, p.h, static_cast<float *>(out), status);
+    else k_conv_halo<CK, __nv_bfloat16><<<p.grid, HT, p.smem, s>>>(x, wm, p.h, static_cast<__nv_bfloat16 *>(out), status);
 }
 
 void conv_launch(const ConvPlan &p, void *out, bool out_f32, int *status, cudaStream_t s)
@@ -643,6 +973,11 @@ void conv_launch(const ConvPlan &p, void *out, bool out_f32, int *status, cudaSt
     CUtensorMap am, wm;
     std::memcpy(&am, p.amap, sizeof am);
     std::memcpy(&wm, p.wmap, sizeof wm);
+    if (p.halo) {
+        if (p.ck == 64) launch_halo<64>(p, wm, out, out_f32, status, s);
+        else launch_halo<32>(p, wm, out, out_f32, status, s);
+        return;
+    }
     if (p.ck == 64) {
         if (out_f32)
             k_conv_umma<64, float><<<p.grid, NT, p.smem, s>>>(am, wm, p.a, static_cast<float *>(out), status);
@@ -723,6 +1058,10 @@ bool gemm_set_attrs()
                     cudaFuncSetAttribute(k_conv_umma<64, __nv_bfloat16>, a, v) == cudaSuccess &&
                     cudaFuncSetAttribute(k_conv_umma<32, float>, a, v) == cudaSuccess &&
                     cudaFuncSetAttribute(k_conv_umma<32, __nv_bfloat16>, a, v) == cudaSuccess &&
+                    cudaFuncSetAttribute(k_conv_halo<64, float>, a, v) == cudaSuccess &&
+                    cudaFuncSetAttribute(k_conv_halo<64, __nv_bfloat16>, a, v) == cudaSuccess &&
+                    cudaFuncSetAttribute(k_conv_halo<32, float>, a, v) == cudaSuccess &&
+                    cudaFuncSetAttribute(k_conv_halo<32, __nv_bfloat16>, a, v) == cudaSuccess &&
                     cudaFuncSetAttribute(k_wgrad_umma, a, v) == cudaSuccess;
     done = ok ? 1 : -1;
     return ok;

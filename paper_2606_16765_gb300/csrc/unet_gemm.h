@@ -27,10 +27,25 @@ struct ConvArgs {
     uint32_t tmem_cols;          // tensor-memory columns (two accumulators)
 };
 
+// The same convolution from blocks of bz x sy rows with their halo.
+struct HaloArgs {
+    int X, Y, Z, B, C;
+    int bz, sy, ty, tz;          // planes and rows of a block, blocks along y and z
+    int ptiles, ntiles, tstep;   // 128-cell tiles per plane and block, cells between their starts
+    int sets;                    // accumulator sets (2: the next block's products overlap the stores)
+    int kchunks, ntile, nntiles, ldo, ooff, stages;
+    int64_t nwork;
+    uint32_t lbo;                // bytes between 8-channel groups
+    uint32_t a_bytes, b_bytes, idesc, tmem_cols;
+};
+
 struct ConvPlan {
     alignas(64) unsigned char amap[128];
     alignas(64) unsigned char wmap[128];
     ConvArgs a;
+    HaloArgs h;
+    bool halo = false;           // the halo kernel (k_conv_halo) takes this convolution
+    const void *act = nullptr;   // its activation
     int ck = 0;                  // chunk width: 64 (128-byte swizzle) or 32 (64-byte)
     size_t smem = 0;
     int grid = 0;
