@@ -139,6 +139,23 @@ __device__ __forceinline__ uint64_t desc_mn64(uint32_t addr, uint32_t lbo)
            ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
 }
 
+// One lane of a full warp.  The issuing loops run inside `if (elect_one())`:
+// there the compiler knows that a single thread runs and moves descriptors and
+// addresses straight to uniform registers (at most 60 cycles per product; 65
+// is what N = 128 takes in the tensor cores), while a lane == 0 branch costs a
+// loop over the active lanes around every instruction, 143 cycles per product
+// whatever its size.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t one = 0;
+    asm volatile(
+        "{\n\t.reg .b32 r;\n\t.reg .pred p;\n\t"
+        "elect.sync r|p, 0xffffffff;\n\t"
+        "@p mov.b32 %0, 1;\n\t}\n"
+        : "+r"(one));
+    return one != 0;
+}
+
 __device__ __forceinline__ void umma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate)
 {
     asm volatile(
@@ -154,6 +171,9 @@ __device__ __forceinline__ void commit(uint32_t bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
                  : "memory");
 }
+
+// a value every lane holds, marked as the same for the whole warp
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 __device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
@@ -296,13 +316,13 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
     unsigned char *sA = sm;
     unsigned char *sB = sm + (size_t)S * a.a_bytes;
     const Ctl c = ctl_at(sB + (size_t)S * a.b_bytes, S);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     ctl_init(c, S, a.tmem_cols);
-    const uint32_t tmem = *c.tslot;
+    const uint32_t tmem = uniform(*c.tslot);
     const int nk = a.ntaps * a.kchunks;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x) {
@@ -329,7 +349,7 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
             drain_loads(c, it, S, status);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0, tc = 0;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x, ++tc) {
@@ -350,8 +370,8 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
                     tc_after();
                     const uint64_t ad = desc_k(saddr(sA + (size_t)s * a.a_bytes), CK * 2);
                     const uint64_t bd = desc_k(saddr(sB + (size_t)s * a.b_bytes), CK * 2);
-#pragma unroll
-                    for (int k = 0; k < CK / 16; ++k)      // K = 16 per product: 32 bytes along the row
+    #pragma unroll
+                    for (int k = 0; k < CK / 16; ++k)          // K = 16 per product: 32 bytes along the row
                         umma(d, ad + 2 * k, bd + 2 * k, a.idesc, (q > 0 || k > 0) ? 1u : 0u);
                     commit(saddr(&c.empty[s]));
                     ++it;
@@ -360,6 +380,7 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
             }
             drain_mma(c, status);
         }
+        __syncwarp();
     } else {
         const int quad = warp & 3;                 // tensor-memory lanes 32 quad .. 32 quad + 31
         const int row = quad * 32 + lane;
@@ -467,7 +488,7 @@ __global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__rest
     const int S = a.stages;
     unsigned char *sB = sm, *sA = sm + (size_t)S * a.b_bytes;
     const HCtl c = hctl_at(sA + a.a_bytes, S);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, planes = a.bz + 2;
+    const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31, planes = a.bz + 2;
     if (threadIdx.x == 0) {
         for (int p = 0; p < planes; ++p) {
             mbar_init(saddr(&c.afull[p]), 128);
@@ -497,18 +518,31 @@ __global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__rest
     tc_before();
     __syncthreads();
     tc_after();
-    const uint32_t tmem = *c.tslot;
+    const uint32_t tmem = uniform(*c.tslot);
     const int rows = a.sy + 2, P = a.X + 2, nk = 27 * a.kchunks;
 
     if (warp < 4) {
-        // 16 bytes (8 channels of a cell) per copy
-        const int G = a.C / 8, per_row = a.X * G;
+        // 16 bytes (8 channels of a cell) per copy; a plane's copies are in
+        // flight while the next plane's are issued
+        constexpr int G = CK / 8, STEP = 128 / G;
+        const int g = (int)threadIdx.x & (G - 1), cell0 = (int)threadIdx.x / G;
         uint32_t n = 0;
+        int pending = -1;
         bool ok = true;
+        auto arrive = [&]() {
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            mbar_arrive(saddr(&c.afull[pending]));
+            pending = -1;
+        };
         for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x, ++n) {
             const HItem it = hitem(a, w);
             for (int p = 0; p < planes; ++p) {
-                if (!wait_bar(saddr(&c.aempty[p]), (n & 1) ^ 1, c.abort)) {
+                const uint32_t ready = saddr(&c.aempty[p]), parity = (n & 1) ^ 1;
+                if (pending >= 0 && !mbar_try(ready, parity)) {
+                    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+                    arrive();
+                }
+                if (!wait_bar(ready, parity, c.abort)) {
                     fail(c.abort, status, 6);
                     ok = false;
                     break;
@@ -517,22 +551,28 @@ __global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__rest
                 for (int r = 0; r < rows; ++r) {
                     const int y = it.y0 + r - 1;
                     const bool in = z >= 0 && z < a.Z && y >= 0 && y < a.Y;
-                    const __nv_bfloat16 *src = x + (((int64_t)it.b * a.Z + (in ? z : 0)) * a.Y + (in ? y : 0)) * a.X * a.C;
-                    const uint32_t dst = saddr(sA) + (uint32_t)(((p * rows + r) * P + 1) * 16);
-                    for (int q = (int)threadIdx.x; q < per_row; q += 128) {
-                        const int g = q & (G - 1), cell = q / G;
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst + g * a.lbo + cell * 16),
-                                     "l"(src + (int64_t)cell * a.C + g * 8), "r"(in ? 16 : 0)
+                    const __nv_bfloat16 *src =
+                        x + ((((int64_t)it.b * a.Z + (in ? z : 0)) * a.Y + (in ? y : 0)) * a.X + cell0) * CK + g * 8;
+                    const uint32_t dst = saddr(sA) + (uint32_t)(((p * rows + r) * P + 1 + cell0) * 16) + g * a.lbo;
+                    const uint32_t bytes = in ? 16 : 0;
+#pragma unroll 4
+                    for (int i = 0; i < a.X - cell0; i += STEP)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst + i * 16),
+                                     "l"(src + i * CK), "r"(bytes)
                                      : "memory");
-                    }
                 }
-                asm volatile("cp.async.wait_all;\n" ::: "memory");
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-                mbar_arrive(saddr(&c.afull[p]));
+                asm volatile("cp.async.commit_group;\n" ::: "memory");
+                if (pending >= 0) {
+                    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+                    arrive();
+                }
+                pending = p;
             }
         }
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        if (pending >= 0) arrive();
     } else if (warp == 4) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x) {
@@ -555,10 +595,11 @@ __global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__rest
                 if (!wait_bar(saddr(&c.full[j % S]), (j / S) & 1, nullptr)) atomicCAS(status, 0, 3);
         }
     } else if (warp == 5) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0, n = 0;
             bool ok = true;
             const uint64_t a0 = desc_plain(saddr(sA), a.lbo);
+            const uint32_t kstep = a.lbo >> 3;                     // two 8-channel groups, in 16 bytes
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x, ++n) {
                 const uint32_t set = a.sets == 2 ? n & 1 : 0, use = a.sets == 2 ? n >> 1 : n;
                 if (!wait_bar(saddr(&c.acce[set]), (use & 1) ^ 1, c.abort)) {
@@ -567,15 +608,12 @@ __global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__rest
                 }
                 tc_after();
                 const uint32_t d0 = tmem + set * (uint32_t)(a.ntiles * a.ntile);
-                int have = 0;                                  // planes that have arrived
-                for (int q = 0; ok && q < nk; ++q) {
-                    const int tap = q / a.kchunks, kc = q % a.kchunks;
-                    const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-                    for (; have < dz + a.bz; ++have)
+                int have = 0, tap = 0, kc = 0, dz = 0, dy = 0, dx = 0;   // planes that have arrived; the tap
+                for (int q = 0; q < nk; ++q) {
+                    for (; ok && have < dz + a.bz; ++have)
                         if (!wait_bar(saddr(&c.afull[have]), n & 1, c.abort)) {
                             fail(c.abort, status, 7);
                             ok = false;
-                            break;
                         }
                     const uint32_t s = it % S;
                     if (!ok || !wait_bar(saddr(&c.full[s]), (it / S) & 1, c.abort)) {
@@ -587,16 +625,27 @@ __global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__rest
                     const uint64_t bd = desc_k(saddr(sB + (size_t)s * a.b_bytes), CK * 2);
                     uint32_t d = d0;
                     for (int zo = 0; zo < a.bz; ++zo) {
-                        uint64_t ad = a0 + (uint64_t)(((zo + dz) * rows + dy) * P + dx) + (uint64_t)(kc * (CK / 8)) * (a.lbo >> 4);
-                        for (int t = 0; t < a.ptiles; ++t, d += (uint32_t)a.ntile, ad += (uint64_t)a.tstep)
-#pragma unroll
+                        uint64_t ad = a0 + (uint64_t)(uint32_t)(((zo + dz) * rows + dy) * P + dx + kc * (CK / 16) * (int)kstep);
+                        for (int t = 0; t < a.ptiles; ++t, d += (uint32_t)a.ntile, ad += (uint64_t)(uint32_t)a.tstep)
+    #pragma unroll
                             for (int k = 0; k < CK / 16; ++k)
-                                umma(d, ad + (uint64_t)(2 * k) * (a.lbo >> 4), bd + 2 * k, a.idesc, (q > 0 || k > 0) ? 1u : 0u);
+                                umma(d, ad + (uint64_t)(k * kstep), bd + 2 * k, a.idesc, (q > 0 || k > 0) ? 1u : 0u);
                     }
                     commit(saddr(&c.empty[s]));
                     ++it;
-                    // planes 0 and 1 have no reader after the last tap of dz = 0 and 1
-                    if (kc == a.kchunks - 1 && (tap == 8 || tap == 17)) commit(saddr(&c.aempty[dz]));
+                    if (++kc == a.kchunks) {
+                        // planes 0 and 1 have no reader after the last tap of dz = 0 and 1
+                        if (tap == 8 || tap == 17) commit(saddr(&c.aempty[dz]));
+                        kc = 0;
+                        ++tap;
+                        if (++dx == 3) {
+                            dx = 0;
+                            if (++dy == 3) {
+                                dy = 0;
+                                ++dz;
+                            }
+                        }
+                    }
                 }
                 if (!ok) break;
                 for (int p = 2; p < planes; ++p) commit(saddr(&c.aempty[p]));
@@ -605,6 +654,7 @@ __global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__rest
             commit(saddr(c.drain));
             if (!wait_bar(saddr(c.drain), 0, nullptr)) atomicCAS(status, 0, 4);
         }
+        __syncwarp();
     } else {
         const int quad = warp & 3, row = quad * 32 + lane;
         uint32_t n = 0;
@@ -672,13 +722,13 @@ __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CU
     unsigned char *sA = sm;
     unsigned char *sB = sm + (size_t)S * a.a_bytes;
     const Ctl c = ctl_at(sB + (size_t)S * a.b_bytes, S);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     ctl_init(c, S, a.tmem_cols);
-    const uint32_t tmem = *c.tslot;
+    const uint32_t tmem = uniform(*c.tslot);
     constexpr uint32_t ATOM = 128 * 64;            // 128 cells x 32 channels
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x) {
@@ -710,7 +760,7 @@ __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CU
             drain_loads(c, it, S, status);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t it = 0, tc = 0;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x) {
@@ -731,11 +781,11 @@ __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CU
                         break;
                     }
                     tc_after();
-                    const uint32_t a0 = saddr(sA + (size_t)s * a.a_bytes), b0 = saddr(sB + (size_t)s * a.b_bytes);
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)            // 16 cells (two 8-row groups) per product
-                        umma(d, desc_mn64(a0 + k * 1024, ATOM), desc_mn64(b0 + k * 1024, ATOM), a.idesc,
-                             (ch > wi.c0 || k > 0) ? 1u : 0u);
+                    const uint64_t ad = desc_mn64(saddr(sA + (size_t)s * a.a_bytes), ATOM),
+                                   bd = desc_mn64(saddr(sB + (size_t)s * a.b_bytes), ATOM);
+    #pragma unroll
+                    for (int k = 0; k < 8; ++k)                // 16 cells (two 8-row groups, 1024 bytes) per product
+                        umma(d, ad + 64 * k, bd + 64 * k, a.idesc, (ch > wi.c0 || k > 0) ? 1u : 0u);
                     commit(saddr(&c.empty[s]));
                     ++it;
                 }
@@ -744,6 +794,7 @@ __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CU
             }
             drain_mma(c, status);
         }
+        __syncwarp();
     } else {
         const int quad = warp & 3;
         const int row = quad * 32 + lane;
