@@ -83,10 +83,15 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// Operands arrive by copies that complete on the barrier (or are fenced by
+// their writers), so the issuing thread needs no tensor-core fence per stage;
+// the accumulators' barriers keep theirs.
+//
 // Wait for the phase of parity `parity`; false after WAIT_CYCLES or, when
 // `abort` is given, as soon as another role has set it.
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int *abort)
 {
+    if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try(bar, parity)) {
         if (abort && *abort) return false;
@@ -166,6 +171,35 @@ __device__ __forceinline__ void umma(uint32_t tmem, uint64_t a, uint64_t b, uint
         : "memory");
 }
 
+// The same with the descriptors' halves apart (only the low ones change).
+template <bool ACC>
+__device__ __forceinline__ void umma_lo(uint32_t tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                        uint32_t idesc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}\n" ::"r"(tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(ACC ? 1 : 0)
+        : "memory");
+}
+
+// One tap of a halo block: NT tiles x CK / 16 products, all
+// unrolled so that only the A address is formed per product (the tensor cores
+// take 32 + N / 4 cycles each, 40 at N = 32; a rolled loop issues one per 90).
+template <int NT, int CK, bool FIRST>
+__device__ __forceinline__ void halo_tap(const uint32_t *d, const uint32_t *off, uint32_t a_lo, uint32_t a_hi,
+                                         uint32_t kstep, uint32_t b_lo, uint32_t b_hi, uint32_t idesc)
+{
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+        umma_lo<!FIRST>(d[t], a_lo + off[t], a_hi, b_lo, b_hi, idesc);
+#pragma unroll
+        for (int k = 1; k < CK / 16; ++k) umma_lo<true>(d[t], a_lo + off[t] + k * kstep, a_hi, b_lo + 2 * k, b_hi, idesc);
+    }
+}
+
 __device__ __forceinline__ void commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
@@ -211,6 +245,19 @@ __device__ __forceinline__ void store16(__nv_bfloat16 *dst, const float *v)
     d[0] = make_uint4(w[0], w[1], w[2], w[3]);
     d[1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
+
+// Position in a ring of S stages: the stage and the parity of its round (kept
+// by counting: a division by S takes the issuing thread longer than a product).
+struct Ring {
+    uint32_t s = 0, round = 0;
+    __device__ __forceinline__ void next(int S)
+    {
+        if (++s == (uint32_t)S) {
+            s = 0;
+            round ^= 1;
+        }
+    }
+};
 
 struct Box {
     int x0, y0, z0, b0;
@@ -324,16 +371,16 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
     if (warp == 0) {
         if (elect_one()) {
             uint32_t it = 0;
+            Ring r;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x) {
                 const Box o = box_origin(w / a.nntiles, a.tx, a.ty, a.tz, a.bx, a.by, a.bz, a.bb);
                 const int n0 = (int)(w % a.nntiles) * a.ntile;
-                for (int q = 0; q < nk; ++q) {
-                    const int tap = q / a.kchunks, kc = q % a.kchunks;
+                for (int q = 0, tap = 0, kc = 0; q < nk; ++q) {
                     const int dz = a.ntaps == 1 ? 1 : tap / 9, dy = a.ntaps == 1 ? 1 : (tap / 3) % 3,
                               dx = a.ntaps == 1 ? 1 : tap % 3;
-                    const uint32_t s = it % S;
-                    if (!wait_bar(saddr(&c.empty[s]), ((it / S) & 1) ^ 1, c.abort)) {
+                    const uint32_t s = r.s;
+                    if (!wait_bar(saddr(&c.empty[s]), r.round ^ 1, c.abort)) {
                         fail(c.abort, status, 1);
                         ok = false;
                         break;
@@ -344,13 +391,19 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
                          o.z0 + dz - 1, o.b0, fb);
                     tma3(saddr(sB + (size_t)s * a.b_bytes), &wmap, kc * CK, n0, tap, fb);
                     ++it;
+                    r.next(S);
+                    if (++kc == a.kchunks) {
+                        kc = 0;
+                        ++tap;
+                    }
                 }
             }
             drain_loads(c, it, S, status);
         }
     } else if (warp == 1) {
         if (elect_one()) {
-            uint32_t it = 0, tc = 0;
+            uint32_t tc = 0;
+            Ring r;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x, ++tc) {
                 const uint32_t acc = tc & 1;
@@ -360,21 +413,19 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
                 }
                 tc_after();
                 const uint32_t d = tmem + acc * (uint32_t)a.ntile;
-                for (int q = 0; q < nk; ++q) {
-                    const uint32_t s = it % S;
-                    if (!wait_bar(saddr(&c.full[s]), (it / S) & 1, c.abort)) {
+                for (int q = 0; q < nk; ++q, r.next(S)) {
+                    const uint32_t s = r.s;
+                    if (!wait_bar(saddr(&c.full[s]), r.round, c.abort)) {
                         fail(c.abort, status, 2);
                         ok = false;
                         break;
                     }
-                    tc_after();
                     const uint64_t ad = desc_k(saddr(sA + (size_t)s * a.a_bytes), CK * 2);
                     const uint64_t bd = desc_k(saddr(sB + (size_t)s * a.b_bytes), CK * 2);
     #pragma unroll
                     for (int k = 0; k < CK / 16; ++k)          // K = 16 per product: 32 bytes along the row
                         umma(d, ad + 2 * k, bd + 2 * k, a.idesc, (q > 0 || k > 0) ? 1u : 0u);
                     commit(saddr(&c.empty[s]));
-                    ++it;
                 }
                 if (ok) commit(saddr(&c.accf[acc]));
             }
@@ -478,6 +529,62 @@ __device__ __forceinline__ HItem hitem(const HaloArgs &a, int64_t w)
     return it;
 }
 
+constexpr int HALO_TILES = 8;                // most tiles of a block
+
+// The issuing thread's loop over its blocks.
+template <int NT, int CK>
+__device__ __forceinline__ void halo_issue(const HaloArgs &a, const HCtl &c, unsigned char *sA, unsigned char *sB,
+                                           uint32_t tmem, int *status)
+{
+    const int S = a.stages, planes = a.bz + 2, rows = a.sy + 2, P = a.X + 2;
+    const uint64_t a0 = desc_plain(saddr(sA), a.lbo);
+    const uint32_t kstep = a.lbo >> 3;                     // two 8-channel groups, in 16 bytes
+    const uint32_t a_lo = (uint32_t)a0, a_hi = (uint32_t)(a0 >> 32);
+    uint32_t off[NT];
+#pragma unroll
+    for (int t = 0; t < NT; ++t) off[t] = (uint32_t)((t / a.ptiles) * rows * P + (t % a.ptiles) * a.tstep);
+    uint32_t n = 0;
+    Ring r;
+    for (int64_t w = blockIdx.x; w < a.nwork; w += gridDim.x, ++n) {
+        const uint32_t set = a.sets == 2 ? n & 1 : 0, use = a.sets == 2 ? n >> 1 : n;
+        if (!wait_bar(saddr(&c.acce[set]), (use & 1) ^ 1, c.abort)) {
+            fail(c.abort, status, 2);
+            return;
+        }
+        tc_after();
+        uint32_t d[NT];
+#pragma unroll
+        for (int t = 0; t < NT; ++t) d[t] = tmem + (set * NT + t) * (uint32_t)a.ntile;
+        int have = 0;                                      // planes that have arrived
+        for (int dz = 0; dz < 3; ++dz) {
+            for (; have < dz + a.bz; ++have)
+                if (!wait_bar(saddr(&c.afull[have]), n & 1, c.abort)) {
+                    fail(c.abort, status, 7);
+                    return;
+                }
+            for (int yx = 0; yx < 9; yx += a.tps, r.next(S)) {
+                if (!wait_bar(saddr(&c.full[r.s]), r.round, c.abort)) {
+                    fail(c.abort, status, 2);
+                    return;
+                }
+                const uint64_t bd = desc_k(saddr(sB + (size_t)r.s * a.b_bytes), CK * 2);
+                const uint32_t b_hi = (uint32_t)(bd >> 32);
+                uint32_t b_lo = (uint32_t)bd;
+                for (int j = yx; j < yx + a.tps; ++j, b_lo += a.tap_bytes >> 4) {
+                    const uint32_t al = a_lo + (uint32_t)((dz * rows + j / 3) * P + j % 3);
+                    if (dz + j == 0) halo_tap<NT, CK, true>(d, off, al, a_hi, kstep, b_lo, b_hi, a.idesc);
+                    else halo_tap<NT, CK, false>(d, off, al, a_hi, kstep, b_lo, b_hi, a.idesc);
+                }
+                commit(saddr(&c.empty[r.s]));
+            }
+            // planes 0 and 1 have no reader after the taps of dz = 0 and 1
+            if (dz < 2) commit(saddr(&c.aempty[dz]));
+        }
+        for (int p = 2; p < planes; ++p) commit(saddr(&c.aempty[p]));
+        commit(saddr(&c.accf[set]));
+    }
+}
+
 template <int CK, class TO>
 __global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__restrict__ x,
                                                      const __grid_constant__ CUtensorMap wmap, const HaloArgs a,
@@ -519,7 +626,7 @@ __global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__rest
     __syncthreads();
     tc_after();
     const uint32_t tmem = uniform(*c.tslot);
-    const int rows = a.sy + 2, P = a.X + 2, nk = 27 * a.kchunks;
+    const int rows = a.sy + 2, P = a.X + 2;
 
     if (warp < 4) {
         // 16 bytes (8 channels of a cell) per copy; a plane's copies are in
@@ -574,82 +681,36 @@ __global__ void __launch_bounds__(HT, 1) k_conv_halo(const __nv_bfloat16 *__rest
     } else if (warp == 4) {
         if (elect_one()) {
             uint32_t it = 0;
+            Ring r;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x) {
                 const int n0 = hitem(a, w).n0;
-                for (int tap = 0; ok && tap < 27; ++tap)
-                    for (int kc = 0; kc < a.kchunks; ++kc) {
-                        const uint32_t s = it % S;
-                        if (!wait_bar(saddr(&c.empty[s]), ((it / S) & 1) ^ 1, c.abort)) {
-                            fail(c.abort, status, 1);
-                            ok = false;
-                            break;
-                        }
-                        const uint32_t fb = saddr(&c.full[s]);
-                        mbar_expect_tx(fb, a.b_bytes);
-                        tma3(saddr(sB + (size_t)s * a.b_bytes), &wmap, kc * CK, n0, tap, fb);
-                        ++it;
+                for (int tap = 0; tap < 27; tap += a.tps, r.next(S)) {
+                    if (!wait_bar(saddr(&c.empty[r.s]), r.round ^ 1, c.abort)) {
+                        fail(c.abort, status, 1);
+                        ok = false;
+                        break;
                     }
+                    const uint32_t fb = saddr(&c.full[r.s]);
+                    mbar_expect_tx(fb, a.b_bytes);
+                    tma3(saddr(sB + (size_t)r.s * a.b_bytes), &wmap, 0, n0, tap, fb);
+                    ++it;
+                }
             }
             for (uint32_t j = it > (uint32_t)S ? it - S : 0; j < it; ++j)
                 if (!wait_bar(saddr(&c.full[j % S]), (j / S) & 1, nullptr)) atomicCAS(status, 0, 3);
         }
     } else if (warp == 5) {
         if (elect_one()) {
-            uint32_t it = 0, n = 0;
-            bool ok = true;
-            const uint64_t a0 = desc_plain(saddr(sA), a.lbo);
-            const uint32_t kstep = a.lbo >> 3;                     // two 8-channel groups, in 16 bytes
-            for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x, ++n) {
-                const uint32_t set = a.sets == 2 ? n & 1 : 0, use = a.sets == 2 ? n >> 1 : n;
-                if (!wait_bar(saddr(&c.acce[set]), (use & 1) ^ 1, c.abort)) {
-                    fail(c.abort, status, 2);
-                    break;
-                }
-                tc_after();
-                const uint32_t d0 = tmem + set * (uint32_t)(a.ntiles * a.ntile);
-                int have = 0, tap = 0, kc = 0, dz = 0, dy = 0, dx = 0;   // planes that have arrived; the tap
-                for (int q = 0; q < nk; ++q) {
-                    for (; ok && have < dz + a.bz; ++have)
-                        if (!wait_bar(saddr(&c.afull[have]), n & 1, c.abort)) {
-                            fail(c.abort, status, 7);
-                            ok = false;
-                        }
-                    const uint32_t s = it % S;
-                    if (!ok || !wait_bar(saddr(&c.full[s]), (it / S) & 1, c.abort)) {
-                        fail(c.abort, status, 2);
-                        ok = false;
-                        break;
-                    }
-                    tc_after();
-                    const uint64_t bd = desc_k(saddr(sB + (size_t)s * a.b_bytes), CK * 2);
-                    uint32_t d = d0;
-                    for (int zo = 0; zo < a.bz; ++zo) {
-                        uint64_t ad = a0 + (uint64_t)(uint32_t)(((zo + dz) * rows + dy) * P + dx + kc * (CK / 16) * (int)kstep);
-                        for (int t = 0; t < a.ptiles; ++t, d += (uint32_t)a.ntile, ad += (uint64_t)(uint32_t)a.tstep)
-    #pragma unroll
-                            for (int k = 0; k < CK / 16; ++k)
-                                umma(d, ad + (uint64_t)(k * kstep), bd + 2 * k, a.idesc, (q > 0 || k > 0) ? 1u : 0u);
-                    }
-                    commit(saddr(&c.empty[s]));
-                    ++it;
-                    if (++kc == a.kchunks) {
-                        // planes 0 and 1 have no reader after the last tap of dz = 0 and 1
-                        if (tap == 8 || tap == 17) commit(saddr(&c.aempty[dz]));
-                        kc = 0;
-                        ++tap;
-                        if (++dx == 3) {
-                            dx = 0;
-                            if (++dy == 3) {
-                                dy = 0;
-                                ++dz;
-                            }
-                        }
-                    }
-                }
-                if (!ok) break;
-                for (int p = 2; p < planes; ++p) commit(saddr(&c.aempty[p]));
-                commit(saddr(&c.accf[set]));
+            switch (a.ntiles) {
+            case 1: halo_issue<1, CK>(a, c, sA, sB, tmem, status); break;
+            case 2: halo_issue<2, CK>(a, c, sA, sB, tmem, status); break;
+            case 3: halo_issue<3, CK>(a, c, sA, sB, tmem, status); break;
+            case 4: halo_issue<4, CK>(a, c, sA, sB, tmem, status); break;
+            case 5: halo_issue<5, CK>(a, c, sA, sB, tmem, status); break;
+            case 6: halo_issue<6, CK>(a, c, sA, sB, tmem, status); break;
+            case 7: halo_issue<7, CK>(a, c, sA, sB, tmem, status); break;
+            default: halo_issue<8, CK>(a, c, sA, sB, tmem, status); break;
             }
             commit(saddr(c.drain));
             if (!wait_bar(saddr(c.drain), 0, nullptr)) atomicCAS(status, 0, 4);
@@ -730,13 +791,14 @@ __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CU
     if (warp == 0) {
         if (elect_one()) {
             uint32_t it = 0;
+            Ring r;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x) {
                 const WItem wi = witem(a, w);
                 for (int64_t ch = wi.c0; ch < wi.c1; ++ch) {
                     const Box o = box_origin(ch, a.tx, a.ty, a.tz, a.bx, a.by, a.bz, a.bb);
-                    const uint32_t s = it % S;
-                    if (!wait_bar(saddr(&c.empty[s]), ((it / S) & 1) ^ 1, c.abort)) {
+                    const uint32_t s = r.s;
+                    if (!wait_bar(saddr(&c.empty[s]), r.round ^ 1, c.abort)) {
                         fail(c.abort, status, 1);
                         ok = false;
                         break;
@@ -755,13 +817,15 @@ __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CU
                         tma5(saddr(sB + (size_t)s * a.b_bytes + j * ATOM), &gmap, wi.nt * a.ntile + j * 32, o.x0, o.y0,
                              o.z0, o.b0, fb);
                     ++it;
+                    r.next(S);
                 }
             }
             drain_loads(c, it, S, status);
         }
     } else if (warp == 1) {
         if (elect_one()) {
-            uint32_t it = 0, tc = 0;
+            uint32_t tc = 0;
+            Ring r;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x) {
                 const WItem wi = witem(a, w);
@@ -773,21 +837,19 @@ __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CU
                 }
                 tc_after();
                 const uint32_t d = tmem + acc * (uint32_t)a.ntile;
-                for (int64_t ch = wi.c0; ch < wi.c1; ++ch) {
-                    const uint32_t s = it % S;
-                    if (!wait_bar(saddr(&c.full[s]), (it / S) & 1, c.abort)) {
+                for (int64_t ch = wi.c0; ch < wi.c1; ++ch, r.next(S)) {
+                    const uint32_t s = r.s;
+                    if (!wait_bar(saddr(&c.full[s]), r.round, c.abort)) {
                         fail(c.abort, status, 2);
                         ok = false;
                         break;
                     }
-                    tc_after();
                     const uint64_t ad = desc_mn64(saddr(sA + (size_t)s * a.a_bytes), ATOM),
                                    bd = desc_mn64(saddr(sB + (size_t)s * a.b_bytes), ATOM);
     #pragma unroll
                     for (int k = 0; k < 8; ++k)                // 16 cells (two 8-row groups, 1024 bytes) per product
                         umma(d, ad + 64 * k, bd + 64 * k, a.idesc, (ch > wi.c0 || k > 0) ? 1u : 0u);
                     commit(saddr(&c.empty[s]));
-                    ++it;
                 }
                 if (ok) commit(saddr(&c.accf[acc]));
                 ++tc;
@@ -900,7 +962,7 @@ size_t ctl_bytes(int S) { return (size_t)(2 * S + 5) * 8 + 16; }
 
 }  // namespace
 
-static bool halo_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, int sms);
+static bool halo_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, const void *wt, int N, int sms);
 
 bool conv_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, const void *w, int N,
                int ntaps, int ldo, int ooff, int sms, const char **err)
@@ -945,7 +1007,7 @@ bool conv_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z
     const cuuint32_t wbox[3] = {(cuuint32_t)p.ck, (cuuint32_t)a.ntile, 1};
     if (!encode(p.wmap, 3, w, wdims, wstr, wbox, sw)) return bad("conv: weight tensor map rejected");
     p.halo = false;
-    if (ntaps == 27) halo_plan(p, act, lda, k, X, Y, Z, B, sms);
+    if (ntaps == 27) halo_plan(p, act, lda, k, X, Y, Z, B, w, N, sms);
     return true;
 }
 
@@ -956,7 +1018,7 @@ bool conv_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z
 // products); taken where that is at most 0.8 of the shifted copies' cost (27
 // taps of cells and weights at the 16.6 bytes a cycle and SM that all SMs
 // together reach).  lda = k: the block's cells are whole runs of channels.
-static bool halo_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, int sms)
+static bool halo_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, const void *wt, int N, int sms)
 {
     if (lda != k || (k != 32 && k != 64) || X < 16 || X > 128 || (reinterpret_cast<uintptr_t>(act) & 15)) return false;
     const ConvArgs &o = p.a;
@@ -971,13 +1033,15 @@ static bool halo_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y
             a.tstep = X == 128 ? P : 128;
             a.ptiles = X == 128 ? sy : (sy * P - 2 + 127) / 128;
             a.ntiles = bz * a.ptiles;
-            if (a.ntiles * o.ntile > 512) continue;
+            if (a.ntiles * o.ntile > 512 || a.ntiles > HALO_TILES) continue;
             a.sets = 2 * a.ntiles * o.ntile <= 512 ? 2 : 1;
             const int cells = (bz + 2) * (sy + 2) * P + 130;           // and what the last tile reads past them
             a.lbo = (uint32_t)cells * 16;
             a.a_bytes = a.lbo * (uint32_t)(k / 8);
-            a.b_bytes = o.b_bytes;
+            a.tap_bytes = o.b_bytes;
             const size_t room = SMEM_MAX - 1024 - 512;
+            a.tps = a.a_bytes + 9 * (size_t)a.tap_bytes <= room ? 3 : 1;     // taps per stage of weights
+            a.b_bytes = (uint32_t)a.tps * a.tap_bytes;
             if (a.a_bytes + 3 * (size_t)a.b_bytes > room) continue;
             a.stages = (int)std::min<size_t>(8, (room - a.a_bytes) / a.b_bytes);
             a.ty = (Y + sy - 1) / sy;
@@ -998,12 +1062,15 @@ static bool halo_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y
     h = best;
     h.X = X; h.Y = Y; h.Z = Z; h.B = B;
     h.C = k;
-    h.kchunks = o.kchunks;
     h.ntile = o.ntile; h.nntiles = o.nntiles;
     h.ldo = o.ldo; h.ooff = o.ooff;
     h.idesc = o.idesc;
     h.tmem_cols = 32;
     while (h.tmem_cols < (uint32_t)(h.sets * h.ntiles * h.ntile)) h.tmem_cols <<= 1;
+    const cuuint64_t wdims[3] = {(cuuint64_t)k, (cuuint64_t)N, 27};
+    const cuuint64_t wstr[2] = {(cuuint64_t)k * 2, (cuuint64_t)k * 2 * N};
+    const cuuint32_t wbox[3] = {(cuuint32_t)k, (cuuint32_t)h.ntile, (cuuint32_t)h.tps};
+    if (!encode(p.wmap, 3, wt, wdims, wstr, wbox, k == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B)) return false;
     p.act = act;
     p.halo = true;
     p.smem = std::max(SMEM_ONE_CTA, 1024 + (size_t)h.stages * h.b_bytes + h.a_bytes + (size_t)(2 * HPL + 5 + 2 * h.stages) * 8 + 16);

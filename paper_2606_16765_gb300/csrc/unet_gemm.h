@@ -33,8 +33,10 @@ struct HaloArgs {
     int bz, sy, ty, tz;          // planes and rows of a block, blocks along y and z
     int ptiles, ntiles, tstep;   // 128-cell tiles per plane and block, cells between their starts
     int sets;                    // accumulator sets (2: the next block's products overlap the stores)
-    int kchunks, ntile, nntiles, ldo, ooff, stages;
+    int ntile, nntiles, ldo, ooff, stages;
+    int tps;                     // taps per stage of weights (3 or 1)
     int64_t nwork;
+    uint32_t tap_bytes;          // weights of one tap
     uint32_t lbo;                // bytes between 8-channel groups
     uint32_t a_bytes, b_bytes, idesc, tmem_cols;
 };
