@@ -1228,6 +1228,30 @@ lbm_status op_check(const void *a, const void *b, const void *c, int32_t B, int3
     return LBM_OK;
 }
 
+// one convolution into FP32, through parts where the plan splits the sum
+lbm_status op_conv(OpScratch &sc, const bf16 *act, int k, int nx, int ny, int nz, int B, const bf16 *w, int N, float *out,
+                   int *status)
+{
+    unet::ConvPlan p;
+    const char *e = nullptr;
+    // the parts are added 16 bytes at a time
+    const bool split = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    if (!unet::conv_plan(p, act, k, k, nx, ny, nz, B, w, N, 27, N, 0, gb300::sm_count(), &e, split)) {
+        cudaStreamSynchronize(sc.s);
+        g_unet_err = e ? e : "plan failed";
+        return LBM_ERR_ARG;
+    }
+    if (p.a.ksplit == 1) {
+        unet::conv_launch(p, out, true, status, sc.s);
+        return LBM_OK;
+    }
+    float *part = sc.get<float>((size_t)p.a.ksplit * p.a.split_stride);
+    if (!part) return LBM_ERR_OOM;
+    unet::conv_launch(p, part, true, status, sc.s);
+    unet::conv_sum(p, part, out, sc.s);
+    return LBM_OK;
+}
+
 lbm_status op_finish(cudaStream_t s, int *status)
 {
     int st = 0;
@@ -1261,15 +1285,8 @@ extern "C" lbm_status unet_conv3_forward(const float *x, const float *w, float *
     cudaMemsetAsync(status, 0, sizeof(int), s);
     k_f2bf<<<grid_for(n * cin / 4), TPB, 0, s>>>(x, xb, n * cin);
     k_pack_w<<<pack_grid(cout, cin), TPB, 0, s>>>(w, cout, cin, cin, wf, nullptr);
-    unet::ConvPlan p;
-    const char *e = nullptr;
-    if (!unet::conv_plan(p, xb, cin, cin, nx, ny, nz, B, wf, cout, 27, cout, 0, gb300::sm_count(), &e)) {
-        cudaStreamSynchronize(s);
-        g_unet_err = e ? e : "plan failed";
-        return LBM_ERR_ARG;
-    }
-    unet::conv_launch(p, y, true, status, s);
-    return op_finish(s, status);
+    st = op_conv(sc, xb, cin, nx, ny, nz, B, wf, cout, y, status);
+    return st == LBM_OK ? op_finish(s, status) : st;
 }
 
 extern "C" lbm_status unet_conv3_backward_data(const float *gy, const float *w, float *gx, int32_t B, int32_t nx,
@@ -1286,15 +1303,8 @@ extern "C" lbm_status unet_conv3_backward_data(const float *gy, const float *w, 
     cudaMemsetAsync(status, 0, sizeof(int), s);
     k_f2bf<<<grid_for(n * cout / 4), TPB, 0, s>>>(gy, gb, n * cout);
     k_pack_w<<<pack_grid(cout, cin), TPB, 0, s>>>(w, cout, cin, cin, nullptr, wb);
-    unet::ConvPlan p;
-    const char *e = nullptr;
-    if (!unet::conv_plan(p, gb, cout, cout, nx, ny, nz, B, wb, cin, 27, cin, 0, gb300::sm_count(), &e)) {
-        cudaStreamSynchronize(s);
-        g_unet_err = e ? e : "plan failed";
-        return LBM_ERR_ARG;
-    }
-    unet::conv_launch(p, gx, true, status, s);
-    return op_finish(s, status);
+    st = op_conv(sc, gb, cout, nx, ny, nz, B, wb, cin, gx, status);
+    return st == LBM_OK ? op_finish(s, status) : st;
 }
 
 extern "C" lbm_status unet_conv3_backward_weights(const float *x, const float *gy, float *gw, int32_t B, int32_t nx,

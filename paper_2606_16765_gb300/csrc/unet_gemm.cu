@@ -367,6 +367,8 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
     ctl_init(c, S, a.tmem_cols);
     const uint32_t tmem = uniform(*c.tslot);
     const int nk = a.ntaps * a.kchunks;
+    // work item: (cell tile, channel tile, slice of the taps and chunks)
+    auto q_of = [&](int sp) { return nk * sp / a.ksplit; };
 
     if (warp == 0) {
         if (elect_one()) {
@@ -374,9 +376,11 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
             Ring r;
             bool ok = true;
             for (int64_t w = blockIdx.x; ok && w < a.nwork; w += gridDim.x) {
-                const Box o = box_origin(w / a.nntiles, a.tx, a.ty, a.tz, a.bx, a.by, a.bz, a.bb);
-                const int n0 = (int)(w % a.nntiles) * a.ntile;
-                for (int q = 0, tap = 0, kc = 0; q < nk; ++q) {
+                const int sp = (int)(w % a.ksplit);
+                const int64_t wt = w / a.ksplit;
+                const Box o = box_origin(wt / a.nntiles, a.tx, a.ty, a.tz, a.bx, a.by, a.bz, a.bb);
+                const int n0 = (int)(wt % a.nntiles) * a.ntile, q0 = q_of(sp), q1 = q_of(sp + 1);
+                for (int q = q0, tap = q0 / a.kchunks, kc = q0 % a.kchunks; q < q1; ++q) {
                     const int dz = a.ntaps == 1 ? 1 : tap / 9, dy = a.ntaps == 1 ? 1 : (tap / 3) % 3,
                               dx = a.ntaps == 1 ? 1 : tap % 3;
                     const uint32_t s = r.s;
@@ -413,7 +417,8 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
                 }
                 tc_after();
                 const uint32_t d = tmem + acc * (uint32_t)a.ntile;
-                for (int q = 0; q < nk; ++q, r.next(S)) {
+                const int sp = (int)(w % a.ksplit), q0 = q_of(sp), q1 = q_of(sp + 1);
+                for (int q = q0; q < q1; ++q, r.next(S)) {
                     const uint32_t s = r.s;
                     if (!wait_bar(saddr(&c.full[s]), r.round, c.abort)) {
                         fail(c.abort, status, 2);
@@ -424,7 +429,7 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
                     const uint64_t bd = desc_k(saddr(sB + (size_t)s * a.b_bytes), CK * 2);
     #pragma unroll
                     for (int k = 0; k < CK / 16; ++k)          // K = 16 per product: 32 bytes along the row
-                        umma(d, ad + 2 * k, bd + 2 * k, a.idesc, (q > 0 || k > 0) ? 1u : 0u);
+                        umma(d, ad + 2 * k, bd + 2 * k, a.idesc, (q > q0 || k > 0) ? 1u : 0u);
                     commit(saddr(&c.empty[s]));
                 }
                 if (ok) commit(saddr(&c.accf[acc]));
@@ -445,11 +450,12 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
                 break;
             }
             tc_after();
-            const Box o = box_origin(w / a.nntiles, a.tx, a.ty, a.tz, a.bx, a.by, a.bz, a.bb);
-            const int n0 = (int)(w % a.nntiles) * a.ntile;
+            const int64_t wt = w / a.ksplit;
+            const Box o = box_origin(wt / a.nntiles, a.tx, a.ty, a.tz, a.bx, a.by, a.bz, a.bb);
+            const int n0 = (int)(wt % a.nntiles) * a.ntile;
             const int b = o.b0 + rb;
             const bool valid = b < a.B;
-            TO *dst = out + ((((int64_t)(valid ? b : 0) * a.Z + o.z0 + rz) * a.Y + o.y0 + ry) * a.X + o.x0 + rx) * a.ldo +
+            TO *dst = out + (w % a.ksplit) * a.split_stride + ((((int64_t)(valid ? b : 0) * a.Z + o.z0 + rz) * a.Y + o.y0 + ry) * a.X + o.x0 + rx) * a.ldo +
                       a.ooff + n0;
             const uint32_t base = tmem + ((uint32_t)(quad * 32) << 16) + acc * (uint32_t)a.ntile;
             for (int cc = 0; cc < a.ntile; cc += 16) {
@@ -965,7 +971,7 @@ size_t ctl_bytes(int S) { return (size_t)(2 * S + 5) * 8 + 16; }
 static bool halo_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, const void *wt, int N, int sms);
 
 bool conv_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, const void *w, int N,
-               int ntaps, int ldo, int ooff, int sms, const char **err)
+               int ntaps, int ldo, int ooff, int sms, const char **err, bool split)
 {
     auto bad = [&](const char *m) {
         if (err) *err = m;
@@ -984,13 +990,26 @@ bool conv_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z
     a.ntaps = ntaps;
     a.kchunks = k / p.ck;
     a.ntile = pick_ntile(N);
+    const int64_t cell_tiles = (int64_t)a.tx * a.ty * a.tz * a.tb;
+    const int nk = ntaps * a.kchunks;
+    // A few cell tiles leave most SMs idle behind one long chain of products:
+    // narrower channel tiles, and (where the caller adds the parts up) slices
+    // of the taps and chunks, at least 8 of them each.  512 channels from 256
+    // at 8x4x4, batch 2 (2 cell tiles): 44 us on 4 SMs, 9 x 16 items 8.9 us and
+    // 3.7 us for the sum of the parts.
+    a.ksplit = 1;
+    if (split && cell_tiles * (N / a.ntile) * 2 <= sms) {
+        while (a.ntile > 64 && a.ntile % 64 == 0 && cell_tiles * (N / a.ntile) * 8 < sms) a.ntile /= 2;
+        a.ksplit = (int)std::max<int64_t>(1, std::min<int64_t>(nk / 8, sms / (cell_tiles * (N / a.ntile))));
+    }
+    a.split_stride = (int64_t)X * Y * Z * B * ldo;
     a.nntiles = N / a.ntile;
     a.ldo = ldo; a.ooff = ooff;
     a.a_bytes = 128u * p.ck * 2;
     a.b_bytes = (uint32_t)a.ntile * p.ck * 2;
     a.stages = (int)std::min<size_t>(8, (SMEM_MAX - 2048 - ctl_bytes(8)) / (a.a_bytes + a.b_bytes));
     if (a.stages < 2) return bad("conv: tile does not fit in shared memory");
-    a.nwork = (int64_t)a.tx * a.ty * a.tz * a.tb * a.nntiles;
+    a.nwork = cell_tiles * a.nntiles * a.ksplit;
     a.idesc = idesc_for(a.ntile, false, false);
     a.tmem_cols = tmem_cols_for(a.ntile);
     p.smem = std::max(SMEM_ONE_CTA, 1024 + (size_t)a.stages * (a.a_bytes + a.b_bytes) + ctl_bytes(a.stages));
@@ -1007,7 +1026,7 @@ bool conv_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z
     const cuuint32_t wbox[3] = {(cuuint32_t)p.ck, (cuuint32_t)a.ntile, 1};
     if (!encode(p.wmap, 3, w, wdims, wstr, wbox, sw)) return bad("conv: weight tensor map rejected");
     p.halo = false;
-    if (ntaps == 27) halo_plan(p, act, lda, k, X, Y, Z, B, w, N, sms);
+    if (ntaps == 27 && a.ksplit == 1) halo_plan(p, act, lda, k, X, Y, Z, B, w, N, sms);
     return true;
 }
 
@@ -1084,6 +1103,30 @@ static void launch_halo(const ConvPlan &p, const CUtensorMap &wm, void *out, boo
     const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(p.act);
     if (out_f32) k_conv_halo<CK, float><<<p.grid, HT, p.smem, s>>>(x, wm, p.h, static_cast<float *>(out), status);
     else k_conv_halo<CK, __nv_bfloat16><<<p.grid, HT, p.smem, s>>>(x, wm, p.h, static_cast<__nv_bfloat16 *>(out), status);
+}
+
+// out = sum of the parts, in their order
+__global__ void __launch_bounds__(256) k_sum_split(const float4 *__restrict__ part, int parts, int64_t n4,
+                                                   float4 *__restrict__ out)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
+        float4 s = part[i];
+        for (int p = 1; p < parts; ++p) {
+            const float4 v = part[p * n4 + i];
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+        out[i] = s;
+    }
+}
+
+void conv_sum(const ConvPlan &p, const float *part, float *out, cudaStream_t s)
+{
+    const int64_t n4 = p.a.split_stride / 4;
+    k_sum_split<<<(unsigned)std::min<int64_t>((n4 + 255) / 256, 2048), 256, 0, s>>>(
+        reinterpret_cast<const float4 *>(part), p.a.ksplit, n4, reinterpret_cast<float4 *>(out));
 }
 
 void conv_launch(const ConvPlan &p, void *out, bool out_f32, int *status, cudaStream_t s)

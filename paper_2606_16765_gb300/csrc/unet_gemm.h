@@ -21,7 +21,9 @@ struct ConvArgs {
     int ntile, nntiles;          // output channels per tile, tiles
     int ldo, ooff;               // output row stride and channel offset
     int stages;                  // pipeline depth
-    int64_t nwork;               // cell tiles x channel tiles
+    int ksplit;                  // slices of the taps and chunks (parts of the sum)
+    int64_t split_stride;        // elements between the parts
+    int64_t nwork;               // cell tiles x channel tiles x slices
     uint32_t a_bytes, b_bytes;   // shared-memory bytes of one stage's operands
     uint32_t idesc;              // instruction descriptor
     uint32_t tmem_cols;          // tensor-memory columns (two accumulators)
@@ -84,7 +86,10 @@ struct WgradPlan {
 
 // false: unsupported shape or tensor-map encoding failed (message in err).
 bool conv_plan(ConvPlan &p, const void *act, int lda, int k, int X, int Y, int Z, int B, const void *w, int N,
-               int ntaps, int ldo, int ooff, int sms, const char **err);
+               int ntaps, int ldo, int ooff, int sms, const char **err, bool split = false);
+// With `split` the plan may write p.a.ksplit > 1 FP32 parts (p.a.split_stride
+// elements apart, contiguous output rows) that conv_sum adds up.
+void conv_sum(const ConvPlan &p, const float *part, float *out, cudaStream_t s);
 void conv_launch(const ConvPlan &p, void *out, bool out_f32, int *status, cudaStream_t s);
 
 bool wgrad_plan(WgradPlan &p, const void *x, int ldx, int cin, const void *gz, int ldg, int N, int X, int Y, int Z,
