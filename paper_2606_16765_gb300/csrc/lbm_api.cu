@@ -137,6 +137,7 @@ struct lbm_ctx {
     double force_w[3] = {0, 0, 0};    // constant w-part of the obstacle force
     bool unstable = false;
     bool in_batch = false;
+    SideStream side{};                // the edge kernel's stream (from the first step on)
     // interpolated bounce-back links (device, owned by the context)
     uint4 *qlinks = nullptr;
     double *qval = nullptr, *qpart = nullptr;
@@ -443,11 +444,48 @@ extern "C" lbm_status lbm_create_in(const lbm_grid *g, const uint8_t *mask, cons
     return create_impl(g, mask, p, stream, workspace, ws_bytes, out);
 }
 
+static void side_destroy(SideStream &d)
+{
+    if (d.s) cudaStreamDestroy(d.s);
+    if (d.fork) cudaEventDestroy(d.fork);
+    if (d.join) cudaEventDestroy(d.join);
+    d = SideStream{};
+}
+
+// The side stream, created on first use; null (the kernels then follow one
+// another) where that fails, where `s` is being captured before it exists, and
+// on large grids: there the bulk kernel fills the chip for long and the edge
+// blocks' registers cost it more than they hide.  Per step, one after the
+// other and side by side: 64x32x32 26.0 and 21.4 us, 256x128x128 197 and 191
+// us (FP32), eight channels of 12 M cells 650 and 645 us (F16C), 512x256x256
+// (33.5 M cells) 1.040 and 1.054 ms (FP16).
+constexpr int64_t SIDE_CELLS = (int64_t)1 << 24;
+
+static const SideStream *side_of(SideStream &d, cudaStream_t s, int64_t cells)
+{
+    if (cells > SIDE_CELLS) return nullptr;
+    if (d.join) return &d;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (cudaStreamCreateWithFlags(&d.s, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&d.fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&d.join, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        side_destroy(d);
+        return nullptr;
+    }
+    return &d;
+}
+
 extern "C" lbm_status lbm_destroy(lbm_ctx *ctx)
 {
     if (!ctx) return LBM_ERR_ARG;
     cudaStreamSynchronize(ctx->stream);
     for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
+    side_destroy(ctx->side);
     cudaFree(ctx->probe_cells);
     cudaFree(ctx->probe_ring);
     cudaFree(ctx->plane_ring);
@@ -524,12 +562,14 @@ static void step_launch(lbm_ctx *ctx, const StepArgs &a, bool odd, bool epi)
             e1 = e2 = nullptr;
         }
     }
+    // timed steps run one kernel after the other: the events lie between them
+    const SideStream *side = ctx->timing ? nullptr : side_of(ctx->side, ctx->stream, ctx->L.n);
     switch (ctx->p.storage) {
-    case LBM_F64: launch_step_f64(a, odd, epi, ctx->plain, ctx->block_x, ctx->block_y, ctx->stream, e1, e2); break;
-    case LBM_F32: launch_step_f32(a, odd, epi, ctx->plain, ctx->block_x, ctx->block_y, ctx->stream, e1, e2); break;
-    case LBM_F16S: launch_step_f16(a, odd, epi, ctx->plain, ctx->block_x, ctx->block_y, ctx->stream, e1, e2); break;
-    case LBM_BF16S: launch_step_bf16(a, odd, epi, ctx->plain, ctx->block_x, ctx->block_y, ctx->stream, e1, e2); break;
-    default: launch_step_f16c(a, odd, epi, ctx->plain, ctx->block_x, ctx->block_y, ctx->stream, e1, e2); break;
+    case LBM_F64: launch_step_f64(a, odd, epi, ctx->plain, ctx->block_x, ctx->block_y, ctx->stream, e1, e2, side); break;
+    case LBM_F32: launch_step_f32(a, odd, epi, ctx->plain, ctx->block_x, ctx->block_y, ctx->stream, e1, e2, side); break;
+    case LBM_F16S: launch_step_f16(a, odd, epi, ctx->plain, ctx->block_x, ctx->block_y, ctx->stream, e1, e2, side); break;
+    case LBM_BF16S: launch_step_bf16(a, odd, epi, ctx->plain, ctx->block_x, ctx->block_y, ctx->stream, e1, e2, side); break;
+    default: launch_step_f16c(a, odd, epi, ctx->plain, ctx->block_x, ctx->block_y, ctx->stream, e1, e2, side); break;
     }
     if (e2) cudaEventRecord(e3, ctx->stream);
     ctx->launches += 1 + (a.n_edge > 0 || a.n_wall > 0 ? 1 : 0) + (a.face_x_hi == FACE_OUTFLOW ? 1 : 0) +
@@ -1343,6 +1383,7 @@ struct lbm_batch {
     int block_x = 128, block_y = 1;
     cudaStream_t user = nullptr, own = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+    SideStream side{};                  // the edge kernel's branch of the captured steps
     BatchMember *d_mem = nullptr;
     int64_t *d_bbegin = nullptr, *d_ebegin = nullptr, *d_qbegin = nullptr, *d_wbegin = nullptr, *d_t = nullptr;
     std::vector<int> live;              // members in the current table
@@ -1383,6 +1424,7 @@ extern "C" lbm_status lbm_batch_destroy(lbm_batch *b)
     if (b->ev_in) cudaEventDestroy(b->ev_in);
     if (b->ev_out) cudaEventDestroy(b->ev_out);
     if (b->own) cudaStreamDestroy(b->own);
+    side_destroy(b->side);
     for (lbm_ctx *c : b->members) lbm_destroy(c);
     delete b;
     return LBM_OK;
@@ -1558,16 +1600,19 @@ static lbm_status batch_rebuild(lbm_batch *b, const std::vector<int> &live)
         b->graph = nullptr;
     }
     cudaGraph_t graph;
+    int64_t cells = 0;
+    for (int g : live) cells += b->members[g]->L.n;
+    const SideStream *side = side_of(b->side, b->own, cells);
     BCK(cudaStreamBeginCapture(b->own, cudaStreamCaptureModeThreadLocal));
     for (int64_t k = 0; k < b->chunk; ++k) {
         const bool odd = (k & 1) != 0;
         const bool epi = b->mean_every > 0 && k == 0;   // chunks start at multiples of mean_every
         switch (b->storage) {
-        case LBM_F64: launch_batch_step_f64(b->launch, odd, epi, b->plain, b->own); break;
-        case LBM_F32: launch_batch_step_f32(b->launch, odd, epi, b->plain, b->own); break;
-        case LBM_F16S: launch_batch_step_f16(b->launch, odd, epi, b->plain, b->own); break;
-        case LBM_BF16S: launch_batch_step_bf16(b->launch, odd, epi, b->plain, b->own); break;
-        default: launch_batch_step_f16c(b->launch, odd, epi, b->plain, b->own); break;
+        case LBM_F64: launch_batch_step_f64(b->launch, odd, epi, b->plain, b->own, side); break;
+        case LBM_F32: launch_batch_step_f32(b->launch, odd, epi, b->plain, b->own, side); break;
+        case LBM_F16S: launch_batch_step_f16(b->launch, odd, epi, b->plain, b->own, side); break;
+        case LBM_BF16S: launch_batch_step_bf16(b->launch, odd, epi, b->plain, b->own, side); break;
+        default: launch_batch_step_f16c(b->launch, odd, epi, b->plain, b->own, side); break;
         }
     }
     const cudaError_t ce = cudaStreamEndCapture(b->own, &graph);
@@ -1631,7 +1676,6 @@ extern "C" lbm_status lbm_batch_run(lbm_batch *b, int64_t nsteps)
         b->graph_launches += chunks;
         b->kernel_launches += chunks * b->chunk *
                               (2 + (b->launch.edge_blocks + b->launch.w_blocks > 0 ? 1 : 0) +
-                               (b->launch.out_chunks > 0 ? 1 : 0) +
                                (b->launch.q_blocks > 0 ? 1 : 0));
         b->t = seg_end;
     }

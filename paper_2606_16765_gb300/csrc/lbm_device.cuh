@@ -200,6 +200,16 @@ struct BatchLaunch {
     int64_t w_blocks;           // wall-row blocks in all (0: none)
 };
 
+// A second stream for the edge kernel of a step: its blocks (few, long, bound
+// by latency and instruction fetch) run beside the bulk kernel's.  Every cell
+// writes exactly the slots it reads, so the two kernels of a step never touch
+// the same word; `fork` and `join` order them after the previous step and
+// before what follows.
+struct SideStream {
+    cudaStream_t s;
+    cudaEvent_t fork, join;
+};
+
 // A parameter in the compute type: the FP32 copy for float kernels.
 template <class R> __device__ __forceinline__ R pick(double d, float f);
 template <> __device__ __forceinline__ float pick<float>(double, float f) { return f; }

@@ -649,8 +649,9 @@ __global__ void __launch_bounds__(EDGE_BLOCK) k_batch_edge(const BatchMember *me
 // End of a batched step: the convective outflow of every member with that
 // outlet (grid x = member, grid y splits its outlet plane, grid z = direction) ...
 template <class S>
-__global__ void __launch_bounds__(256) k_batch_outflow(const BatchMember *mem, int nm, int fix, int next_odd)
+__global__ void __launch_bounds__(256) k_batch_outflow(const BatchMember *mem, int nm, int fix, int next_odd, int64_t *tick)
 {
+    if (tick && threadIdx.x + blockIdx.x + blockIdx.y + blockIdx.z == 0) *tick += 1;     // nothing here reads it
     const StepArgs &a = mem[blockIdx.x].a;
     if (a.face_x_hi != FACE_OUTFLOW) return;
     const uint32_t P = (uint32_t)a.ny * (uint32_t)a.nz;
@@ -686,10 +687,29 @@ static __global__ void k_batch_tick(int64_t *t)
 }
 
 template <class S>
-void launch_batch_step_t(const BatchLaunch &L, bool odd, bool epi, bool plain, cudaStream_t s)
+void launch_batch_step_t(const BatchLaunch &L, bool odd, bool epi, bool plain, cudaStream_t s, const SideStream *side)
 {
     const dim3 blk(L.block_x, L.block_y);
     const unsigned nb = (unsigned)L.bulk_blocks, ne = (unsigned)(L.edge_blocks + L.w_blocks);
+    const bool fork = side && ne > 0;
+    const cudaStream_t se = fork ? side->s : s;
+    auto edge = [&]() {
+        if (ne == 0) return;
+#define LBM_BE(O, P) k_batch_edge<S, O, P><<<ne, EDGE_BLOCK, 0, se>>>(L.mem, L.edge_begin, L.nm, L.t, epi, \
+                                                                     L.edge_blocks, L.w_begin)
+        if (plain) {
+            if (odd) LBM_BE(true, true); else LBM_BE(false, true);
+        } else {
+            if (odd) LBM_BE(true, false); else LBM_BE(false, false);
+        }
+#undef LBM_BE
+    };
+    if (fork) {
+        cudaEventRecord(side->fork, s);
+        cudaStreamWaitEvent(side->s, side->fork, 0);
+        edge();
+        cudaEventRecord(side->join, side->s);
+    }
 #define LBM_BB(O, E, P) k_batch_bulk<S, O, E, P><<<nb, blk, 0, s>>>(L.mem, L.bulk_begin, L.nm, L.t)
     if (plain) {
         if (odd) { if (epi) LBM_BB(true, true, true); else LBM_BB(true, false, true); }
@@ -699,29 +719,44 @@ void launch_batch_step_t(const BatchLaunch &L, bool odd, bool epi, bool plain, c
         else     { if (epi) LBM_BB(false, true, false); else LBM_BB(false, false, false); }
     }
 #undef LBM_BB
-    if (ne > 0) {
-        if (plain) {
-#define LBM_BE(O, P) k_batch_edge<S, O, P><<<ne, EDGE_BLOCK, 0, s>>>(L.mem, L.edge_begin, L.nm, L.t, epi, \
-                                                                    L.edge_blocks, L.w_begin)
-            if (odd) LBM_BE(true, true); else LBM_BE(false, true);
-        } else {
-            if (odd) LBM_BE(true, false); else LBM_BE(false, false);
-#undef LBM_BE
-        }
-    }
+    if (fork) cudaStreamWaitEvent(s, side->join, 0);
+    else edge();
     if (L.q_blocks > 0)
         k_batch_qbb<S><<<(unsigned)L.q_blocks, EDGE_BLOCK, 0, s>>>(L.mem, L.q_begin, L.nm, L.t, odd ? 0 : 1);
     if (L.out_chunks > 0)
-        k_batch_outflow<S><<<dim3((unsigned)L.nm, (unsigned)L.out_chunks, 9), 256, 0, s>>>(L.mem, L.nm, 1, odd ? 0 : 1);
-    k_batch_tick<<<1, 32, 0, s>>>(L.t);
+        k_batch_outflow<S><<<dim3((unsigned)L.nm, (unsigned)L.out_chunks, 9), 256, 0, s>>>(L.mem, L.nm, 1, odd ? 0 : 1, L.t);
+    else
+        k_batch_tick<<<1, 32, 0, s>>>(L.t);
 }
 
 template <class S>
 void launch_step_t(const StepArgs &a, bool odd, bool epi, bool plain, int block_x, int block_y, cudaStream_t s,
-                   cudaEvent_t ev_interior, cudaEvent_t ev_bulk)
+                   cudaEvent_t ev_interior, cudaEvent_t ev_bulk, const SideStream *side)
 {
     const cudaEvent_t e = ev_interior;
     const int bx = block_x, by = block_y;
+    const int eb = (int)((a.n_edge + EDGE_BLOCK - 1) / EDGE_BLOCK);
+    const int wx = (a.nx + WALL_BLOCK - 1) / WALL_BLOCK;
+    const int64_t wb = a.n_wall > 0 ? (int64_t)wx * wall_rows(a.ny, a.nz) : 0;
+    const dim3 eg((unsigned)(eb + wb));
+    const bool edges = a.n_edge > 0 || a.n_wall > 0, fork = side && edges;
+    const cudaStream_t se = fork ? side->s : s;
+    auto edge = [&]() {
+        if (!edges) return;
+        if (plain) {
+            if (odd) k_step_edge<S, true, true><<<eg, EDGE_BLOCK, 0, se>>>(a, eb, wx);
+            else     k_step_edge<S, false, true><<<eg, EDGE_BLOCK, 0, se>>>(a, eb, wx);
+        } else {
+            if (odd) k_step_edge<S, true, false><<<eg, EDGE_BLOCK, 0, se>>>(a, eb, wx);
+            else     k_step_edge<S, false, false><<<eg, EDGE_BLOCK, 0, se>>>(a, eb, wx);
+        }
+    };
+    if (fork) {
+        cudaEventRecord(side->fork, s);
+        cudaStreamWaitEvent(side->s, side->fork, 0);
+        edge();
+        cudaEventRecord(side->join, side->s);
+    }
     if (plain) {
         if (odd) { if (epi) launch_bulk<S, true, true, true>(a, bx, by, s, e); else launch_bulk<S, true, false, true>(a, bx, by, s, e); }
         else     { if (epi) launch_bulk<S, false, true, true>(a, bx, by, s, e); else launch_bulk<S, false, false, true>(a, bx, by, s, e); }
@@ -730,19 +765,8 @@ void launch_step_t(const StepArgs &a, bool odd, bool epi, bool plain, int block_
         else     { if (epi) launch_bulk<S, false, true, false>(a, bx, by, s, e); else launch_bulk<S, false, false, false>(a, bx, by, s, e); }
     }
     if (ev_bulk) cudaEventRecord(ev_bulk, s);
-    if (a.n_edge > 0 || a.n_wall > 0) {
-        const int eb = (int)((a.n_edge + EDGE_BLOCK - 1) / EDGE_BLOCK);
-        const int wx = (a.nx + WALL_BLOCK - 1) / WALL_BLOCK;
-        const int64_t wb = a.n_wall > 0 ? (int64_t)wx * wall_rows(a.ny, a.nz) : 0;
-        const dim3 eg((unsigned)(eb + wb));
-        if (plain) {
-            if (odd) k_step_edge<S, true, true><<<eg, EDGE_BLOCK, 0, s>>>(a, eb, wx);
-            else     k_step_edge<S, false, true><<<eg, EDGE_BLOCK, 0, s>>>(a, eb, wx);
-        } else {
-            if (odd) k_step_edge<S, true, false><<<eg, EDGE_BLOCK, 0, s>>>(a, eb, wx);
-            else     k_step_edge<S, false, false><<<eg, EDGE_BLOCK, 0, s>>>(a, eb, wx);
-        }
-    }
+    if (fork) cudaStreamWaitEvent(s, side->join, 0);
+    else edge();
     launch_qbb<S>(a, !odd, s);
     launch_outflow<S>(a, true, !odd, s);
 }

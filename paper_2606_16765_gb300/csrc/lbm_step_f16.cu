@@ -5,14 +5,14 @@
 
 namespace lbm {
 void launch_step_f16(const StepArgs &a, bool odd, bool epi, bool plain, int block_x, int block_y,
-                    cudaStream_t s, cudaEvent_t ev_interior, cudaEvent_t ev_bulk)
+                    cudaStream_t s, cudaEvent_t ev_interior, cudaEvent_t ev_bulk, const SideStream *side)
 {
-    launch_step_t<__half>(a, odd, epi, plain, block_x, block_y, s, ev_interior, ev_bulk);
+    launch_step_t<__half>(a, odd, epi, plain, block_x, block_y, s, ev_interior, ev_bulk, side);
 }
 
-void launch_batch_step_f16(const BatchLaunch &L, bool odd, bool epi, bool plain, cudaStream_t s)
+void launch_batch_step_f16(const BatchLaunch &L, bool odd, bool epi, bool plain, cudaStream_t s, const SideStream *side)
 {
-    launch_batch_step_t<__half>(L, odd, epi, plain, s);
+    launch_batch_step_t<__half>(L, odd, epi, plain, s, side);
 }
 
 void launch_outflow_record_f16(const StepArgs &a, bool odd, cudaStream_t s)
