@@ -21,7 +21,7 @@
 // Weight gradient: G[(tap, i)][o] = sum over cells of X[cell + tap - 1][i] *
 // GZ[cell][o]: M = 128 (tap, input-channel) rows taken as four 32-channel
 // atoms, N = output channels, K = cells.  Here both operands are MN-major: the
-// same channel-last boxes, 64-byte rows of 32 channels, consecutive cells
+// same channel-last boxes, rows of 32 or 64 channels, consecutive cells
 // the contraction index.  The cell range is split over CTAs, each adding its
 // FP32 tile into G atomically.
 //
@@ -135,13 +135,14 @@ __device__ __forceinline__ uint64_t desc_k(uint32_t addr, uint32_t row_bytes)
            ((uint64_t)1 << 46) | (mode << 61);
 }
 
-// MN-major with the 64-byte swizzle: atoms of 32 MN elements x 8 K rows
-// (512 bytes); `lbo` bytes between atoms along MN (leading field), 512 bytes
-// between 8-row groups along K (stride field).
-__device__ __forceinline__ uint64_t desc_mn64(uint32_t addr, uint32_t lbo)
+// MN-major, rows of W channels: atoms of W MN elements x 8 K rows with the 64-
+// or 128-byte swizzle (W = 32, 64); `lbo` bytes between atoms along MN (leading
+// field), an atom's 16 W bytes between 8-row groups along K (stride field).
+template <int W>
+__device__ __forceinline__ uint64_t desc_mn(uint32_t addr, uint32_t lbo)
 {
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(512 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)W << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)(W == 64 ? 2 : 4) << 61);
 }
 
 // One lane of a full warp.  The issuing loops run inside `if (elect_one())`:
@@ -427,7 +428,7 @@ __global__ void __launch_bounds__(NT, 1) k_conv_umma(const __grid_constant__ CUt
                     }
                     const uint64_t ad = desc_k(saddr(sA + (size_t)s * a.a_bytes), CK * 2);
                     const uint64_t bd = desc_k(saddr(sB + (size_t)s * a.b_bytes), CK * 2);
-    #pragma unroll
+#pragma unroll
                     for (int k = 0; k < CK / 16; ++k)          // K = 16 per product: 32 bytes along the row
                         umma(d, ad + 2 * k, bd + 2 * k, a.idesc, (q > q0 || k > 0) ? 1u : 0u);
                     commit(saddr(&c.empty[s]));
@@ -779,6 +780,11 @@ __device__ __forceinline__ WItem witem(const WgradArgs &a, int64_t w)
     return it;
 }
 
+// W: channels per copied row.  The copies go at a row every 4 to 6 cycles
+// whether it has 64 or 128 bytes, and the kernel waits for them, so channel
+// counts that are multiples of 64 take 128-byte rows (64 -> 64 channels at
+// 64x32x32, batch 8: 461 against 394 us).
+template <int W>
 __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CUtensorMap xmap,
                                                       const __grid_constant__ CUtensorMap gmap, const WgradArgs a,
                                                       float *__restrict__ g, int *status)
@@ -792,7 +798,7 @@ __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CU
     const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     ctl_init(c, S, a.tmem_cols);
     const uint32_t tmem = uniform(*c.tslot);
-    constexpr uint32_t ATOM = 128 * 64;            // 128 cells x 32 channels
+    constexpr uint32_t ATOM = 128 * W * 2;         // 128 cells x W channels
 
     if (warp == 0) {
         if (elect_one()) {
@@ -811,16 +817,16 @@ __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CU
                     }
                     const uint32_t fb = saddr(&c.full[s]);
                     mbar_expect_tx(fb, a.a_bytes + a.b_bytes);
-                    for (int at = 0; at < 4; ++at) {
-                        const int ga = wi.mt * 4 + at;
+                    for (int at = 0; at < 128 / W; ++at) {
+                        const int ga = wi.mt * (128 / W) + at;
                         // rows past 27 * cin load a valid tap and are discarded
                         const int tap = min(ga / a.cin_blocks, 26), cb = ga / a.cin_blocks > 26 ? 0 : ga % a.cin_blocks;
                         const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-                        tma5(saddr(sA + (size_t)s * a.a_bytes + at * ATOM), &xmap, cb * 32, o.x0 + dx - 1,
+                        tma5(saddr(sA + (size_t)s * a.a_bytes + at * ATOM), &xmap, cb * W, o.x0 + dx - 1,
                              o.y0 + dy - 1, o.z0 + dz - 1, o.b0, fb);
                     }
-                    for (int j = 0; j < a.ntile / 32; ++j)
-                        tma5(saddr(sB + (size_t)s * a.b_bytes + j * ATOM), &gmap, wi.nt * a.ntile + j * 32, o.x0, o.y0,
+                    for (int j = 0; j < a.ntile / W; ++j)
+                        tma5(saddr(sB + (size_t)s * a.b_bytes + j * ATOM), &gmap, wi.nt * a.ntile + j * W, o.x0, o.y0,
                              o.z0, o.b0, fb);
                     ++it;
                     r.next(S);
@@ -850,11 +856,11 @@ __global__ void __launch_bounds__(NT, 1) k_wgrad_umma(const __grid_constant__ CU
                         ok = false;
                         break;
                     }
-                    const uint64_t ad = desc_mn64(saddr(sA + (size_t)s * a.a_bytes), ATOM),
-                                   bd = desc_mn64(saddr(sB + (size_t)s * a.b_bytes), ATOM);
-    #pragma unroll
-                    for (int k = 0; k < 8; ++k)                // 16 cells (two 8-row groups, 1024 bytes) per product
-                        umma(d, ad + 64 * k, bd + 64 * k, a.idesc, (ch > wi.c0 || k > 0) ? 1u : 0u);
+                    const uint64_t ad = desc_mn<W>(saddr(sA + (size_t)s * a.a_bytes), ATOM),
+                                   bd = desc_mn<W>(saddr(sB + (size_t)s * a.b_bytes), ATOM);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)                // 16 cells (two 8-row groups) per product
+                        umma(d, ad + 2 * W * k, bd + 2 * W * k, a.idesc, (ch > wi.c0 || k > 0) ? 1u : 0u);
                     commit(saddr(&c.empty[s]));
                 }
                 if (ok) commit(saddr(&c.accf[acc]));
@@ -1169,10 +1175,13 @@ bool wgrad_plan(WgradPlan &p, const void *x, int ldx, int cin, const void *gz, i
     a.X = X; a.Y = Y; a.Z = Z; a.B = B;
     box_for(X, Y, Z, a.bx, a.by, a.bz, a.bb);
     a.tx = X / a.bx; a.ty = Y / a.by; a.tz = Z / a.bz; a.tb = (B + a.bb - 1) / a.bb;
-    a.cin_blocks = cin / 32;
+    const int W = cin % 64 == 0 && N % 64 == 0 ? 64 : 32;
+    p.w = W;
+    a.cin_blocks = cin / W;
     a.m_total = 27 * cin;
     a.mtiles = (a.m_total + 127) / 128;
     a.ntile = pick_ntile(N);
+    while (a.ntile % W || N % a.ntile) a.ntile -= 32;
     a.nntiles = N / a.ntile;
     a.nchunks = (int64_t)a.tx * a.ty * a.tz * a.tb;
     const int64_t items = (int64_t)a.mtiles * a.nntiles;
@@ -1180,8 +1189,8 @@ bool wgrad_plan(WgradPlan &p, const void *x, int ldx, int cin, const void *gz, i
     ks = std::min<int64_t>(ks, std::max<int64_t>(1, a.nchunks / 4));
     a.ksplit = (int)std::max<int64_t>(1, ks);
     a.nwork = items * a.ksplit;
-    a.a_bytes = 4u * 128 * 64;
-    a.b_bytes = (uint32_t)(a.ntile / 32) * 128 * 64;
+    a.a_bytes = 128u * 128 * 2;
+    a.b_bytes = (uint32_t)a.ntile * 128 * 2;
     a.stages = (int)std::min<size_t>(6, (SMEM_MAX - 2048 - ctl_bytes(6)) / (a.a_bytes + a.b_bytes));
     if (a.stages < 2) return bad("wgrad: tile does not fit in shared memory");
     a.idesc = idesc_for(a.ntile, true, true);
@@ -1189,15 +1198,16 @@ bool wgrad_plan(WgradPlan &p, const void *x, int ldx, int cin, const void *gz, i
     a.ldg = N;
     p.smem = std::max(SMEM_ONE_CTA, 1024 + (size_t)a.stages * (a.a_bytes + a.b_bytes) + ctl_bytes(a.stages));
     p.grid = (int)std::min<int64_t>(a.nwork, std::max(1, sms));
-    const cuuint32_t box[5] = {32, (cuuint32_t)a.bx, (cuuint32_t)a.by, (cuuint32_t)a.bz, (cuuint32_t)a.bb};
+    const CUtensorMapSwizzle sw = W == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    const cuuint32_t box[5] = {(cuuint32_t)W, (cuuint32_t)a.bx, (cuuint32_t)a.by, (cuuint32_t)a.bz, (cuuint32_t)a.bb};
     const cuuint64_t xd[5] = {(cuuint64_t)ldx, (cuuint64_t)X, (cuuint64_t)Y, (cuuint64_t)Z, (cuuint64_t)B};
     const cuuint64_t xs[4] = {(cuuint64_t)ldx * 2, (cuuint64_t)ldx * 2 * X, (cuuint64_t)ldx * 2 * X * Y,
                               (cuuint64_t)ldx * 2 * X * Y * Z};
-    if (!encode(p.xmap, 5, x, xd, xs, box, CU_TENSOR_MAP_SWIZZLE_64B)) return bad("wgrad: input tensor map rejected");
+    if (!encode(p.xmap, 5, x, xd, xs, box, sw)) return bad("wgrad: input tensor map rejected");
     const cuuint64_t gd[5] = {(cuuint64_t)ldgz, (cuuint64_t)X, (cuuint64_t)Y, (cuuint64_t)Z, (cuuint64_t)B};
     const cuuint64_t gs[4] = {(cuuint64_t)ldgz * 2, (cuuint64_t)ldgz * 2 * X, (cuuint64_t)ldgz * 2 * X * Y,
                               (cuuint64_t)ldgz * 2 * X * Y * Z};
-    if (!encode(p.gmap, 5, gz, gd, gs, box, CU_TENSOR_MAP_SWIZZLE_64B)) return bad("wgrad: gradient tensor map rejected");
+    if (!encode(p.gmap, 5, gz, gd, gs, box, sw)) return bad("wgrad: gradient tensor map rejected");
     return true;
 }
 
@@ -1206,7 +1216,8 @@ void wgrad_launch(const WgradPlan &p, float *g, int *status, cudaStream_t s)
     CUtensorMap xm, gm;
     std::memcpy(&xm, p.xmap, sizeof xm);
     std::memcpy(&gm, p.gmap, sizeof gm);
-    k_wgrad_umma<<<p.grid, NT, p.smem, s>>>(xm, gm, p.a, g, status);
+    if (p.w == 64) k_wgrad_umma<64><<<p.grid, NT, p.smem, s>>>(xm, gm, p.a, g, status);
+    else k_wgrad_umma<32><<<p.grid, NT, p.smem, s>>>(xm, gm, p.a, g, status);
 }
 
 bool gemm_set_attrs()
@@ -1223,7 +1234,8 @@ bool gemm_set_attrs()
                     cudaFuncSetAttribute(k_conv_halo<64, __nv_bfloat16>, a, v) == cudaSuccess &&
                     cudaFuncSetAttribute(k_conv_halo<32, float>, a, v) == cudaSuccess &&
                     cudaFuncSetAttribute(k_conv_halo<32, __nv_bfloat16>, a, v) == cudaSuccess &&
-                    cudaFuncSetAttribute(k_wgrad_umma, a, v) == cudaSuccess;
+                    cudaFuncSetAttribute(k_wgrad_umma<32>, a, v) == cudaSuccess &&
+                    cudaFuncSetAttribute(k_wgrad_umma<64>, a, v) == cudaSuccess;
     done = ok ? 1 : -1;
     return ok;
 }

@@ -62,7 +62,7 @@ struct WgradArgs {
     int X, Y, Z, B;
     int bx, by, bz, bb;
     int tx, ty, tz, tb;
-    int cin_blocks;              // cin / 32
+    int cin_blocks;              // cin / WgradPlan::w
     int m_total;                 // 27 * cin
     int mtiles;                  // ceil(m_total / 128)
     int ntile, nntiles;
@@ -80,6 +80,7 @@ struct WgradPlan {
     alignas(64) unsigned char xmap[128];
     alignas(64) unsigned char gmap[128];
     WgradArgs a;
+    int w = 32;                  // channels per copied row (64: 128-byte rows)
     size_t smem = 0;
     int grid = 0;
 };

@@ -42,3 +42,19 @@ def test_conv_routes_match_fp64(case):
     ex = np.abs(gx.cpu().numpy() - rgx).max() / np.abs(rgx).max()
     print(f"conv {case}: forward {ey:.2e}, input gradient {ex:.2e}")
     assert ey < _sum_tol(27 * cin) and ex < _sum_tol(27 * cout)
+
+
+@pytest.mark.parametrize("case", [(2, 4, 8, 16, 64, 64), (1, 2, 2, 4, 128, 192), (3, 4, 4, 8, 64, 320), (2, 4, 4, 8, 192, 64)])
+def test_weight_gradient_with_64_channel_rows(case):
+    """Weight gradients whose operands are copied 64 channels at a time (both
+    counts multiples of 64), tiles past the batch and channel tiles included."""
+    _need_gpu()
+    from paper_2606_16765_gb300 import unet as N
+    B, nz, ny, nx, cin, cout = case
+    x, w, g = _conv_case(sum(case), B, nz, ny, nx, cin, cout)
+    gw = torch.full((cout, cin, 27), float("nan"), device="cuda")
+    N.conv3_backward_weights(_dev(x), _dev(g), gw)
+    ref = U.conv3_backward(_first(x), _w5(w), _first(g))[1].reshape(cout, cin, 27)
+    err = np.abs(gw.cpu().numpy() - ref).max() / np.abs(ref).max()
+    print(f"weight gradient {case}: {err:.2e}")
+    assert err < _sum_tol(B * nz * ny * nx)
