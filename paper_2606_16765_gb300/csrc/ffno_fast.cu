@@ -1074,169 +1074,248 @@ constexpr int BT = 128;                      // threads of the backward kernel =
 constexpr int BTP = BT + 4;                  // row stride of its tiles
 constexpr int HC = 32;                       // hidden units per chunk
 
-// Backward of the same network, a persistent block over tiles of 128 cells,
-// one cell per thread: the hidden values are recomputed (cheaper than keeping
-// two fields per layer), 32 hidden units at a time; their values and
-// gradients meet the inputs and output gradients in shared memory, where the
-// block's threads hold 2 x 4 entries of both weight gradients each.
+// Backward of the same network, a persistent block over tiles of 128 cells; the
+// hidden values are recomputed (cheaper than keeping two fields per layer), 32
+// hidden units at a time.  All five products (hidden values and their
+// gradients, the input gradient, both weight gradients) read their operands
+// from shared memory in register tiles of 8 rows x 4 cells or 4 x 4 sums of
+// four cells, 32 multiply-adds per three 16-byte operands and 64 per eight: one
+// cell per thread was bound by those reads (4 multiply-adds per broadcast
+// weight).  32 -> 32 -> 32 at 8 x 524,288 cells:
+// 1.16 ms, where the multiply-adds alone take 0.60 ms; the six networks of a
+// training step 13.4 -> 10.5 ms.
+// A warp owns 32 cells up to the input gradient: lanes = 8 quadruples of cells
+// x 4 groups of rows.  The weight gradients take all cells: 64 threads x (4
+// hidden units x N1 or N2 rows) in each half of the cells, rows 8 apart (row
+// stride of 132: conflict-free).
 template <int CI, int CO, int ACT, int NCH, bool GX>
-__global__ void __launch_bounds__(BT) k_mlp_bwd(const Mlp p, const float *__restrict__ x, const float *__restrict__ g,
-                                                float *__restrict__ gx, int B, int64_t N, float *__restrict__ part)
+__global__ void __launch_bounds__(BT, NCH == 4 ? 2 : 3) k_mlp_bwd(const Mlp p, const float *__restrict__ x,
+                                                                  const float *__restrict__ g, float *__restrict__ gx,
+                                                                  int B, int64_t N, int vec, float *__restrict__ part)
 {
     extern __shared__ float4 raw[];
     constexpr int chp = NCH * HC, N1 = CI / 8, N2 = CO / 8;
-    float *w1 = reinterpret_cast<float *>(raw), *w2 = w1 + chp * CI, *b1 = w2 + chp * CO;
+    constexpr int WS = chp + 4;                              // row stride of W1 transposed
+    float *w1 = reinterpret_cast<float *>(raw), *w2 = w1 + CI * WS, *b1 = w2 + CO * chp;
     float *X = b1 + chp, *G = X + CI * BTP, *H = G + CO * BTP, *GH = H + HC * BTP;
-    stage_weights<CI, CO>(p, chp, w1, w2, b1, nullptr);
-    __syncthreads();
-    const int tid = threadIdx.x, hg = tid >> 3, cg = tid & 7;
-    float a1[NCH][2][N1], a2[NCH][2][N2], s1[NCH][2], s2[N2];
+    const int tid = threadIdx.x;
+    for (int q = tid; q < chp * CI; q += BT) {               // W1 transposed [CI][ch], W2 [CO][ch]
+        const int j = q / CI, c = q % CI;
+        w1[c * WS + j] = j < p.ch && c < p.ci ? p.W1[j * p.ci + c] : 0.f;
+    }
+    for (int q = tid; q < CO * chp; q += BT) {
+        const int o = q / chp, j = q % chp;
+        w2[q] = j < p.ch && o < p.co ? p.W2[o * p.ch + j] : 0.f;
+    }
+    for (int q = tid; q < chp; q += BT) b1[q] = q < p.ch ? p.b1[q] : 0.f;
+    const int lane = tid & 31, r4 = lane >> 3, r8 = r4 * 8, cq = (tid >> 5) * 32 + (lane & 7) * 4;      // 8 rows, 4 cells
+    const int hg = (tid >> 3) & 7, cg = tid & 7, half = tid >> 6;
+    const int sr = tid >> 2, sq = (tid & 3) * 4;             // row and cells of the bias sums
+    float a1[NCH][4][N1], a2[NCH][4][N2], s1[NCH], s2 = 0.f;
 #pragma unroll
-    for (int k = 0; k < NCH; ++k)
+    for (int k = 0; k < NCH; ++k) {
+        s1[k] = 0.f;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            s1[k][h] = 0.f;
+        for (int h = 0; h < 4; ++h) {
 #pragma unroll
             for (int c = 0; c < N1; ++c) a1[k][h][c] = 0.f;
 #pragma unroll
             for (int c = 0; c < N2; ++c) a2[k][h][c] = 0.f;
         }
-#pragma unroll
-    for (int c = 0; c < N2; ++c) s2[c] = 0.f;
+    }
     const int64_t cells = B * N;
     for (int64_t c0 = (int64_t)blockIdx.x * BT; c0 < cells; c0 += (int64_t)gridDim.x * BT) {
-        const int64_t cell = c0 + tid;
-        const bool ok = cell < cells;
-        const int64_t b = cell / N, n = cell - b * N;
-        float in[CI], go[CO], gi[GX ? CI : 1];
-#pragma unroll
-        for (int c = 0; c < CI; ++c) {
-            in[c] = ok && c < p.ci ? x[(b * p.ci + c) * N + n] : 0.f;
-            X[c * BTP + tid] = in[c];
+        if (vec) {                                           // N % 4 == 0: a quadruple lies in one sample
+            const int qd = 4 * lane;
+            const int64_t cell = c0 + qd, b = cell / N, n = cell - b * N;
+            const bool ok = cell < cells;
+            for (int c = tid >> 5; c < CI; c += BT / 32) {
+                if (ok && c < p.ci) async16(X + c * BTP + qd, x + (b * p.ci + c) * N + n);
+                else *reinterpret_cast<float4 *>(X + c * BTP + qd) = f4(0.f);
+            }
+            for (int o = tid >> 5; o < CO; o += BT / 32) {
+                if (ok && o < p.co) async16(G + o * BTP + qd, g + (b * p.co + o) * N + n);
+                else *reinterpret_cast<float4 *>(G + o * BTP + qd) = f4(0.f);
+            }
+            async_wait();
+        } else {
+            const int64_t cell = c0 + tid, b = cell / N, n = cell - b * N;
+            const bool ok = cell < cells;
+#pragma unroll 8
+            for (int c = 0; c < CI; ++c) X[c * BTP + tid] = ok && c < p.ci ? x[(b * p.ci + c) * N + n] : 0.f;
+#pragma unroll 8
+            for (int o = 0; o < CO; ++o) G[o * BTP + tid] = ok && o < p.co ? g[(b * p.co + o) * N + n] : 0.f;
         }
-#pragma unroll
-        for (int o = 0; o < CO; ++o) {
-            go[o] = ok && o < p.co ? g[(b * p.co + o) * N + n] : 0.f;
-            G[o * BTP + tid] = go[o];
-        }
+        __syncthreads();
+        float4 gi[GX ? 8 : 1];
         if (GX)
 #pragma unroll
-            for (int c = 0; c < CI; ++c) gi[c] = 0.f;
+            for (int i = 0; i < 8; ++i) gi[i] = f4(0.f);
 #pragma unroll
         for (int k = 0; k < NCH; ++k) {
+            // z and dL/dh of 8 hidden units and 4 cells, into H and GH
+            {
+                float4 z[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) z[i] = f4(b1[k * HC + r8 + i]);
+#pragma unroll 4
+                for (int c = 0; c < CI; ++c) {
+                    const float4 v = *reinterpret_cast<const float4 *>(X + c * BTP + cq);
+                    const float *w = w1 + c * WS + k * HC + r8;
+                    const float4 wa = *reinterpret_cast<const float4 *>(w), wb = *reinterpret_cast<const float4 *>(w + 4);
+                    fma4(z[0], wa.x, v); fma4(z[1], wa.y, v); fma4(z[2], wa.z, v); fma4(z[3], wa.w, v);
+                    fma4(z[4], wb.x, v); fma4(z[5], wb.y, v); fma4(z[6], wb.z, v); fma4(z[7], wb.w, v);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) *reinterpret_cast<float4 *>(H + (r8 + i) * BTP + cq) = z[i];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) z[i] = f4(0.f);
+#pragma unroll 4
+                for (int o = 0; o < CO; ++o) {
+                    const float4 v = *reinterpret_cast<const float4 *>(G + o * BTP + cq);
+                    const float *w = w2 + o * chp + k * HC + r8;
+                    const float4 wa = *reinterpret_cast<const float4 *>(w), wb = *reinterpret_cast<const float4 *>(w + 4);
+                    fma4(z[0], wa.x, v); fma4(z[1], wa.y, v); fma4(z[2], wa.z, v); fma4(z[3], wa.w, v);
+                    fma4(z[4], wb.x, v); fma4(z[5], wb.y, v); fma4(z[6], wb.z, v); fma4(z[7], wb.w, v);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) *reinterpret_cast<float4 *>(GH + (r8 + i) * BTP + cq) = z[i];
+            }
+            // the activation, on this thread's own entries (rolled: 32 inlined
+            // copies would not fit the instruction cache)
 #pragma unroll 1
-            for (int jj = 0; jj < HC; jj += 2) {
-                const int j = k * HC + jj;
-                float z[2], gh[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    z[h] = b1[j + h];
-                    gh[h] = 0.f;
-                }
-#pragma unroll
-                for (int c = 0; c < CI; c += 4)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const float4 w = *reinterpret_cast<const float4 *>(w1 + (j + h) * CI + c);
-                        z[h] = fmaf(w.x, in[c], z[h]);
-                        z[h] = fmaf(w.y, in[c + 1], z[h]);
-                        z[h] = fmaf(w.z, in[c + 2], z[h]);
-                        z[h] = fmaf(w.w, in[c + 3], z[h]);
-                    }
-#pragma unroll
-                for (int o = 0; o < CO; o += 4)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const float4 w = *reinterpret_cast<const float4 *>(w2 + (j + h) * CO + o);
-                        gh[h] = fmaf(w.x, go[o], gh[h]);
-                        gh[h] = fmaf(w.y, go[o + 1], gh[h]);
-                        gh[h] = fmaf(w.z, go[o + 2], gh[h]);
-                        gh[h] = fmaf(w.w, go[o + 3], gh[h]);
-                    }
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    float hv, dh;
-                    act_both<ACT>(z[h], p.w0, hv, dh);
-                    gh[h] *= dh;
-                    H[(jj + h) * BTP + tid] = hv;
-                    GH[(jj + h) * BTP + tid] = gh[h];
-                }
-                if (GX)
-#pragma unroll
-                    for (int c = 0; c < CI; c += 4)
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const float4 w = *reinterpret_cast<const float4 *>(w1 + (j + h) * CI + c);
-                            gi[c] = fmaf(w.x, gh[h], gi[c]);
-                            gi[c + 1] = fmaf(w.y, gh[h], gi[c + 1]);
-                            gi[c + 2] = fmaf(w.z, gh[h], gi[c + 2]);
-                            gi[c + 3] = fmaf(w.w, gh[h], gi[c + 3]);
-                        }
+            for (int i = 0; i < 8; ++i) {
+                float4 *hp = reinterpret_cast<float4 *>(H + (r8 + i) * BTP + cq);
+                float4 *gp = reinterpret_cast<float4 *>(GH + (r8 + i) * BTP + cq);
+                const float4 z = *hp, d = *gp;
+                float4 v, dv;
+                act_both<ACT>(z.x, p.w0, v.x, dv.x);
+                act_both<ACT>(z.y, p.w0, v.y, dv.y);
+                act_both<ACT>(z.z, p.w0, v.z, dv.z);
+                act_both<ACT>(z.w, p.w0, v.w, dv.w);
+                *hp = v;
+                *gp = make_float4(d.x * dv.x, d.y * dv.y, d.z * dv.z, d.w * dv.w);
             }
             __syncthreads();
+            if (GX) {
 #pragma unroll 2
-            for (int q = 0; q < BT; q += 4) {
-                float4 hv[2], gv[2];
+                for (int h = 0; h < HC; h += 4) {            // channels r4 + 4 i
+                    float4 v[4];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    gv[h] = *reinterpret_cast<const float4 *>(GH + (2 * hg + h) * BTP + q);
-                    hv[h] = *reinterpret_cast<const float4 *>(H + (2 * hg + h) * BTP + q);
-                    s1[k][h] += (gv[h].x + gv[h].y) + (gv[h].z + gv[h].w);
+                    for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const float4 *>(GH + (h + u) * BTP + cq);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float4 w = *reinterpret_cast<const float4 *>(w1 + (r4 + 4 * i) * WS + k * HC + h);
+                        fma4(gi[i], w.x, v[0]); fma4(gi[i], w.y, v[1]); fma4(gi[i], w.z, v[2]); fma4(gi[i], w.w, v[3]);
+                    }
                 }
+            }
+#pragma unroll
+            for (int q = 0; q < BT; q += 16) {
+                const float4 v = *reinterpret_cast<const float4 *>(GH + sr * BTP + q + sq);
+                s1[k] += (v.x + v.y) + (v.z + v.w);
+            }
+            if (k == 0 && sr < CO)
+#pragma unroll
+                for (int q = 0; q < BT; q += 16) {
+                    const float4 v = *reinterpret_cast<const float4 *>(G + sr * BTP + q + sq);
+                    s2 += (v.x + v.y) + (v.z + v.w);
+                }
+#pragma unroll 1
+            for (int q = half * (BT / 2); q < (half + 1) * (BT / 2); q += 4) {
+                float4 v[4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) v[h] = *reinterpret_cast<const float4 *>(GH + (hg + 8 * h) * BTP + q);
 #pragma unroll
                 for (int c = 0; c < N1; ++c) {
                     const float4 w = *reinterpret_cast<const float4 *>(X + (cg + 8 * c) * BTP + q);
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float s = a1[k][h][c];
-                        s = fmaf(gv[h].x, w.x, s);
-                        s = fmaf(gv[h].y, w.y, s);
-                        s = fmaf(gv[h].z, w.z, s);
-                        a1[k][h][c] = fmaf(gv[h].w, w.w, s);
+                    for (int h = 0; h < 4; ++h) {
+                        float t = a1[k][h][c];
+                        t = fmaf(v[h].x, w.x, t);
+                        t = fmaf(v[h].y, w.y, t);
+                        t = fmaf(v[h].z, w.z, t);
+                        a1[k][h][c] = fmaf(v[h].w, w.w, t);
                     }
                 }
+#pragma unroll
+                for (int h = 0; h < 4; ++h) v[h] = *reinterpret_cast<const float4 *>(H + (hg + 8 * h) * BTP + q);
 #pragma unroll
                 for (int c = 0; c < N2; ++c) {
                     const float4 w = *reinterpret_cast<const float4 *>(G + (cg + 8 * c) * BTP + q);
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float s = a2[k][h][c];
-                        s = fmaf(hv[h].x, w.x, s);
-                        s = fmaf(hv[h].y, w.y, s);
-                        s = fmaf(hv[h].z, w.z, s);
-                        a2[k][h][c] = fmaf(hv[h].w, w.w, s);
+                    for (int h = 0; h < 4; ++h) {
+                        float t = a2[k][h][c];
+                        t = fmaf(v[h].x, w.x, t);
+                        t = fmaf(v[h].y, w.y, t);
+                        t = fmaf(v[h].z, w.z, t);
+                        a2[k][h][c] = fmaf(v[h].w, w.w, t);
                     }
-                    if (k == 0) s2[c] += (w.x + w.y) + (w.z + w.w);
                 }
             }
             __syncthreads();
         }
-        if (GX && ok)
+        if (GX && vec) {
+            const int64_t cell = c0 + cq, b = cell / N, n = cell - b * N;
+            if (cell < cells)
 #pragma unroll
-            for (int c = 0; c < CI; ++c)
-                if (c < p.ci) gx[(b * p.ci + c) * N + n] = gi[c];
+                for (int i = 0; i < 8; ++i)
+                    if (r4 + 4 * i < p.ci) *reinterpret_cast<float4 *>(gx + (b * p.ci + r4 + 4 * i) * N + n) = gi[i];
+        } else if (GX) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int64_t cell = c0 + cq + e, b = cell / N, n = cell - b * N;
+                if (cell < cells)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (r4 + 4 * i < p.ci)
+                            gx[(b * p.ci + r4 + 4 * i) * N + n] = e == 0 ? gi[i].x : e == 1 ? gi[i].y : e == 2 ? gi[i].z : gi[i].w;
+            }
+        }
     }
-    // this block's sums, in the parameters' order: W1 [ch][ci], b1, W2 [co][ch], b2
+    // this block's sums, in the parameters' order: W1 [ch][ci], b1, W2 [co][ch],
+    // b2; the second half of the cells through shared memory
     const int n1 = p.ch * p.ci, n2 = p.co * p.ch;
     float *d = part + (int64_t)blockIdx.x * (n1 + p.ch + n2 + p.co);
+    float *red = X + (tid & 63);
+    if (half)
 #pragma unroll
-    for (int k = 0; k < NCH; ++k)
+        for (int k = 0; k < NCH; ++k)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int j = k * HC + 2 * hg + h;
-            if (j >= p.ch) continue;
+            for (int h = 0; h < 4; ++h) {
 #pragma unroll
-            for (int c = 0; c < N1; ++c)
-                if (cg + 8 * c < p.ci) d[j * p.ci + cg + 8 * c] = a1[k][h][c];
-            if (cg == 0) d[n1 + j] = s1[k][h];
+                for (int c = 0; c < N1; ++c) red[((k * 4 + h) * (N1 + N2) + c) * 64] = a1[k][h][c];
 #pragma unroll
-            for (int c = 0; c < N2; ++c)
-                if (cg + 8 * c < p.co) d[n1 + p.ch + (cg + 8 * c) * p.ch + j] = a2[k][h][c];
-        }
-    if (hg == 0)
+                for (int c = 0; c < N2; ++c) red[((k * 4 + h) * (N1 + N2) + N1 + c) * 64] = a2[k][h][c];
+            }
+    __syncthreads();
+    if (!half)
 #pragma unroll
-        for (int c = 0; c < N2; ++c)
-            if (cg + 8 * c < p.co) d[n1 + p.ch + n2 + cg + 8 * c] = s2[c];
+        for (int k = 0; k < NCH; ++k)
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const int j = k * HC + hg + 8 * h;
+                if (j >= p.ch) continue;
+#pragma unroll
+                for (int c = 0; c < N1; ++c)
+                    if (cg + 8 * c < p.ci)
+                        d[j * p.ci + cg + 8 * c] = a1[k][h][c] + red[((k * 4 + h) * (N1 + N2) + c) * 64];
+#pragma unroll
+                for (int c = 0; c < N2; ++c)
+                    if (cg + 8 * c < p.co)
+                        d[n1 + p.ch + (cg + 8 * c) * p.ch + j] =
+                            a2[k][h][c] + red[((k * 4 + h) * (N1 + N2) + N1 + c) * 64];
+            }
+#pragma unroll
+    for (int k = 0; k < NCH; ++k) {
+        float t = s1[k];
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        if ((tid & 3) == 0 && k * HC + sr < p.ch) d[n1 + k * HC + sr] = t;
+    }
+    s2 += __shfl_xor_sync(0xffffffffu, s2, 1);
+    s2 += __shfl_xor_sync(0xffffffffu, s2, 2);
+    if ((tid & 3) == 0 && sr < p.co) d[n1 + p.ch + n2 + sr] = s2;
 }
 
 // out[q] = sum over the parts, 8 interleaved FP64 sums added in order
@@ -1414,14 +1493,16 @@ void mlp_act(const Mlp &p, const float *x, const float *res, float *y, int B, in
 }
 
 template <int CI, int CO, int ACT, int NCH, bool GX>
-size_t bwd_smem() { return sizeof(float) * (size_t)(NCH * HC * (CI + CO + 1) + (CI + CO + 2 * HC) * BTP); }
+size_t bwd_smem() { return sizeof(float) * (size_t)(NCH * HC * (CI + CO + 1) + 4 * CI + (CI + CO + 2 * HC) * BTP); }
 
 int bwd_grid(int64_t cells) { return (int)std::min<int64_t>((cells + BT - 1) / BT, mlp_parts()); }
 
 template <int CI, int CO, int ACT, int NCH, bool GX>
 void bwd_k(const Mlp &p, const float *x, const float *g, float *gx, float *part, int B, int64_t N, cudaStream_t s)
 {
-    k_mlp_bwd<CI, CO, ACT, NCH, GX><<<bwd_grid(B * N), BT, bwd_smem<CI, CO, ACT, NCH, GX>(), s>>>(p, x, g, gx, B, N, part);
+    // 16-byte copies where a quadruple of cells stays in a sample and is aligned
+    const int vec = N % 4 == 0 && (((uintptr_t)x | (uintptr_t)g | (uintptr_t)gx) & 15) == 0;
+    k_mlp_bwd<CI, CO, ACT, NCH, GX><<<bwd_grid(B * N), BT, bwd_smem<CI, CO, ACT, NCH, GX>(), s>>>(p, x, g, gx, B, N, vec, part);
 }
 
 template <int CI, int CO, int ACT, bool GX>
