@@ -21,8 +21,8 @@
  * F1_b, F2_w [width][ff_hidden], F2_b; then Q1_w [hidden][width], Q1_b,
  * Q2_w [cout][hidden], Q2_b.
  *
- * This first GPU path computes in FP32 with one thread per output element
- * (transforms as explicit sums against twiddle tables).  Conventions as in
+ * Everything is computed in FP32.  Widths up to 32 with hidden widths up to
+ * 128 run on tiled kernels, others on general ones.  Conventions as in
  * lbm.h: every call returns lbm_status; x, t, m and y may be host or device
  * memory; work runs on the stream given at creation.
  */

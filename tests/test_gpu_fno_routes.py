@@ -59,7 +59,7 @@ def test_pointwise_input_gradients(grid, hidden):
                                                  (16, 5, (2, 8, 16), 32, 3), (32, 4, (2, 4, 16), 32, 1),
                                                  (5, 5, (2, 2, 16), 3, 1), (7, 5, (2, 2, 16), 32, 3)])
 def test_tensor_core_stages(ny, nz, modes, width, B):
-    y, yr, g, gr = _run(128, ny, nz, modes, width, 128, 32, B, act_bf16=1, tensor_cores=1)
+    y, yr, g, gr = _run(128, ny, nz, modes, width, 128, 32, B, act_bf16=1, tensor_cores=int(width % 8 == 0))
     worst = max(rel_l2(g[k], gr[k]) for k in gr)
     print(f"FNO 128x{ny}x{nz}, width {width}: forward {rel_l2(y, yr):.2e}, worst gradient group {worst:.2e}")
     assert rel_l2(y, yr) < 2e-2
