@@ -1095,14 +1095,15 @@ constexpr int HC = 32;                       // hidden units per chunk
 // four cells, 32 multiply-adds per three 16-byte operands and 64 per eight: one
 // cell per thread was bound by those reads (4 multiply-adds per broadcast
 // weight).  32 -> 32 -> 32 at 8 x 524,288 cells:
-// 1.16 ms, where the multiply-adds alone take 0.60 ms; the six networks of a
-// training step 13.4 -> 10.5 ms.
+// 1.16 ms, where the multiply-adds alone take 0.60 ms; 32 -> 128 -> 4: 3.63 ms
+// (three blocks per SM with some spills; two without: 5.10); the six networks
+// of a training step 13.4 -> 9.1 ms.
 // A warp owns 32 cells up to the input gradient: lanes = 8 quadruples of cells
 // x 4 groups of rows.  The weight gradients take all cells: 64 threads x (4
 // hidden units x N1 or N2 rows) in each half of the cells, rows 8 apart (row
 // stride of 132: conflict-free).
 template <int CI, int CO, int ACT, int NCH, bool GX>
-__global__ void __launch_bounds__(BT, NCH == 4 ? 2 : 3) k_mlp_bwd(const Mlp p, const float *__restrict__ x,
+__global__ void __launch_bounds__(BT, NCH == 4 && CO > 8 ? 2 : 3) k_mlp_bwd(const Mlp p, const float *__restrict__ x,
                                                                   const float *__restrict__ g, float *__restrict__ gx,
                                                                   int B, int64_t N, int vec, float *__restrict__ part)
 {
