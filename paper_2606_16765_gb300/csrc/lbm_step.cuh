@@ -419,6 +419,8 @@ __global__ void __launch_bounds__(EDGE_BLOCK) k_step_edge(StepArgs a, int eblock
 // gather never reads.
 // All loads of a link are issued before any is used (the flags decide which
 // values count, not which are read): one latency instead of five in a row.
+// Only the step's parity leaves some out: each costs a sector of its own on
+// this strided plane, which many large outlets feel.
 template <class S>
 __device__ __forceinline__ void outflow_link(const StepArgs &a, uint32_t yz, int k, bool fix, bool next_odd)
 {
@@ -438,9 +440,9 @@ __device__ __forceinline__ void outflow_link(const StepArgs &a, uint32_t yz, int
     // the inner cell's source (nx - 1, y - cy, z - cz)
     const int64_t s2 = (int64_t)(a.nx - 1) + (int64_t)a.nx * ((int64_t)sy + (int64_t)a.ny * sz);
     const int64_t ci = a.nx >= 2 ? c - 1 : c;
-    const uint8_t flag_c = a.flags[c], flag_in = a.flags[ci], flag_s = a.flags[s2];
+    const uint8_t flag_c = a.flags[c], flag_in = a.flags[ci], flag_s = next_odd ? a.flags[s2] : (uint8_t)CELL_SOLID;
     const R was_own = *own, was_in = *in, here = T::ld(p + (int64_t)i * a.slot + c);
-    const R there = T::ld(p + (int64_t)i * a.slot + ci), across = T::ld(p + (int64_t)(Q - 1 - i) * a.slot + s2);
+    const R there = T::ld(p + (int64_t)i * a.slot + ci), across = next_odd ? T::ld(p + (int64_t)(Q - 1 - i) * a.slot + s2) : R(0);
     if (flag_c & CELL_SOLID) return;
     const bool inner = a.nx >= 2 && !(flag_in & CELL_SOLID);
     R mine = here;
