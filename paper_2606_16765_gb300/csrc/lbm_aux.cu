@@ -281,12 +281,17 @@ __global__ void k_set(S *pdf, int64_t slot, const uint8_t *flags, int64_t n, con
 // (ux, uy, uz, p), rho = 1 + 3 p: f_i = rho phi(cx, ux) phi(cy, uy) phi(cz, uz)
 // with phi(0, u) = 2/3 - u^2 and phi(+-1, u) = (1/3 + u^2 +- u)/2 (the
 // equilibrium whose cumulants above second order vanish); stored shifted,
-// solid cells at rest.  Evaluated to twice the precision of the result: FP64
-// for FP64 storage, for the others pairs of floats (an unevaluated sum, about
-// 46 bits; products by fused multiply-add, sums by Knuth's two-sum), because
-// the FP64 pipe is the slowest of this chip: 432 FP64 operations per cell took
-// 25.9 ms on 512x256x256 FP16 cells and 3.25 ms on 256x128x128 FP32 cells, the
-// pairs 0.9 and 0.11 ms (reads and stores alone: 0.35 and 0.08 ms).
+// solid cells at rest.  FP64 storage evaluates f_i - w_i in FP64.  The others
+// take pairs of floats (an unevaluated sum, about 46 bits; products by fused
+// multiply-add, sums by Knuth's two-sum) and build f_i - w_i from the small
+// terms alone: with phi(c, u) = t(c) + d(c, u) and rho = 1 + r, each factor adds
+// its part of the deviation, so that w_i is never subtracted and what is stored
+// is good to its last bit however close to rest the field is (relative L2 error
+// of FP32 deviations 2.4e-8 to 2.6e-8 for velocities from 1e-25 to 15; FP64
+// minus w_i: the same down to 1e-7, 1.3e-7 at 1e-9, 1.3e-6 at 1e-10).  The FP64
+// pipe is the slowest of this chip: 432 FP64 operations per cell took 25.9 ms
+// on 512x256x256 FP16 cells and 3.25 ms on 256x128x128 FP32 cells, the pairs
+// 1.02 and 0.13 ms (reads and stores alone: 0.35 and 0.08 ms).
 __device__ __forceinline__ double eq_phi(int c, double u)
 {
     return c == 0 ? 2.0 / 3.0 - u * u : 0.5 * (1.0 / 3.0 + u * u + c * u);
@@ -333,14 +338,23 @@ __device__ __forceinline__ Pair operator+(Pair a, Pair b)
     return renorm(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
 }
 
-// phi(-1, u), phi(0, u), phi(1, u)
-__device__ __forceinline__ void eq_phi3(float u, Pair *p)
+// a b + c rounded once to FP32 (nothing normalised in between)
+__device__ __forceinline__ float mul_add(Pair a, Pair b, Pair c)
 {
-    const Pair u2 = two_prod(u, u), t = pair_const(1.0 / 3.0) + u2;
-    const Pair a = t + Pair{-u, 0.f}, b = t + Pair{u, 0.f};
-    p[0] = Pair{0.5f * a.h, 0.5f * a.l};
-    p[1] = pair_const(2.0 / 3.0) + Pair{-u2.h, -u2.l};
-    p[2] = Pair{0.5f * b.h, 0.5f * b.l};
+    const Pair p = two_prod(a.h, b.h), s = two_sum(p.h, c.h);
+    const float l = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, p.l));
+    return __fadd_rn(s.h, __fadd_rn(s.l, __fadd_rn(l, c.l)));
+}
+
+__device__ __forceinline__ Pair scaled(float k, Pair a) { return Pair{k * a.h, k * a.l}; }     // k a power of two
+
+// d(c, u) = phi(c, u) - t(c) for c = -1, 0, 1
+__device__ __forceinline__ void eq_small3(float u, Pair *d)
+{
+    const Pair u2 = two_prod(u, u);
+    d[0] = scaled(0.5f, u2 + Pair{-u, 0.f});
+    d[1] = Pair{-u2.h, -u2.l};
+    d[2] = scaled(0.5f, u2 + Pair{u, 0.f});
 }
 
 template <class S>
@@ -373,22 +387,29 @@ __global__ void k_equilibrium(S *pdf, int64_t slot, const uint8_t *flags, int64_
             equilibrium_f64<S>(pdf + c, slot, v, solid);
             continue;
         }
-        Pair px[3], py[3], pz[3];
-        eq_phi3(v.x, px);
-        eq_phi3(v.y, py);
-        eq_phi3(v.z, pz);
-        const Pair rho = two_prod(3.f, v.w) + Pair{1.f, 0.f};
+        // deviations after one, two and three factors: (b + e)(t + d) - b t =
+        // e (t + d) + b d, where b t is a power of two times 1/6 or 1/36
+        Pair dx[3], dy[3], dz[3], ey[3], ez[3];
+        eq_small3(v.x, dx);
+        eq_small3(v.y, dy);
+        eq_small3(v.z, dz);
+        const Pair r = two_prod(3.f, v.w);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            ey[k] = pair_const(1.0 / 6.0) * dy[k];
+            ez[k] = pair_const(1.0 / 36.0) * dz[k];
+        }
 #pragma unroll
         for (int x = 0; x < 3; ++x) {
-            const Pair a = rho * px[x];
+            const Pair a = dx[x] + r * (pair_const(tw(x)) + dx[x]);
 #pragma unroll
             for (int y = 0; y < 3; ++y) {
-                const Pair b = a * py[y];
+                const Pair b = a * (pair_const(tw(y)) + dy[y]) + scaled(x == 1 ? 4.f : 1.f, ey[y]);
 #pragma unroll
                 for (int z = 0; z < 3; ++z) {
-                    const int i = x + 3 * y + 9 * z;
-                    const Pair f = b * pz[z], w = pair_const(w_of(i)), d = two_sum(f.h, -w.h);
-                    T::st(pdf + i * slot + c, (typename T::R)(solid ? 0.f : d.h + (d.l + (f.l - w.l))));
+                    const float f = mul_add(b, pair_const(tw(z)) + dz[z],
+                                            scaled((x == 1 ? 4.f : 1.f) * (y == 1 ? 4.f : 1.f), ez[z]));
+                    T::st(pdf + (x + 3 * y + 9 * z) * slot + c, (typename T::R)(solid ? 0.f : f));
                 }
             }
         }
