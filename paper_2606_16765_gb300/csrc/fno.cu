@@ -2408,15 +2408,21 @@ size_t smem_dfty_inv(const Dims &d)
     return sizeof(float2) * ((size_t)d.Ky * nyp + (size_t)dfty_inv_slabs(d) * d.Ky * d.Kx);
 }
 
-bool set_smem_limits(size_t bytes)
+// most dynamic shared memory of the kernels whose size follows the grid and the modes
+constexpr size_t SMEM_LIMIT = 160 * 1024;
+
+bool set_smem_limits()
 {
-    const int b = (int)bytes;
+    const int b = (int)SMEM_LIMIT;
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     return cudaFuncSetAttribute(k_dftx_fwd<float>, a, b) == cudaSuccess &&
            cudaFuncSetAttribute(k_dftx_fwd<__nv_bfloat16>, a, b) == cudaSuccess &&
            cudaFuncSetAttribute(k_dftx_inv<float>, a, b) == cudaSuccess &&
            cudaFuncSetAttribute(k_dftx_inv<__nv_bfloat16>, a, b) == cudaSuccess &&
            cudaFuncSetAttribute(k_dfty_fwd, a, b) == cudaSuccess && cudaFuncSetAttribute(k_dfty_inv, a, b) == cudaSuccess &&
+           cudaFuncSetAttribute(k_cdft_tc<4, 4>, a, b) == cudaSuccess &&
+           cudaFuncSetAttribute(k_cdft_tc<4, 2>, a, b) == cudaSuccess &&
+           cudaFuncSetAttribute(k_cdft_tc<4, 1>, a, b) == cudaSuccess &&
            cudaFuncSetAttribute(k_outer<float, 1>, a, b) == cudaSuccess &&
            cudaFuncSetAttribute(k_outer<float, 2>, a, b) == cudaSuccess &&
            cudaFuncSetAttribute(k_outer<__nv_bfloat16, 1>, a, b) == cudaSuccess &&
@@ -2551,7 +2557,7 @@ extern "C" lbm_status fno_create(const fno_config *cfg, void *stream, fno_ctx **
     if (c.tensor_cores && c.width % 8 != 0) return bad("tensor-core contraction needs width % 8 == 0");
     if (2 * c.mx > 256) return bad("2mx must be <= 256");
     const Dims d0{c.nx, c.ny, c.nz, 2 * c.mx, 2 * c.my, c.mz, 1};
-    const size_t sm_max = 160 * 1024;
+    const size_t sm_max = SMEM_LIMIT;
     if (smem_dftx_fwd(d0) > sm_max || smem_dftx_inv(d0) > sm_max || smem_dfty_fwd(d0) > sm_max ||
         smem_dfty_inv(d0) > sm_max)
         return bad("grid x modes too large for the shared-memory twiddle tables");
@@ -2561,7 +2567,7 @@ extern "C" lbm_status fno_create(const fno_config *cfg, void *stream, fno_ctx **
         return bad("layer too wide for the gradient reduction");
     if (smem_outer(c.hidden, c.width) > sm_max || smem_outer(c.cout, c.hidden) > sm_max)
         return bad("layer too wide for the gradient reduction tiles");
-    if (!set_smem_limits(sm_max)) return bad("cannot raise the shared-memory limit of the FNO kernels");
+    if (!set_smem_limits()) return bad("cannot raise the shared-memory limit of the FNO kernels");
     fno_ctx *f = new fno_ctx();
     f->c = c;
     f->s = static_cast<cudaStream_t>(stream);
@@ -2836,13 +2842,15 @@ void outer(fno_ctx *f, const float *g, int co, const T *x, int ci, int64_t oW, i
     }
 }
 
+size_t smem_cdft(const Dims &d) { return 2 * sizeof(uint4) * (size_t)(d.Ky / 8) * (d.ny / 8) * 32; }
 // the y stages on tensor cores: BF16-activation configuration, whole
-// m-tiles and k-steps of eight modes or rows, 32 x modes
+// m-tiles and k-steps of eight modes or rows, 32 x modes, and twiddle
+// fragments that fit shared memory (16 bytes per mode and row: 128 rows up to
+// 80 modes; the others take k_dfty_fwd and k_dfty_inv, half as much)
 bool ydft_tc(const fno_ctx *f, const Dims &d)
 {
-    return f->c.act_bf16 && d.ny % 8 == 0 && d.Ky % 8 == 0 && d.Kx == 32;
+    return f->c.act_bf16 && d.ny % 8 == 0 && d.Ky % 8 == 0 && d.Kx == 32 && smem_cdft(d) <= SMEM_LIMIT;
 }
-size_t smem_cdft(const Dims &d) { return 2 * sizeof(uint4) * (size_t)(d.Ky / 8) * (d.ny / 8) * 32; }
 
 void cdft_tc(const Dims &d, const float2 *X, float2 *Y, const float2 *tw, int inv, int64_t S, cudaStream_t s)
 {
