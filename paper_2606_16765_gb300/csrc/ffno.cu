@@ -408,6 +408,15 @@ lbm_status alloc(ffno_ctx *f, T *&p, int64_t count)
     return LBM_OK;
 }
 
+// Host data onto the context's own stream, there when this returns: a plain
+// cudaMemcpy goes through the default stream, may return before its last part
+// has landed, and orders nothing for a stream created non-blocking.
+bool upload(const ffno_ctx *f, void *dst, const void *src, size_t bytes)
+{
+    return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, f->s) == cudaSuccess &&
+           cudaStreamSynchronize(f->s) == cudaSuccess;
+}
+
 uint64_t splitmix(uint64_t &s)
 {
     uint64_t z = (s += 0x9E3779B97F4A7C15ull);
@@ -577,9 +586,9 @@ extern "C" lbm_status ffno_create(const ffno_config *cfg, void *stream, ffno_ctx
             const double cw = (k == 0 || (Ld % 2 == 0 && k == Ld / 2)) ? 1.0 : 2.0;
             ck[k] = (float)(cw / Ld);
         }
-        if (cudaMemcpy(f->tw[d], tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(f->ck[d], ck.data(), ck.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(f->ones[d], on.data(), on.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) {
+        if (!upload(f, f->tw[d], tw.data(), tw.size() * sizeof(float2)) ||
+            !upload(f, f->ck[d], ck.data(), ck.size() * sizeof(float)) ||
+            !upload(f, f->ones[d], on.data(), on.size() * sizeof(float))) {
             ffno_destroy(f);
             return ffail(nullptr, LBM_ERR_CUDA, "table upload failed");
         }
@@ -594,7 +603,7 @@ extern "C" lbm_status ffno_create(const ffno_config *cfg, void *stream, ffno_ctx
             all.insert(all.end(), one.begin(), one.end());
         }
         if (alloc(f, f->tables, (int64_t)all.size()) != LBM_OK ||
-            cudaMemcpy(f->tables, all.data(), all.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) {
+            !upload(f, f->tables, all.data(), all.size() * sizeof(float))) {
             ffno_destroy(f);
             return ffail(nullptr, LBM_ERR_CUDA, "table upload failed");
         }
@@ -621,14 +630,18 @@ extern "C" lbm_status ffno_create(const ffno_config *cfg, void *stream, ffno_ctx
     fill(f->oQ1w, (int64_t)c.hidden * W, 1.0 / W); fill(f->oQ1b, c.hidden, 1 / std::sqrt((double)W));
     fill(f->oQ2w, (int64_t)c.cout * c.hidden, std::sqrt(6.0 / c.hidden) / c.omega0);
     fill(f->oQ2b, c.cout, 1 / std::sqrt((double)c.hidden));
-    if (cudaMemcpy(f->params, p.data(), p.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(f->m1, 0, f->np * sizeof(float)) != cudaSuccess ||
-        cudaMemset(f->m2, 0, f->np * sizeof(float)) != cudaSuccess ||
-        cudaMemset(f->grads, 0, f->np * sizeof(float)) != cudaSuccess) {
+    if (!upload(f, f->params, p.data(), p.size() * sizeof(float)) ||
+        cudaMemsetAsync(f->m1, 0, f->np * sizeof(float), f->s) != cudaSuccess ||
+        cudaMemsetAsync(f->m2, 0, f->np * sizeof(float), f->s) != cudaSuccess ||
+        cudaMemsetAsync(f->grads, 0, f->np * sizeof(float), f->s) != cudaSuccess) {
         ffno_destroy(f);
         return ffail(nullptr, LBM_ERR_CUDA, "parameter upload failed");
     }
     pack_weights(f);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(f->s) != cudaSuccess) {
+        ffno_destroy(f);
+        return ffail(nullptr, LBM_ERR_CUDA, "packing the spectral weights failed");
+    }
     *out = f;
     return LBM_OK;
 }

@@ -2657,8 +2657,10 @@ extern "C" lbm_status fno_create(const fno_config *cfg, void *stream, fno_ctx **
         const double ck = (k == 0 || (c.nz % 2 == 0 && k == c.nz / 2)) ? 1.0 : 2.0;
         inv[k] = (float)(ck / (double)N);
     }
-    ok = ok && cudaMemcpy(f->scale_one, one, sizeof one, cudaMemcpyHostToDevice) == cudaSuccess &&
-         cudaMemcpy(f->scale_inv, inv, sizeof inv, cudaMemcpyHostToDevice) == cudaSuccess;
+    // all on the context's own stream, waited for below: the default stream
+    // orders nothing for one created non-blocking
+    ok = ok && cudaMemcpyAsync(f->scale_one, one, sizeof one, cudaMemcpyHostToDevice, f->s) == cudaSuccess &&
+         cudaMemcpyAsync(f->scale_inv, inv, sizeof inv, cudaMemcpyHostToDevice, f->s) == cudaSuccess;
     // initial parameters: uniform within 1/sqrt(fan-in); the SIREN projection
     // as Sitzmann et al. (first layer within 1/fan-in, output layer within
     // sqrt(6/fan-in)/omega0)
@@ -2678,10 +2680,12 @@ extern "C" lbm_status fno_create(const fno_config *cfg, void *stream, fno_ctx **
     fill(f->oQ1_b, H, 1.0 / std::sqrt((double)W));
     fill(f->oQ2_w, (int64_t)c.cout * H, std::sqrt(6.0 / (double)H) / (double)c.omega0);
     fill(f->oQ2_b, c.cout, 1.0 / std::sqrt((double)H));
-    ok = ok && cudaMemcpy(f->params, p0.data(), o * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
-         cudaMemset(f->m1, 0, o * sizeof(float)) == cudaSuccess && cudaMemset(f->m2, 0, o * sizeof(float)) == cudaSuccess &&
-         cudaMemset(f->grads, 0, o * sizeof(float)) == cudaSuccess;
-    ok = ok && cudaMemset(f->ustatus, 0, 4 * sizeof(int)) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(f->params, p0.data(), o * sizeof(float), cudaMemcpyHostToDevice, f->s) == cudaSuccess &&
+         cudaMemsetAsync(f->m1, 0, o * sizeof(float), f->s) == cudaSuccess &&
+         cudaMemsetAsync(f->m2, 0, o * sizeof(float), f->s) == cudaSuccess &&
+         cudaMemsetAsync(f->grads, 0, o * sizeof(float), f->s) == cudaSuccess &&
+         cudaMemsetAsync(f->ustatus, 0, 4 * sizeof(int), f->s) == cudaSuccess;
+    ok = cudaStreamSynchronize(f->s) == cudaSuccess && ok;
     if (ok && c.umma) {
         // tensor maps of the layer inputs [max_batch * width * nz * ny rows][128]
         if (!(c.act_bf16 && c.nx == 128 && f->Kx == 32) || !umma_set_smem()) {
@@ -3193,10 +3197,10 @@ extern "C" lbm_status fno_load(fno_ctx *f, const char *path)
         f->err = same ? "checkpoint truncated" : "checkpoint does not match this network's shape";
         return LBM_ERR_IO;
     }
+    FCK(cudaMemcpyAsync(f->params, buf.data(), f->np * sizeof(float), cudaMemcpyHostToDevice, f->s));
+    FCK(cudaMemcpyAsync(f->m1, buf.data() + f->np, f->np * sizeof(float), cudaMemcpyHostToDevice, f->s));
+    FCK(cudaMemcpyAsync(f->m2, buf.data() + 2 * f->np, f->np * sizeof(float), cudaMemcpyHostToDevice, f->s));
     FCK(cudaStreamSynchronize(f->s));
-    FCK(cudaMemcpy(f->params, buf.data(), f->np * sizeof(float), cudaMemcpyHostToDevice));
-    FCK(cudaMemcpy(f->m1, buf.data() + f->np, f->np * sizeof(float), cudaMemcpyHostToDevice));
-    FCK(cudaMemcpy(f->m2, buf.data() + 2 * f->np, f->np * sizeof(float), cudaMemcpyHostToDevice));
     f->adam_t = h.adam_t;
     return LBM_OK;
 }

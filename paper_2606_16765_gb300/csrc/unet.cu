@@ -1028,11 +1028,12 @@ extern "C" lbm_status unet_create(const unet_config *cfg, void *stream, unet_ctx
     }
     const double lim = 1.0 / std::sqrt((double)c.channels[0]);
     for (int64_t i = 0; i < (int64_t)c.cout * c.channels[0]; ++i) h[u->oOw + i] = (float)(lim * (2.0 * unif01(st) - 1.0));
-    if (cudaMemcpy(u->params, h.data(), u->np * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(u->grads, 0, u->np * sizeof(float)) != cudaSuccess ||
-        cudaMemset(u->m1, 0, u->np * sizeof(float)) != cudaSuccess ||
-        cudaMemset(u->m2, 0, u->np * sizeof(float)) != cudaSuccess ||
-        cudaMemset(u->ustatus, 0, sizeof(int)) != cudaSuccess) {
+    // on the context's own stream: the default stream orders nothing for one created non-blocking
+    if (cudaMemcpyAsync(u->params, h.data(), u->np * sizeof(float), cudaMemcpyHostToDevice, u->s) != cudaSuccess ||
+        cudaMemsetAsync(u->grads, 0, u->np * sizeof(float), u->s) != cudaSuccess ||
+        cudaMemsetAsync(u->m1, 0, u->np * sizeof(float), u->s) != cudaSuccess ||
+        cudaMemsetAsync(u->m2, 0, u->np * sizeof(float), u->s) != cudaSuccess ||
+        cudaMemsetAsync(u->ustatus, 0, sizeof(int), u->s) != cudaSuccess) {
         g_unet_err = "device initialisation failed";
         unet_destroy(u);
         return LBM_ERR_CUDA;
