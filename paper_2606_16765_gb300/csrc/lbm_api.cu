@@ -832,9 +832,10 @@ extern "C" lbm_status lbm_set_wall_distances(lbm_ctx *ctx, int64_t n, const int6
     CK(cudaMalloc(&ctx->qval, m * sizeof(double)));
     CK(cudaMalloc(&ctx->qpart, 3 * sizeof(double) * nb));
     CK(cudaMalloc(&ctx->qcount, sizeof(unsigned)));
-    CK(cudaMemcpy(ctx->qlinks, L.data(), m * sizeof(uint4), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(ctx->qval, V.data(), m * sizeof(double), cudaMemcpyHostToDevice));
-    CK(cudaMemset(ctx->qcount, 0, sizeof(unsigned)));
+    CK(cudaMemcpyAsync(ctx->qlinks, L.data(), m * sizeof(uint4), cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(ctx->qval, V.data(), m * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemsetAsync(ctx->qcount, 0, sizeof(unsigned), ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
     ctx->n_qlinks = m;
     return LBM_OK;
 }
@@ -860,7 +861,8 @@ extern "C" lbm_status lbm_set_probes(lbm_ctx *ctx, int64_t n, const int64_t *cel
     if (n == 0) return LBM_OK;
     CK(cudaMalloc(&ctx->probe_cells, sizeof(int64_t) * n));
     CK(cudaMalloc(&ctx->probe_ring, sizeof(float) * 4 * n * capacity));
-    CK(cudaMemcpy(ctx->probe_cells, cells, sizeof(int64_t) * n, cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(ctx->probe_cells, cells, sizeof(int64_t) * n, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
     ctx->n_probes = n;
     ctx->probe_every = every;
     ctx->probe_cap = capacity;
@@ -1157,11 +1159,13 @@ extern "C" lbm_status lbm_load(lbm_ctx *ctx, const char *path)
     if (h.snap_count) ok = ok && std::fread(taken.data(), 1, taken.size(), fp) == taken.size();
     std::fclose(fp);
     if (!ok) return fail(ctx, LBM_ERR_IO, "checkpoint truncated");
+    CK(cudaMemcpyAsync(ctx->base + L.pdf, buf.data(), pdf_bytes, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(ctx->base + L.ub, buf.data() + pdf_bytes, ub_bytes, cudaMemcpyHostToDevice, ctx->stream));
+    if (ms_bytes)
+        CK(cudaMemcpyAsync(ctx->base + L.msum, buf.data() + pdf_bytes + ub_bytes, ms_bytes, cudaMemcpyHostToDevice,
+                           ctx->stream));
+    CK(cudaMemsetAsync(ctx->base + L.status, 0, sizeof(int), ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    CK(cudaMemcpy(ctx->base + L.pdf, buf.data(), pdf_bytes, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(ctx->base + L.ub, buf.data() + pdf_bytes, ub_bytes, cudaMemcpyHostToDevice));
-    if (ms_bytes) CK(cudaMemcpy(ctx->base + L.msum, buf.data() + pdf_bytes + ub_bytes, ms_bytes, cudaMemcpyHostToDevice));
-    CK(cudaMemset(ctx->base + L.status, 0, sizeof(int)));
     ctx->t = h.t;
     ctx->msamples = h.msamples;
     ctx->force_host = frows;
@@ -1488,7 +1492,7 @@ extern "C" lbm_status lbm_batch_create(int32_t n, const lbm_grid *grids, const u
         cudaMalloc(&b->d_qbegin, sizeof(int64_t) * (n + 1)) != cudaSuccess ||
         cudaMalloc(&b->d_wbegin, sizeof(int64_t) * (n + 1)) != cudaSuccess ||
         cudaMalloc(&b->d_t, sizeof(int64_t)) != cudaSuccess ||
-        cudaMemset(b->d_t, 0, sizeof(int64_t)) != cudaSuccess)
+        cudaMemsetAsync(b->d_t, 0, sizeof(int64_t), b->own) != cudaSuccess)
         st = LBM_ERR_CUDA;
     if (st != LBM_OK) {
         cudaGetLastError();
@@ -1729,7 +1733,7 @@ static lbm_status batch_reset(lbm_batch *b)
         const lbm_status st = lbm_reset(c);
         if (st != LBM_OK) return st;
     }
-    BCK(cudaMemset(b->d_t, 0, sizeof(int64_t)));
+    BCK(cudaMemsetAsync(b->d_t, 0, sizeof(int64_t), b->own));
     b->t = 0;
     b->updates = 0;
     return LBM_OK;
