@@ -1229,27 +1229,36 @@ lbm_status op_check(const void *a, const void *b, const void *c, int32_t B, int3
     return LBM_OK;
 }
 
-// one convolution into FP32, through parts where the plan splits the sum
+// One convolution into FP32, through parts where the plan splits the sum.  The
+// kernels store 16 bytes at a time: an output on any other boundary of floats
+// is formed in scratch and copied.
 lbm_status op_conv(OpScratch &sc, const bf16 *act, int k, int nx, int ny, int nz, int B, const bf16 *w, int N, float *out,
                    int *status)
 {
+    const size_t n = (size_t)B * nx * ny * nz * N;
+    const bool whole = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    float *dst = whole ? out : sc.get<float>(n);
+    if (!dst) return LBM_ERR_OOM;
     unet::ConvPlan p;
     const char *e = nullptr;
-    // the parts are added 16 bytes at a time
-    const bool split = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
-    if (!unet::conv_plan(p, act, k, k, nx, ny, nz, B, w, N, 27, N, 0, gb300::sm_count(), &e, split)) {
+    if (!unet::conv_plan(p, act, k, k, nx, ny, nz, B, w, N, 27, N, 0, gb300::sm_count(), &e, true)) {
         cudaStreamSynchronize(sc.s);
         g_unet_err = e ? e : "plan failed";
         return LBM_ERR_ARG;
     }
     if (p.a.ksplit == 1) {
-        unet::conv_launch(p, out, true, status, sc.s);
-        return LBM_OK;
+        unet::conv_launch(p, dst, true, status, sc.s);
+    } else {
+        float *part = sc.get<float>((size_t)p.a.ksplit * p.a.split_stride);
+        if (!part) return LBM_ERR_OOM;
+        unet::conv_launch(p, part, true, status, sc.s);
+        unet::conv_sum(p, part, dst, sc.s);
     }
-    float *part = sc.get<float>((size_t)p.a.ksplit * p.a.split_stride);
-    if (!part) return LBM_ERR_OOM;
-    unet::conv_launch(p, part, true, status, sc.s);
-    unet::conv_sum(p, part, out, sc.s);
+    if (!whole && cudaMemcpyAsync(out, dst, n * sizeof(float), cudaMemcpyDeviceToDevice, sc.s) != cudaSuccess) {
+        cudaGetLastError();
+        g_unet_err = "convolution: copy of the output failed";
+        return LBM_ERR_CUDA;
+    }
     return LBM_OK;
 }
 
