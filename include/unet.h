@@ -111,15 +111,18 @@ const char *unet_last_error(const unet_ctx *u);
  *   unet_conv3_backward_data gx[b][p][i] = sum_{d,o} w[o][i][d] gy[b][p - d + 1][o]
  *   unet_conv3_backward_weights gw[o][i][d] = sum_{b,p} gy[b][p][o] x[b][p + d - 1][i]
  * x [batch][nz][ny][nx][cin], y and gy [batch][nz][ny][nx][cout], w and gw
- * [cout][cin][27] (d = (dz*3 + dy)*3 + dx), zero outside the grid.  The call
- * allocates its own temporaries and waits for the stream; status as
- * unet_sync. */
+ * [cout][cin][27] (d = (dz*3 + dy)*3 + dx), zero outside the grid; any of them
+ * may start on any float.  The call takes its temporaries from a pool of the
+ * device and waits for the stream; status as unet_sync.  The pool keeps up to
+ * 1 GiB per device for the next call; unet_conv3_trim gives back what no call
+ * is using (on every device, from any thread). */
 lbm_status unet_conv3_forward(const float *x, const float *w, float *y, int32_t batch, int32_t nx, int32_t ny,
                               int32_t nz, int32_t cin, int32_t cout, void *cuda_stream);
 lbm_status unet_conv3_backward_data(const float *gy, const float *w, float *gx, int32_t batch, int32_t nx, int32_t ny,
                                     int32_t nz, int32_t cin, int32_t cout, void *cuda_stream);
 lbm_status unet_conv3_backward_weights(const float *x, const float *gy, float *gw, int32_t batch, int32_t nx,
                                        int32_t ny, int32_t nz, int32_t cin, int32_t cout, void *cuda_stream);
+lbm_status unet_conv3_trim(void);
 
 #ifdef __cplusplus
 }

@@ -1160,19 +1160,30 @@ namespace {
 
 // Scratch of one call, from a stream-ordered pool of the device that keeps up
 // to a gigabyte between calls (more goes back to the device at the next
-// synchronisation): cudaMalloc and cudaFree of the converted operands took
-// 0.26 to 0.38 ms per call.  Pools are created once per device under a lock;
-// the driver serialises their use by threads and orders it by stream.
+// synchronisation, the rest with unet_conv3_trim): cudaMalloc and cudaFree of
+// the converted operands took 0.26 to 0.38 ms per call.  Pools are created once
+// per device under a lock; the driver serialises their use by threads and
+// orders it by stream.
 constexpr int MAX_DEV = 64;
+
+struct OpPools {
+    std::mutex lock;
+    cudaMemPool_t pool[MAX_DEV] = {};
+};
+
+OpPools &op_pools()
+{
+    static OpPools p;
+    return p;
+}
 
 cudaMemPool_t op_pool()
 {
-    static std::mutex lock;
-    static cudaMemPool_t pool[MAX_DEV];
+    OpPools &all = op_pools();
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev >= MAX_DEV) return nullptr;
-    std::lock_guard<std::mutex> hold(lock);
-    if (!pool[dev]) {
+    std::lock_guard<std::mutex> hold(all.lock);
+    if (!all.pool[dev]) {
         cudaMemPoolProps pr{};
         pr.allocType = cudaMemAllocationTypePinned;
         pr.location.type = cudaMemLocationTypeDevice;
@@ -1184,9 +1195,9 @@ cudaMemPool_t op_pool()
             return nullptr;
         }
         cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
-        pool[dev] = p;
+        all.pool[dev] = p;
     }
-    return pool[dev];
+    return all.pool[dev];
 }
 
 struct OpScratch {
@@ -1280,6 +1291,18 @@ lbm_status op_finish(cudaStream_t s, int *status)
 }
 
 }  // namespace
+
+extern "C" lbm_status unet_conv3_trim(void)
+{
+    OpPools &all = op_pools();
+    std::lock_guard<std::mutex> hold(all.lock);
+    for (cudaMemPool_t p : all.pool)
+        if (p && cudaMemPoolTrimTo(p, 0) != cudaSuccess) {
+            g_unet_err = std::string("convolution scratch: ") + cudaGetErrorString(cudaGetLastError());
+            return LBM_ERR_CUDA;
+        }
+    return LBM_OK;
+}
 
 extern "C" lbm_status unet_conv3_forward(const float *x, const float *w, float *y, int32_t B, int32_t nx, int32_t ny,
                                          int32_t nz, int32_t cin, int32_t cout, void *stream)

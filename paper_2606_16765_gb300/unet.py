@@ -56,6 +56,7 @@ def lib():
             "unet_conv3_forward": conv,
             "unet_conv3_backward_data": conv,
             "unet_conv3_backward_weights": conv,
+            "unet_conv3_trim": (C.c_int, []),
         }
         for name, (res, args) in sig.items():
             fn = getattr(L, name)
@@ -109,6 +110,11 @@ def conv3_backward_weights(x, gy, gw, stream=0):
     B, nz, ny, nx, cin = x.shape
     _check(lib().unet_conv3_backward_weights(_ptr(x), _ptr(gy), _ptr(gw), B, nx, ny, nz, cin, gy.shape[-1],
                                              _vp(stream)), None)
+
+
+def conv3_trim():
+    """Give back the scratch memory that the convolution calls keep between them (up to 1 GiB per device)."""
+    _check(lib().unet_conv3_trim(), None)
 
 
 class UNet:
