@@ -24,7 +24,9 @@
  * Everything is computed in FP32.  Widths up to 32 with hidden widths up to
  * 128 run on tiled kernels, others on general ones.  Conventions as in
  * lbm.h: every call returns lbm_status; x, t, m and y may be host or device
- * memory; work runs on the stream given at creation.
+ * memory (the tiled kernels use memory of the context's own device in place,
+ * any other is copied) and start on any float; work runs on the stream given
+ * at creation.
  */
 #ifndef GB300_FFNO_H
 #define GB300_FFNO_H

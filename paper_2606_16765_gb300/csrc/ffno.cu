@@ -33,6 +33,7 @@
 
 #include "../../include/ffno.h"
 #include "ffno_fast.h"
+#include "ffno_place.h"
 #include "sm_count.h"
 
 namespace {
@@ -346,6 +347,7 @@ __global__ void k_adam(float *p, const float *g, float *m1, float *m2, int64_t n
 struct ffno_ctx {
     ffno_config c{};
     cudaStream_t s = nullptr;
+    int device = 0;
     std::string err;
     int64_t N = 0, np = 0, adam_t = 0;
     Ext fe{}, se[3]{};
@@ -427,14 +429,14 @@ uint64_t splitmix(uint64_t &s)
 
 double unif(uint64_t &s) { return 2.0 * ((splitmix(s) >> 11) * (1.0 / 9007199254740992.0)) - 1.0; }
 
-bool is_host(const void *p)
+ffno::Place place_of(const ffno_ctx *f, const void *p)
 {
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
-        return true;
+        return ffno::PLACE_HOST;
     }
-    return at.type != cudaMemoryTypeDevice && at.type != cudaMemoryTypeManaged;
+    return ffno::place_of(at, f->device);
 }
 
 // spectral weights per wave number, for the forward and (conjugate
@@ -495,6 +497,7 @@ extern "C" lbm_status ffno_create(const ffno_config *cfg, void *stream, ffno_ctx
     ffno_ctx *f = new ffno_ctx();
     f->c = *cfg;
     f->s = static_cast<cudaStream_t>(stream);
+    if (cudaGetDevice(&f->device) != cudaSuccess) cudaGetLastError();       // the allocations below fail then
     const ffno_config &c = f->c;
     const int W = c.width, H = c.ff_hidden, LH = c.lift_hidden, L = c.layers, B = c.max_batch;
     f->N = (int64_t)c.nx * c.ny * c.nz;
@@ -794,22 +797,24 @@ extern "C" lbm_status ffno_forward(ffno_ctx *f, const float *x, float *y, int32_
     if (!f || !x || !y) return ffail(f, LBM_ERR_ARG, "null argument");
     if (batch < 1) return ffail(f, LBM_ERR_ARG, "batch must be positive");
     const ffno_config &c = f->c;
-    const bool xh = is_host(x), yh = is_host(y);        // device memory is read and written where it is
+    // memory of this device is read and written where it is
+    const ffno::Place xp = place_of(f, x), yp = place_of(f, y);
+    const bool xs = !f->fast || xp != ffno::PLACE_HERE, ys = !f->fast || yp != ffno::PLACE_HERE;
     for (int32_t b0 = 0; b0 < batch; b0 += c.max_batch) {
         const int B = std::min(c.max_batch, batch - b0);
         const float *xb = x + (int64_t)b0 * c.cin * f->N;
         float *yb = y + (int64_t)b0 * c.cout * f->N;
-        if (!f->fast || xh) {
+        if (xs) {
             FCK(cudaMemcpyAsync(f->xin, xb, sizeof(float) * B * c.cin * f->N, cudaMemcpyDefault, f->s));
             xb = f->xin;
         }
-        if (f->fast) forward_fast(f, xb, yh ? f->y : yb, B, false);
+        if (f->fast) forward_fast(f, xb, ys ? f->y : yb, B, false);
         else forward_impl(f, B);
         FCK(cudaGetLastError());
-        if (!f->fast || yh)
+        if (ys)
             FCK(cudaMemcpyAsync(yb, f->y, sizeof(float) * B * c.cout * f->N, cudaMemcpyDefault, f->s));
     }
-    if (yh) FCK(cudaStreamSynchronize(f->s));
+    if (yp == ffno::PLACE_HOST) FCK(cudaStreamSynchronize(f->s));
     return LBM_OK;
 }
 
@@ -822,7 +827,7 @@ extern "C" lbm_status ffno_loss_grad(ffno_ctx *f, const float *x, const float *t
     const int B = batch;
     const int64_t N = f->N;
     auto stage = [&](const float *&src, float *dst, int64_t n) {
-        if (f->fast && !is_host(src)) return cudaSuccess;
+        if (f->fast && place_of(f, src) == ffno::PLACE_HERE) return cudaSuccess;
         const cudaError_t e = cudaMemcpyAsync(dst, src, sizeof(float) * n, cudaMemcpyDefault, f->s);
         src = dst;
         return e;
