@@ -1589,6 +1589,12 @@ __global__ void __launch_bounds__(TPB) k_dftx_inv_tc(const float2 *It, float *ou
 // columns 2t, 2t+1, 2t+8, 2t+9: the order of a contraction is free), so that a
 // row is one 16- and one 8-byte load, and the next k-step's loads are issued
 // ahead of this one's products.
+// A fragment takes at most OUTER_STEPS k-steps before it goes into the block's
+// sums: the tensor cores' additions drop what lies below their accumulator, and
+// a chunk is as long as the batch makes it (55,000 cells a block, 430 k-steps a
+// warp, for 128 outputs at 8 x 524,288 cells; summed in one go, sums of one sign
+// are off by 8.9e-6, in pieces by 7e-7, as with fixed chunks of 8192 cells).
+constexpr int OUTER_STEPS = OUTER_CHUNK / (16 * (TPB / 32));
 __global__ void __launch_bounds__(TPB, 2) k_outer_tc(const float *__restrict__ g, int co,
                                                      const __nv_bfloat16 *__restrict__ x, float *gW, float *gb,
                                                      int64_t N, int B, int64_t chunk)
@@ -1623,9 +1629,25 @@ __global__ void __launch_bounds__(TPB, 2) k_outer_tc(const float *__restrict__ g
         }
     };
     constexpr int KSTEP = 16 * (TPB / 32);
+    // fragment (mt, nt): e = 0, 1: row 16 mt + gq, column 8 nt + 2t + e;
+    // e = 2, 3: row 16 mt + gq + 8; the bias sits in column 0 of n-tile 4
+    auto add_up = [&] {
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    atomicAdd(&red[16 * mt + gq + 8 * (e >> 1)][8 * nt + 2 * t + (e & 1)], acc[mt][nt][e]);
+            if (t == 0) {
+                atomicAdd(&red[16 * mt + gq][32], acc[mt][4][0]);
+                atomicAdd(&red[16 * mt + gq + 8][32], acc[mt][4][2]);
+            }
+        }
+    };
     int64_t k0 = c0 + 16 * warp;
     if (k0 < c1) fetch(k0, ga, bx);
-    for (; k0 < c1; k0 += KSTEP) {
+    for (int steps = 1; k0 < c1; k0 += KSTEP, ++steps) {
         if (k0 + KSTEP < c1) fetch(k0 + KSTEP, gn, bn);
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) {
@@ -1651,21 +1673,17 @@ __global__ void __launch_bounds__(TPB, 2) k_outer_tc(const float *__restrict__ g
             ga[q >> 1][q & 1] = gn[q >> 1][q & 1];
             bx[q] = bn[q];
         }
-    }
-    // fragment (mt, nt): e = 0, 1: row 16 mt + gq, column 8 nt + 2t + e;
-    // e = 2, 3: row 16 mt + gq + 8; the bias sits in column 0 of n-tile 4
+        if (steps % OUTER_STEPS == 0) {
+            add_up();
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
+            for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
+                for (int nt = 0; nt < 5; ++nt)
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                atomicAdd(&red[16 * mt + gq + 8 * (e >> 1)][8 * nt + 2 * t + (e & 1)], acc[mt][nt][e]);
-        if (t == 0) {
-            atomicAdd(&red[16 * mt + gq][32], acc[mt][4][0]);
-            atomicAdd(&red[16 * mt + gq + 8][32], acc[mt][4][2]);
+                    for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.f;
         }
     }
+    add_up();
     __syncthreads();
     for (int k = threadIdx.x; k < 32 * 32; k += blockDim.x) atomicAdd(&gW[(int64_t)(o0 + k / 32) * 32 + k % 32], red[k / 32][k % 32]);
     for (int k = threadIdx.x; k < 32; k += blockDim.x) atomicAdd(&gb[o0 + k], red[k][32]);
