@@ -996,7 +996,7 @@ __global__ void __launch_bounds__(TPB) k_dftx_fwd(const TI *x, float2 *A, const 
 // as a BF16 pair hi + lo (hi = bf16(t), lo = bf16(t - hi)).  BF16 samples
 // are exact: two products per tile (hi, lo table); FP32 samples are split
 // the same way: three products (hi hi, hi lo, lo hi).  Either keeps about
-// 2^-16 relative error.  A warp takes 32 rows per pass.  Lane (g, c)
+// 2^-16 relative error.  A warp takes 16 M rows per pass.  Lane (g, c)
 // (g = lane / 4, c = lane % 4) loads the 32 consecutive samples
 // x in [32c, 32c + 32) of rows g, g + 8, g + 16 and g + 24 with 16-byte loads, and the
 // contraction index is permuted to match: in k-step s, fragment column
@@ -1025,7 +1025,7 @@ __device__ __forceinline__ void mma_bf16(float *acc, uint32_t a0, uint32_t a1, u
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b.x), "r"(b.y));
 }
 
-template <class TI>
+template <class TI, int M>
 __global__ void __launch_bounds__(TPB, 2) k_dftx_fwd_tc(const TI *x, float2 *A, const float2 *twx, int64_t R)
 {
     __shared__ uint2 bt[2][8 * 8 * 32];     // [hi, lo][(k-step * 8 + n-tile) * 32 + lane]
@@ -1047,22 +1047,22 @@ __global__ void __launch_bounds__(TPB, 2) k_dftx_fwd_tc(const TI *x, float2 *A, 
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
-    // two m-tiles per pass: a table fragment read from shared memory, which
-    // bounds this kernel, serves both
-    const int64_t tiles = (R + 31) / 32;
+    // two m-tiles per pass (M = 2): a table fragment read from shared memory,
+    // which bounds this kernel, serves both
+    const int64_t tiles = (R + 16 * M - 1) / (16 * M);
     for (int64_t tile = (int64_t)blockIdx.x * (TPB / 32) + warp; tile < tiles; tile += (int64_t)gridDim.x * (TPB / 32)) {
-        const int64_t r0 = tile * 32 + g;                    // rows r0 + 8 i of fragment half i
-        float acc[2][8][4];
+        const int64_t r0 = tile * 16 * M + g;                    // rows r0 + 8 i of fragment half i
+        float acc[M][8][4];
 #pragma unroll
-        for (int m = 0; m < 2; ++m)
+        for (int m = 0; m < M; ++m)
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[m][nt][e] = 0.f;
         if (std::is_same<TI, __nv_bfloat16>::value) {
-            uint4 v[4][4];
+            uint4 v[2 * M][4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < 2 * M; ++i) {
                 const uint4 *p = reinterpret_cast<const uint4 *>(x + (r0 + 8 * i) * TCX_NX + 32 * c);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) v[i][q] = r0 + 8 * i < R ? p[q] : make_uint4(0u, 0u, 0u, 0u);
@@ -1077,7 +1077,7 @@ __global__ void __launch_bounds__(TPB, 2) k_dftx_fwd_tc(const TI *x, float2 *A, 
 #pragma unroll
                         for (int u = 0; u < 4; ++u) b[u] = bt[part][(st * 8 + n4 + u) * 32 + lane];
 #pragma unroll
-                        for (int m = 0; m < 2; ++m) {
+                        for (int m = 0; m < M; ++m) {
                             const uint4 &ua = v[2 * m][st >> 1], &ub = v[2 * m + 1][st >> 1];
                             const uint32_t a0 = (st & 1) ? ua.z : ua.x, a2 = (st & 1) ? ua.w : ua.y;
                             const uint32_t a1 = (st & 1) ? ub.z : ub.x, a3 = (st & 1) ? ub.w : ub.y;
@@ -1089,19 +1089,19 @@ __global__ void __launch_bounds__(TPB, 2) k_dftx_fwd_tc(const TI *x, float2 *A, 
             }
         } else {
             const float4 *p = reinterpret_cast<const float4 *>(x + r0 * TCX_NX + 32 * c);
-            float4 f[4], fn[4];
+            float4 f[2 * M], fn[2 * M];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) f[i] = r0 + 8 * i < R ? p[i * 8 * TCX_NX / 4] : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int i = 0; i < 2 * M; ++i) f[i] = r0 + 8 * i < R ? p[i * 8 * TCX_NX / 4] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int st = 0; st < 8; ++st) {
                 // samples 32c + 4st + {0..3}, the next step's ahead of the products
                 if (st < 7)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
+                    for (int i = 0; i < 2 * M; ++i)
                         fn[i] = r0 + 8 * i < R ? p[i * 8 * TCX_NX / 4 + st + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
-                uint32_t hh[2][4], ll[2][4];
+                uint32_t hh[M][4], ll[M][4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < 2 * M; ++i) {
                     __nv_bfloat16 h[4], l[4];
                     split_bf16(f[i].x, h[0], l[0]); split_bf16(f[i].y, h[1], l[1]);
                     split_bf16(f[i].z, h[2], l[2]); split_bf16(f[i].w, h[3], l[3]);
@@ -1118,15 +1118,15 @@ __global__ void __launch_bounds__(TPB, 2) k_dftx_fwd_tc(const TI *x, float2 *A, 
                         bl[u] = bt[1][(st * 8 + n4 + u) * 32 + lane];
                     }
 #pragma unroll
-                    for (int m = 0; m < 2; ++m)
+                    for (int m = 0; m < M; ++m)
 #pragma unroll
                         for (int u = 0; u < 4; ++u) mma_bf16(acc[m][n4 + u], hh[m][0], hh[m][1], hh[m][2], hh[m][3], bh[u]);
 #pragma unroll
-                    for (int m = 0; m < 2; ++m)
+                    for (int m = 0; m < M; ++m)
 #pragma unroll
                         for (int u = 0; u < 4; ++u) mma_bf16(acc[m][n4 + u], hh[m][0], hh[m][1], hh[m][2], hh[m][3], bl[u]);
 #pragma unroll
-                    for (int m = 0; m < 2; ++m)
+                    for (int m = 0; m < M; ++m)
 #pragma unroll
                         for (int u = 0; u < 4; ++u) mma_bf16(acc[m][n4 + u], ll[m][0], ll[m][1], ll[m][2], ll[m][3], bh[u]);
                 }
@@ -1134,7 +1134,7 @@ __global__ void __launch_bounds__(TPB, 2) k_dftx_fwd_tc(const TI *x, float2 *A, 
         }
         // D: columns n = 8 nt + 2c + {0, 1} are mode 4 nt + c's re, im
 #pragma unroll
-        for (int m = 0; m < 2; ++m)
+        for (int m = 0; m < M; ++m)
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 const int64_t r = r0 + 16 * m + 8 * i;
@@ -1831,7 +1831,7 @@ __device__ __forceinline__ int swz(int row, int x) { return row * 256 + ((((x >>
 __global__ void __launch_bounds__(FUSE_WARPS * 32, 1) k_layer_tc(const float2 *It, const __nv_bfloat16 *v,
                                                                const float *W, const float *bias, const float2 *twx,
                                                                __nv_bfloat16 *pre, __nv_bfloat16 *out, int act,
-                                                               int64_t lines_per_sample, int64_t N, int B)
+                                                               int64_t lines_per_sample, int64_t N, int B, int line_warps)
 {
     extern __shared__ __align__(16) unsigned char fsm[];
     uint2 *bt = reinterpret_cast<uint2 *>(fsm);                          // [2][4 * 16 * 32]
@@ -1870,6 +1870,7 @@ __global__ void __launch_bounds__(FUSE_WARPS * 32, 1) k_layer_tc(const float2 *I
     __syncthreads();
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+    if (warp >= line_warps) return;                              // they helped with the fragments
     unsigned char *vt = tiles + (size_t)warp * (FUSE_C * TCX_NX * 2 + 16 * TCX_NX * 2);
     unsigned char *ot = vt + FUSE_C * TCX_NX * 2;
     const int64_t lines = (int64_t)B * lines_per_sample;
@@ -1896,7 +1897,7 @@ __global__ void __launch_bounds__(FUSE_WARPS * 32, 1) k_layer_tc(const float2 *I
         }
         cp_async_commit();
     };
-    const int64_t first = (int64_t)blockIdx.x * FUSE_WARPS + warp, step = (int64_t)gridDim.x * FUSE_WARPS;
+    const int64_t first = (int64_t)blockIdx.x * line_warps + warp, step = (int64_t)gridDim.x * line_warps;
     if (first < lines) {
         copy_v(first);
         copy_it(first, 0);
@@ -2903,8 +2904,12 @@ void dft_fwd(fno_ctx *f, const T *x, float2 *S, const float *scale, int B, int l
         const int blocks = (int)std::min<int64_t>(tiles, (int64_t)gb300::sm_count() * 2);
         umma_dftx_fwd(f->vmaps[layer_map].data(), f->twx, f->stA, R, f->ustatus, blocks, f->s);
     } else if (tc_input && d.nx == TCX_NX && d.Kx == TCX_KX && (reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
-        const int64_t warps = (R + 31) / 32;
-        k_dftx_fwd_tc<T><<<(int)std::min<int64_t>((warps + TPB / 32 - 1) / (TPB / 32), gb300::sm_count() * 8), TPB, 0, f->s>>>(
+        // one m-tile per pass while that leaves a warp slot of one block per SM for each
+        // (2,048 rows 7.8 and 5.5 us, 8,192 rows 8.1 and 5.7, 32,768 rows 9.0 and 9.3)
+        const bool one = (R + 15) / 16 <= (int64_t)gb300::sm_count() * (TPB / 32);
+        const int64_t warps = one ? (R + 15) / 16 : (R + 31) / 32;
+        auto k = one ? k_dftx_fwd_tc<T, 1> : k_dftx_fwd_tc<T, 2>;
+        k<<<(int)std::min<int64_t>((warps + TPB / 32 - 1) / (TPB / 32), gb300::sm_count() * 8), TPB, 0, f->s>>>(
             x, f->stA, f->twx, R);
     } else {
         k_dftx_fwd<T><<<(int)std::min<int64_t>((R + DFT_ROWS - 1) / DFT_ROWS, gb300::sm_count() * 8), TPB, smem_dftx_fwd(d),
@@ -3000,12 +3005,15 @@ lbm_status forward_impl(fno_ctx *f, const float *x, int B, bool keep = true)
         if (fuse) {
             dft_inv_zy(f, f->G, f->scale_inv, B);
             const int64_t lps = (int64_t)c.ny * c.nz;
-            const int blocks = (int)std::min<int64_t>(((int64_t)B * lps + FUSE_WARPS - 1) / FUSE_WARPS,
-                                                      (int64_t)gb300::sm_count());
+            // few lines go to as many SMs as there are: the warps of one share its
+            // instruction issue (64 lines on 6 SMs 21.4 us, on 64 13.0; 256 lines 21.8 and 13.6)
+            const int64_t lines = (int64_t)B * lps, sms = gb300::sm_count();
+            const int line_warps = (int)std::min<int64_t>(FUSE_WARPS, (lines + sms - 1) / sms);
+            const int blocks = (int)std::min<int64_t>((lines + line_warps - 1) / line_warps, sms);
             k_layer_tc<<<blocks, FUSE_WARPS * 32, FUSE_SMEM, f->s>>>(
                 f->stA, reinterpret_cast<const __nv_bfloat16 *>(vin), f->params + f->oW_w[l], f->params + f->oW_b[l],
                 f->twx, keep ? reinterpret_cast<__nv_bfloat16 *>(f->pre[l]) : nullptr,
-                reinterpret_cast<__nv_bfloat16 *>(f->v[l + 1]), l < c.layers - 1 ? ACT_GELU : ACT_NONE, lps, f->N, B);
+                reinterpret_cast<__nv_bfloat16 *>(f->v[l + 1]), l < c.layers - 1 ? ACT_GELU : ACT_NONE, lps, f->N, B, line_warps);
             continue;
         }
         dft_inv<T>(f, f->G, f->spec, f->scale_inv, 0, nullptr, B);
