@@ -378,12 +378,19 @@ __device__ __forceinline__ void edge_cell(const StepArgs &a, const StepOut &o, i
 
 static_assert(WALL_BLOCK == EDGE_BLOCK, "wall-row blocks run in the edge kernel's launch");
 
+// Blocks per SM that the edge kernels are compiled for (0: no bound).  The odd
+// step's 27 loads in flight take 109 to 124 registers where they may, four blocks
+// per SM; large batches need the fifth (32 channels of 49 M cells, FP16S: odd
+// edge kernel 202 us, held to 96 registers 167).
+template <class S, bool ODD>
+__host__ __device__ constexpr int edge_blocks_per_sm() { return ODD && sizeof(typename Store<S>::R) == 4 ? 5 : 0; }
+
 // Single-grid edge kernel: blocks [0, eblocks) take one record of the compact
 // list per thread; the blocks after them take the wall rows, block b covering
 // cells [(b % wx) WALL_BLOCK, ...) of wall row b / wx (they have no obstacle
 // links and stay out of the force reduction).
 template <class S, bool ODD, bool PLAIN>
-__global__ void __launch_bounds__(EDGE_BLOCK) k_step_edge(StepArgs a, int eblocks, int wx)
+__global__ void __launch_bounds__(EDGE_BLOCK, edge_blocks_per_sm<S, ODD>()) k_step_edge(StepArgs a, int eblocks, int wx)
 {
     using R = typename Store<S>::R;
     const StepOut o = step_out(a);
@@ -419,8 +426,10 @@ __global__ void __launch_bounds__(EDGE_BLOCK) k_step_edge(StepArgs a, int eblock
 // gather never reads.
 // All loads of a link are issued before any is used (the flags decide which
 // values count, not which are read): one latency instead of five in a row.
-// Only the step's parity leaves some out: each costs a sector of its own on
-// this strided plane, which many large outlets feel.
+// What the step's parity and the link's direction rule out is not read: each
+// value is a sector of its own on this strided plane, which many large outlets
+// feel (32 channels, after an even and an odd step, everything read but for the
+// parity: FP32 202 and 136 us, FP16S 184 and 125; now 179 and 137, 162 and 132).
 template <class S>
 __device__ __forceinline__ void outflow_link(const StepArgs &a, uint32_t yz, int k, bool fix, bool next_odd)
 {
@@ -440,13 +449,15 @@ __device__ __forceinline__ void outflow_link(const StepArgs &a, uint32_t yz, int
     // the inner cell's source (nx - 1, y - cy, z - cz)
     const int64_t s2 = (int64_t)(a.nx - 1) + (int64_t)a.nx * ((int64_t)sy + (int64_t)a.ny * sz);
     const int64_t ci = a.nx >= 2 ? c - 1 : c;
-    const uint8_t flag_c = a.flags[c], flag_in = a.flags[ci], flag_s = next_odd ? a.flags[s2] : (uint8_t)CELL_SOLID;
-    const R was_own = *own, was_in = *in, here = T::ld(p + (int64_t)i * a.slot + c);
-    const R there = T::ld(p + (int64_t)i * a.slot + ci), across = next_odd ? T::ld(p + (int64_t)(Q - 1 - i) * a.slot + s2) : R(0);
+    const bool fixed = fix && through_face, crosses = next_odd && through_face;
+    const uint8_t flag_c = a.flags[c], flag_in = a.flags[ci], flag_s = crosses ? a.flags[s2] : (uint8_t)CELL_SOLID;
+    const R was_own = fixed ? *own : R(0), was_in = fixed ? *in : R(0);
+    const R here = fixed ? R(0) : T::ld(p + (int64_t)i * a.slot + c);
+    R next = T::ld(crosses ? p + (int64_t)(Q - 1 - i) * a.slot + s2 : p + (int64_t)i * a.slot + ci);
     if (flag_c & CELL_SOLID) return;
     const bool inner = a.nx >= 2 && !(flag_in & CELL_SOLID);
     R mine = here;
-    if (fix && through_face) {
+    if (fixed) {
         const R cs = R(0.57735026918962576451);
         mine = cs * (inner ? was_in : was_own) + (R(1) - cs) * was_own;
         S stored;
@@ -455,7 +466,9 @@ __device__ __forceinline__ void outflow_link(const StepArgs &a, uint32_t yz, int
         mine = T::ld(&stored);                             // the stored (rounded) value
     }
     *own = mine;                                            // every cx = -1 link of an outlet cell reads its own slot
-    if (inner) *in = next_odd && through_face && !(flag_s & CELL_SOLID) ? across : there;
+    if (!inner) return;
+    if (crosses && (flag_s & CELL_SOLID)) next = T::ld(p + (int64_t)i * a.slot + ci);       // an obstacle's link: the cell's own
+    *in = next;
 }
 
 // One thread per outlet column and direction (blocks along y of the grid; the
@@ -612,7 +625,7 @@ __global__ void __launch_bounds__(256, (bulk_min_blocks<S, ODD, EPI, PLAIN>())) 
 // Batched edge kernel: blocks [0, eblocks) are the members' edge blocks,
 // the blocks after them the members' wall-row blocks (numbered by w_begin).
 template <class S, bool ODD, bool PLAIN>
-__global__ void __launch_bounds__(EDGE_BLOCK) k_batch_edge(const BatchMember *mem, const int64_t *begin, int nm,
+__global__ void __launch_bounds__(EDGE_BLOCK, edge_blocks_per_sm<S, ODD>()) k_batch_edge(const BatchMember *mem, const int64_t *begin, int nm,
                                                            const int64_t *tdev, int epi, int64_t eblocks,
                                                            const int64_t *w_begin)
 {
