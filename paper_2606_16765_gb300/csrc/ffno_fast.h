@@ -67,7 +67,7 @@ struct Mlp {
 };
 bool mlp_fits(int ci, int ch, int co);
 void mlp(const Mlp &p, const float *x, const float *res, float *y, int B, int64_t N, cudaStream_t s);
-// gx = dL/dx (may be null) and the gradients of (W1, b1, W2, b2), contiguous at
+// gx = dL/dx (may be null with ACT_GELU) and the gradients of (W1, b1, W2, b2), contiguous at
 // gw, from g = dL/dy; part: mlp_parts() x (sizes of the four) floats
 int mlp_parts();
 void mlp_bwd(const Mlp &p, const float *x, const float *g, float *gx, float *part, float *gw, int B, int64_t N,
