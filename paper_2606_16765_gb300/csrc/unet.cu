@@ -1340,6 +1340,27 @@ extern "C" lbm_status unet_conv3_backward_data(const float *gy, const float *w, 
     return st == LBM_OK ? op_finish(s, status) : st;
 }
 
+// What conv_plan chooses for a call of these sizes (for the tests): route[0] 0
+// shifted copies, 1 halo block, 2 split sums; [1] parts; [2] channel tile; [3]
+// taps per stage and [4] accumulator sets of the halo kernel.  `act` is any
+// device buffer on a 16-byte boundary; nothing is read.
+extern "C" lbm_status unet_conv3_route(const void *act, int32_t B, int32_t nx, int32_t ny, int32_t nz, int32_t cin,
+                                       int32_t cout, int32_t route[5])
+{
+    unet::ConvPlan p;
+    const char *e = nullptr;
+    if (!act || !route || !unet::conv_plan(p, act, cin, cin, nx, ny, nz, B, act, cout, 27, cout, 0, gb300::sm_count(), &e, true)) {
+        g_unet_err = e ? e : "null argument";
+        return LBM_ERR_ARG;
+    }
+    route[0] = p.a.ksplit > 1 ? 2 : p.halo ? 1 : 0;
+    route[1] = p.a.ksplit;
+    route[2] = p.a.ntile;
+    route[3] = p.halo ? p.h.tps : 0;
+    route[4] = p.halo ? p.h.sets : 0;
+    return LBM_OK;
+}
+
 extern "C" lbm_status unet_conv3_backward_weights(const float *x, const float *gy, float *gw, int32_t B, int32_t nx,
                                                   int32_t ny, int32_t nz, int32_t cin, int32_t cout, void *stream)
 {
