@@ -2779,7 +2779,8 @@ void pw_fwd(fno_ctx *f, const T *x, int ci, int co, int64_t oW, int64_t ob, cons
         // cores pay off.  32 -> 32 stays on the paired SIMT kernel: there the
         // per-element stores of the fragment layout (2 bytes into 4 channel
         // planes per warp instruction) cost more than the multiply-adds saved
-        // (0.50 against 0.39 ms per layer at batch 8).
+        // (0.50 against 0.39 ms per layer at batch 8, before store_quads; not
+        // measured with it).
         if (std::is_same<T, __nv_bfloat16>::value && ci == PTC_CI && co == 128 && f->N % 16 == 0) {
             const int64_t warps = (int64_t)B * f->N / 16;
             const int blocks = (int)std::min<int64_t>((warps + TPB / 32 - 1) / (TPB / 32), gb300::sm_count() * 8);
@@ -2905,7 +2906,7 @@ void dft_fwd(fno_ctx *f, const T *x, float2 *S, const float *scale, int B, int l
         umma_dftx_fwd(f->vmaps[layer_map].data(), f->twx, f->stA, R, f->ustatus, blocks, f->s);
     } else if (tc_input && d.nx == TCX_NX && d.Kx == TCX_KX && (reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
         // one m-tile per pass while that leaves a warp slot of one block per SM for each
-        // (2,048 rows 7.8 and 5.5 us, 8,192 rows 8.1 and 5.7, 32,768 rows 9.0 and 9.3)
+        // (two and one: 2,048 rows 7.8 and 5.5 us, 8,192 rows 8.1 and 5.7, 32,768 rows 9.0 and 9.3)
         const bool one = (R + 15) / 16 <= (int64_t)gb300::sm_count() * (TPB / 32);
         const int64_t warps = one ? (R + 15) / 16 : (R + 31) / 32;
         auto k = one ? k_dftx_fwd_tc<T, 1> : k_dftx_fwd_tc<T, 2>;

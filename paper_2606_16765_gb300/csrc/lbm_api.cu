@@ -455,10 +455,13 @@ static void side_destroy(SideStream &d)
 // The side stream, created on first use; null (the kernels then follow one
 // another) where that fails, where `s` is being captured before it exists, and
 // on large grids: there the bulk kernel fills the chip for long and the edge
-// blocks' registers cost it more than they hide.  Per step, one after the
-// other and side by side: 64x32x32 26.0 and 21.4 us, 256x128x128 197 and 191
-// us (FP32), eight channels of 12 M cells 650 and 645 us (F16C), 512x256x256
-// (33.5 M cells) 1.040 and 1.054 ms (FP16).
+// blocks' registers cost it more than they hide.  The limit is where that begins
+// for binary16 and bfloat16; FP32 and F16C would still gain a little above it.
+// Per step, one after the other and side by side: 64x32x32 26.0 and 21.4 us,
+// 256x128x128 197 and 191 us (FP32), eight channels of 12 M cells 650 and 645 us
+// (F16C); 12.6 M cells the same for every storage; 18.9 M FP32 701 and 693,
+// F16C 665 and 659, FP16S 551 and 558, BF16S 554 and 562 us; 33.6 M FP32 1209 and
+// 1203, F16C 1094 and 1089, FP16S 913 and 920, BF16S 919 and 927 us.
 constexpr int64_t SIDE_CELLS = (int64_t)1 << 24;
 
 static const SideStream *side_of(SideStream &d, cudaStream_t s, int64_t cells)

@@ -145,7 +145,9 @@ __device__ __forceinline__ void bulk_cell(const StepArgs &a, const StepOut &o, i
 // take 40 registers (six blocks) without the epilogue; FP32 runs its odd
 // step at 40 and its even step at 48 (five blocks), the bandwidth each
 // measured best at; the general collision 64 (four), FP64 the plain
-// collision 80 (three).  Each at no or one spilled value.
+// collision 80 (three).  A single lattice's kernels spill two values at most;
+// the batched ones, whose arguments sit in shared memory, 108 bytes in the odd
+// plain step at 40 registers and up to 76 in its epilogue variants.
 template <class S, bool ODD, bool EPI, bool PLAIN>
 constexpr int bulk_min_blocks()
 {
